@@ -329,6 +329,20 @@ ap_dvm_status flush(ap_dvm_handle* h) {
   h->up_rows.assign(1, 0);
   h->up_rhs.assign(1, 0);
   h->up_cols.assign(1, 0);
+  // Transform work per item: an equal share of all transforms for each resident block, at most what
+  // the blocks' shared memory holds (eblk, eblk_cols).  Large batches reach that cap (2048^2: one
+  // row pair, 4 FP32 or 2 FP64 columns of 32-byte row segments); on small grids full items would
+  // leave most SMs idle (at 64^2 one block took every column).  FP64 column pass, full items against
+  // shares, per launch: 64^2 65 -> 24 us, 256^2 98 -> 28 us, 512^2 117 -> 37 us; row passes at 256^2
+  // 29 -> 16 us; from 1000^2 on the two rules give the same items (CUDA events, launch gap included).
+  long long row_elems = 0, col_elems = 0;
+  for (const Slot& s : h->slots) {
+    if (!s.attached || s.paused) continue;
+    row_elems += (long long)((s.p.ny + 1) / 2) << s.dev.lnx;
+    col_elems += (long long)(s.p.nx / 2 + 1) << s.dev.lny;
+  }
+  const int row_share = (int)(row_elems / std::min(h->grid_rows, h->grid_fft));
+  const int col_share = (int)(col_elems / std::min(h->grid_cols, h->grid_fft));
   for (Slot& s : h->slots) {
     if (!s.attached || s.paused) continue;
     if (s.p.nx < TX || s.p.ny < TY) return fail(h, AP_DVM_ERR_ARG, "grid %dx%d smaller than the tile %dx%d", s.p.nx, s.p.ny, TX, TY);
@@ -336,17 +350,16 @@ ap_dvm_status flush(ap_dvm_handle* h) {
     d.tiles_x = (s.p.nx + TX - 1) / TX;   // ragged tiles at the high edges
     d.tiles_y = (s.p.ny + TY - 1) / TY;
     const int pairs = (s.p.ny + 1) / 2;   // row pairs (the last one single when ny is odd)
-    d.row_pairs = std::max(1, std::min(h->eblk >> d.lnx, pairs));
-    // power-of-two columns: as many adjacent columns per item as the item's buffer holds
-    // (4 FP32 or 2 FP64 of 2048 cells: 32-byte row segments; more on shorter columns), up to
-    // the power of two that covers the nx/2 + 1 spectral columns
+    d.row_pairs = std::max(1, std::min(std::min(h->eblk, row_share) >> d.lnx, pairs));
+    // power-of-two columns: as many adjacent columns per item as the share holds, up to the
+    // power of two that covers the nx/2 + 1 spectral columns
     if (is_pow2(s.p.ny)) {
       const int cap = std::max(1, h->eblk_cols >> d.lny), nh = s.p.nx / 2 + 1;
       int g = 1;
-      while (g < cap && g < nh) g <<= 1;
+      while (g < cap && g < nh && (g << d.lny) < col_share) g <<= 1;
       d.col_group = g;
     } else {
-      d.col_group = std::max(1, h->eblk >> d.lny);
+      d.col_group = std::max(1, std::min(h->eblk, col_share) >> d.lny);
     }
     for (int par = 0; par < 2; ++par) {   // the instance as steps of either parity see it
       InstDev v = view(s, par);
