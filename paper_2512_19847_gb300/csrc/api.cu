@@ -93,13 +93,15 @@ struct ap_dvm_handle {
   // upload staging (kept alive across async copies)
   std::vector<InstDev> up_inst[2];
   std::vector<int> up_tiles, up_rows, up_cols, up_rhs;
-  int up_counts[5] = {0, 0, 0, 0, 0};
+  int up_counts[6] = {0, 0, 0, 0, 0, 0};
   // kernels
   StencilSet ks{};
   MiscSet km{};
   int grid_explicit = 0, grid_rhs = 0, grid_update = 0, grid_fft = 0, grid_cols = 0, grid_finish = 0, grid_rows = 0;
+  int grid_explicit_split = 0, grid_update_split = 0;
   unsigned fft_kinds = 0;   // FftKinds of the attached solves (the launches a step enqueues)
-  size_t smem_update = 0;
+  unsigned stencil_kinds = 0;   // ... and their StencilKinds
+  size_t smem_update = 0, smem_update_split = 0;
   bool kernels_ready = false;
   // graph
   int graph_steps = 0;
@@ -228,7 +230,7 @@ size_t batch_bytes(int capacity, int nmax) {
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
-  take(sizeof(int) * 5);
+  take(sizeof(int) * 6);
   take(sizeof(double2) * (nmax / 2));
   take(sizeof(float2) * (nmax / 2));
   take(sizeof(unsigned) * 4);
@@ -246,6 +248,14 @@ unsigned fft_kinds_of(const ap_dvm_handle* h) {
     if (s.attached) add(s.p);
   if (!k) add(h->tmpl);
   return k;
+}
+
+// StencilKinds of the attached solves (of the template while none is attached).
+unsigned stencil_kinds_of(const ap_dvm_handle* h) {
+  unsigned k = 0;
+  for (const Slot& s : h->slots)
+    if (s.attached) k |= split_fluxes(s.p) ? STENCIL_SPLIT : STENCIL_WHOLE;
+  return k ? k : (split_fluxes(h->tmpl) ? STENCIL_SPLIT : STENCIL_WHOLE);
 }
 
 int auto_tile(const ap_dvm_handle* h) {
@@ -292,6 +302,11 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
   if ((st = occupancy_grid(h, h->ks.k_rhs, h->ks.rhs_threads, 0, &h->grid_rhs))) return st;
   h->smem_update = update_smem(h->ks, h->tmpl);
   if ((st = occupancy_grid(h, h->ks.k_update, thr, h->smem_update, &h->grid_update))) return st;
+  if (h->ks.k_explicit_split) {
+    h->smem_update_split = update_smem_split(h->ks, h->tmpl);
+    if ((st = occupancy_grid(h, h->ks.k_explicit_split, thr, h->ks.smem_explicit_split, &h->grid_explicit_split))) return st;
+    if ((st = occupancy_grid(h, h->ks.k_update_split, thr, h->smem_update_split, &h->grid_update_split))) return st;
+  }
   if ((st = occupancy_grid(h, h->km.k_finish, thr, 0, &h->grid_finish))) return st;
   h->grid_fft = 1 << 30;
   for (const void* fn : {h->km.k_rows_fwd_bs, h->km.k_cols_bs, h->km.k_rows_inv_bs}) {
@@ -322,7 +337,12 @@ ap_dvm_status flush(ap_dvm_handle* h) {
     return fail(h, AP_DVM_ERR_ARG, "the set of solves changed while the stream is being captured");
   const int TX = h->ks.tx, TY = h->ks.ty;
   const unsigned kinds = fft_kinds_of(h);
-  if (kinds != h->fft_kinds) { h->fft_kinds = kinds; h->graph_valid[0] = h->graph_valid[1] = false; }   // the launch sequence changed
+  const unsigned skinds = stencil_kinds_of(h);
+  if (kinds != h->fft_kinds || skinds != h->stencil_kinds) {   // the launch sequence changed
+    h->fft_kinds = kinds;
+    h->stencil_kinds = skinds;
+    h->graph_valid[0] = h->graph_valid[1] = false;
+  }
   h->up_inst[0].clear();
   h->up_inst[1].clear();
   h->up_tiles.assign(1, 0);
@@ -343,8 +363,14 @@ ap_dvm_status flush(ap_dvm_handle* h) {
   }
   const int row_share = (int)(row_elems / std::min(h->grid_rows, h->grid_fft));
   const int col_share = (int)(col_elems / std::min(h->grid_cols, h->grid_fft));
-  for (Slot& s : h->slots) {
-    if (!s.attached || s.paused) continue;
+  // the instances with split fluxes come last: a tile range for each kind of stencil kernel
+  std::vector<Slot*> order;
+  for (int split = 0; split < 2; ++split)
+    for (Slot& s : h->slots)
+      if (s.attached && !s.paused && split_fluxes(s.p) == (split != 0)) order.push_back(&s);
+  h->up_counts[5] = 0;
+  for (Slot* sp : order) {
+    Slot& s = *sp;
     if (s.p.nx < TX || s.p.ny < TY) return fail(h, AP_DVM_ERR_ARG, "grid %dx%d smaller than the tile %dx%d", s.p.nx, s.p.ny, TX, TY);
     InstDev& d = s.dev;
     d.tiles_x = (s.p.nx + TX - 1) / TX;   // ragged tiles at the high edges
@@ -371,6 +397,7 @@ ap_dvm_status flush(ap_dvm_handle* h) {
       h->up_inst[par].push_back(v);
     }
     h->up_tiles.push_back(h->up_tiles.back() + d.tiles_x * d.tiles_y);
+    if (!split_fluxes(s.p)) h->up_counts[5] = h->up_tiles.back();
     h->up_rows.push_back(h->up_rows.back() + (pairs + d.row_pairs - 1) / d.row_pairs);
     h->up_rhs.push_back(h->up_rhs.back() + rhs_items(s.p.nx, s.p.ny, h->f32));
     h->up_cols.push_back(h->up_cols.back() + (s.p.nx / 2 + 1 + d.col_group - 1) / d.col_group);
@@ -391,7 +418,7 @@ ap_dvm_status flush(ap_dvm_handle* h) {
     CUDA_TRY(h, cudaMemcpyAsync(h->d_rhs_start, h->up_rhs.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(h->d_col_start, h->up_cols.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
   }
-  CUDA_TRY(h, cudaMemcpyAsync(h->d_counts, h->up_counts, sizeof(int) * 5, cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(h->d_counts, h->up_counts, sizeof(int) * 6, cudaMemcpyHostToDevice, h->stream));
   h->dirty = false;
   return AP_DVM_OK;
 }
@@ -441,7 +468,7 @@ ap_dvm_status profile_collect(ap_dvm_handle* h) {
 ap_dvm_status enqueue_step(ap_dvm_handle* h, cudaStream_t stream, int parity) {
   StepKernels K{h->ks,       h->km,         h->grid_explicit, h->grid_rhs,   h->grid_update, h->grid_finish,
                 h->grid_fft, h->grid_cols, h->km.cols_threads, fft_smem(h), cols_smem(h), h->smem_update, h->fft_kinds,
-                h->grid_rows};
+                h->grid_rows, h->stencil_kinds, h->grid_explicit_split, h->grid_update_split, h->smem_update_split};
   auto ln = [&](const void* fn, int grid, dim3 block, size_t smem, void** args, int kind) -> int {
     return (int)launch(h, stream, fn, grid, block, smem, args, kind);
   };
@@ -558,7 +585,7 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   h->d_row_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   h->d_col_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   h->d_rhs_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
-  h->d_counts = reinterpret_cast<int*>(take(sizeof(int) * 5));
+  h->d_counts = reinterpret_cast<int*>(take(sizeof(int) * 6));
   h->d_tw = reinterpret_cast<double2*>(take(sizeof(double2) * (h->nmax / 2)));
   h->d_tw32 = reinterpret_cast<float2*>(take(sizeof(float2) * (h->nmax / 2)));
   h->d_err = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 4));
@@ -595,7 +622,7 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   for (int par = 0; par < 2; ++par)
     CUDA_TRY(h, cudaMemcpyAsync(h->d_batch[par], &h->hb[par], sizeof(BatchDev), cudaMemcpyHostToDevice, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned) * 4, h->stream));
-  CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, sizeof(int) * 5, h->stream));
+  CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, sizeof(int) * 6, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->slots.resize(capacity);
   h->dirty = true;
@@ -904,8 +931,10 @@ int ap_dvm_launches_per_step(const ap_dvm_handle* h) {
   if (!h) return 0;
   const ap_dvm_params& t = h->tmpl;
   const int f = fft_launches(fft_kinds_of(h));   // transform launches per implicit stage
+  const unsigned sk = stencil_kinds_of(h);
+  const int n = ((sk & STENCIL_WHOLE) ? 1 : 0) + ((sk & STENCIL_SPLIT) ? 1 : 0);   // explicit, and update, launches per stage
   // the last stage's update closes the step (no finish kernel)
-  return t.A_im[0] != 0.0 ? 1 + (2 + f) + (3 + f) * (t.s - 1) : (3 + f) * (t.s - 1);
+  return t.A_im[0] != 0.0 ? 1 + (1 + n + f) + (1 + 2 * n + f) * (t.s - 1) : (1 + 2 * n + f) * (t.s - 1);
 }
 
 ap_dvm_status ap_dvm_run_host(ap_dvm_handle* h, int slot, const double* h_in, double* h_out, double* d_stage, int nsteps) {

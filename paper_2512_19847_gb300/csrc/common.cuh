@@ -30,6 +30,8 @@ template <typename T>
 struct Coef {
   T dt, te2, qtau, htau;                  // dt, tau eps^2, tau/4, tau/2
   T inv_dx, inv_dy;
+  // with the fourth-order difference's 1/12: 1/(12 h), times tau/4, times tau eps^2; 1/(12 h^2)
+  T cdx, cdy, qcx, qcy, tcx, tcy, ldx, ldy;
   T kappa[APD_MAXS + 1];                  // 2 eps^2 / (dt a_ii)^2
   T aex[APD_MAXS + 1][APD_MAXS + 1];      // atilde_ij
   T aim[APD_MAXS + 1][APD_MAXS + 1];      // a_ij
@@ -115,7 +117,8 @@ struct BatchDev {
   int* row_start;        // [n+1]
   int* col_start;        // [n+1]
   int* rhs_start;        // [n+1]
-  int* counts;           // [0] tiles, [1] row items, [2] column items, [3] instances, [4] k_rhs items
+  int* counts;           // [0] tiles, [1] row items, [2] column items, [3] instances, [4] k_rhs items,
+                         // [5] tiles of the instances whose fluxes are not split (they come first)
   double2* tw;           // twiddles exp(-2 pi i k / nmax), k < nmax/2
   float2* tw32;          // the same, rounded once to FP32 (FP32 form)
   int lnmax;             // log2 of the largest transform length

@@ -14,6 +14,10 @@ struct StencilSet {
   const void* k_explicit;
   const void* k_rhs;
   const void* k_update;
+  const void* k_explicit_split;        // FP64 WENO: the same with split fluxes (null otherwise)
+  const void* k_update_split;
+  size_t smem_explicit_split, update_fixed_split;
+  int nbuf_split;
   size_t smem_explicit;
   int rhs_threads;                     // k_rhs: threads per block (no dynamic shared memory)
   size_t plane_bytes, update_fixed;   // k_update: update_fixed + nbuf * (planes staged) * plane_bytes

@@ -1,0 +1,162 @@
+// FP64 WENO fluxes with their nonlinear part on the FP32 pipe.
+//
+// This GPU issues FP64 instructions at 1/64 of the FP32 rate, and a WENO5 flux
+// in FP64 takes about 55 of them per interface.  Here the flux is taken apart
+// into a part that is linear in the data, which stays in FP64, and the weights'
+// correction, which is a sum of products (nonlinear weight) x (third difference)
+// and is evaluated in pairs of floats (h + l, 48 bits and more).  The differences
+// it starts from are taken in FP64, so that the pair's relative rounding (2^-48)
+// applies to increments between neighbouring cells and not to the values.
+//
+// WENO5.  With g+- = g +- U (twice the Lax-Friedrichs split), interface i + 1/2,
+// D_k = f_{k+1} - f_k, third differences T_k = f_{k+2} - 3 f_{k+1} + 3 f_k - f_{k-1},
+// and the reconstruction about its centred candidate,
+//   6 (L(g+) + R(g-)) = [-g_{i-1} + 7 g_i + 7 g_{i+1} - g_{i+2}] + T_i(U) + N_{i+1/2},
+//   N = -(2 w0 T_{i-1} + w2 T_i)(g+) + (2 w0 T_{i+1} + w2 T_i)(g-),
+// so that the flux difference of cell i is 1/(12 h) times
+//   8 (g_{i+1} - g_{i-1}) - (g_{i+2} - g_{i-2}) + (fourth difference of U) + N_{i+1/2} - N_{i-1/2}.
+// The smoothness indicators (times 4, plus 4 eps_W) are sums of squares of
+// increments: (13/3) (D_k - D_{k-1})^2 + l^2 + 4 eps_W with l = 3 D_k - D_{k-1},
+// D_{k-1} + D_k or D_k - 3 D_{k-1} for the three candidates.
+//
+// WENO3.  The same with w0 = 1/3 + (w0 - 1/3) for the weight of the outer candidate: the 1/3 gives
+// the linear part above, and
+//   N = -3 ((w0 - 1/3)(g+) c_i(g+) + (w0 - 1/3)(g-) c_{i+1}(g-))
+// with second differences c_k (taken whole, w0 c would be less exact than FP64 at 256 cells a side).
+#pragma once
+#include "common.cuh"
+
+namespace apd {
+
+// h + l, |l| small against the operands it came from (not always against h).
+struct F2 { float h, l; };
+
+__device__ __forceinline__ F2 f2(float h, float l) { F2 r; r.h = h; r.l = l; return r; }
+
+// a + k b for k = 1, -1, 2, -2: the error of the leading sum kept exactly (Knuth's two-sum).
+template <int K>
+__device__ __forceinline__ F2 f2_addk(F2 a, F2 b) {
+  const float k = float(K);
+  const float s = __fmaf_rn(k, b.h, a.h), bb = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fmaf_rn(k, b.h, -bb));
+  return f2(s, __fadd_rn(e, __fmaf_rn(k, b.l, a.l)));
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) { return f2_addk<1>(a, b); }
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) { return f2_addk<-1>(a, b); }
+// The same value with |l| <= ulp(h)/2.
+__device__ __forceinline__ F2 f2_norm(F2 a) {
+  const float h = __fadd_rn(a.h, a.l);
+  return f2(h, __fsub_rn(a.l, __fsub_rn(h, a.h)));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return f2(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ F2 f2_sqr(F2 a) {
+  const float p = __fmul_rn(a.h, a.h);
+  const float t = __fmul_rn(a.h, a.l);
+  return f2(p, __fadd_rn(t, __fadd_rn(t, __fmaf_rn(a.h, a.h, -p))));
+}
+// k a for an integer k that is a float.
+__device__ __forceinline__ F2 f2_scale(F2 a, float k) {
+  const float p = __fmul_rn(k, a.h);
+  return f2(p, __fmaf_rn(k, a.l, __fmaf_rn(k, a.h, -p)));
+}
+// n / d: one approximate quotient and the remainder's, with the same reciprocal.
+__device__ __forceinline__ F2 f2_div(F2 n, F2 d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d.h));
+  const float q = __fmul_rn(n.h, r);
+  const float rem = __fadd_rn(__fmaf_rn(-q, d.h, n.h), __fmaf_rn(-q, d.l, n.l));
+  return f2(q, __fmul_rn(rem, r));
+}
+// 2^-(exponent of x) for 0 < x finite (0, infinity and NaN give something harmless or not finite).
+__device__ __forceinline__ float inv_pow2(float x) {
+  return __uint_as_float(0x7f000000u - (__float_as_uint(x) & 0x7f800000u));
+}
+
+// An FP64 increment as a pair, by integer operations (a conversion instruction takes a
+// slot of the FP64 pipe): h the leading 24 bits truncated, l the other 29 rounded to 24.
+__device__ __forceinline__ F2 f2_from_double(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned ea = (hi >> 20) & 0x7ffu;
+  if (ea - 949u <= 1150u - 949u) {   // 2^-74 <= |d| < 2^128
+    const unsigned s = hi & 0x80000000u;
+    const float h = __uint_as_float((__funnelshift_l(lo, hi, 3) - (384u << 23)) | s);   // 896 mod 512
+    const float m = __uint2float_rn(lo & 0x1fffffffu);
+    return f2(h, __fmul_rn(m, __uint_as_float(((ea - 948u) << 23) | s)));
+  }
+  if ((hi << 1 | lo) == 0u) return f2(0.f, 0.f);
+  const float h = __double2float_rn(d);
+  return f2(h, __double2float_rn(d - (double)h));
+}
+
+// h + l in FP64 (one FP64 operation; the widenings on the integer pipe).
+__device__ __forceinline__ double f2_widen1(float x) {
+  const unsigned u = __float_as_uint(x);
+  if (((u >> 23) & 0xffu) - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+  if ((u << 1) == 0u) return 0.0;
+  return (double)x;
+}
+__device__ __forceinline__ double f2_to_double(F2 a) { return f2_widen1(a.h) + f2_widen1(a.l); }
+
+// Nonlinear part of one WENO5 reconstruction for each of KR neighbouring interfaces:
+// q[m] = 2 w0 T_{out} + w2 T_{in} from the increments D[m .. m + 3] of its stencil (upwind
+// to downwind; T_out = D[m+2] - 2 D[m+1] + D[m], T_in one further), w = 16 eps_W (the
+// indicators times 4, the doubled split).  With the e_k scaled by a power of two so that the
+// largest is about 1, and then their products likewise, every step stays in the float range
+// whatever the data and eps_W: what underflows is below 2^-60 of the sum it belongs to.
+template <int KR>
+__device__ __forceinline__ void w5_split(const F2* D, F2 w, F2* q) {
+  F2 c[KR + 3], C[KR + 3];
+#pragma unroll
+  for (int k = 1; k < KR + 3; ++k) {
+    c[k] = f2_sub(D[k], D[k - 1]);
+    const F2 s = f2_sqr(c[k]);
+    const float kh = 4.3333335f, kl = -1.5894572e-07f;   // 13/3
+    const float p = __fmul_rn(kh, s.h);
+    const float pl = __fmaf_rn(kl, s.h, __fmaf_rn(kh, s.l, __fmaf_rn(kh, s.h, -p)));
+    C[k] = f2_add(w, f2(p, pl));
+  }
+#pragma unroll
+  for (int m = 0; m < KR; ++m) {
+    F2 e0 = f2_add(C[m + 1], f2_sqr(f2_addk<2>(c[m + 1], D[m + 1])));
+    F2 e1 = f2_add(C[m + 2], f2_sqr(f2_add(D[m + 1], D[m + 2])));
+    F2 e2 = f2_add(C[m + 3], f2_sqr(f2_addk<-2>(c[m + 3], D[m + 2])));
+    const float se = inv_pow2(fmaxf(fmaxf(e0.h, e1.h), e2.h));
+    e0 = f2(e0.h * se, e0.l * se);
+    e1 = f2(e1.h * se, e1.l * se);
+    e2 = f2(e2.h * se, e2.l * se);
+    F2 pa = f2_mul(e1, e2), pb = f2_mul(e0, e2), pc = f2_mul(e0, e1);
+    const float sp = inv_pow2(fmaxf(fmaxf(pa.h, pb.h), pc.h));
+    pa = f2(pa.h * sp, pa.l * sp);
+    pb = f2(pb.h * sp, pb.l * sp);
+    pc = f2(pc.h * sp, pc.l * sp);
+    const F2 A = f2_sqr(pa), B = f2_scale(f2_sqr(pb), 6.f), E = f2_scale(f2_sqr(pc), 3.f);
+    const F2 den = f2_add(f2_add(A, E), B);
+    const F2 to = f2_sub(c[m + 2], c[m + 1]), ti = f2_sub(c[m + 3], c[m + 2]);
+    q[m] = f2_div(f2_addk<2>(f2_mul(E, ti), f2_mul(A, to)), den);
+  }
+}
+
+// The same for WENO3: q[m] = 3 (w0 - 1/3) c with c = D[m+1] - D[m] (upwind, then downwind increment),
+// w = 4 eps_W, indicators e_k = D_k^2 + w: w0 = e1^2 / (e1^2 + 2 e0^2) and
+// 3 (w0 - 1/3) = 2 (e1 - e0)(e1 + e0) / (e1^2 + 2 e0^2), e1 - e0 = c (D[m] + D[m+1]).
+template <int KR>
+__device__ __forceinline__ void w3_split(const F2* D, F2 w, F2* q) {
+  F2 e[KR + 1];
+#pragma unroll
+  for (int k = 0; k < KR + 1; ++k) e[k] = f2_add(w, f2_sqr(D[k]));
+#pragma unroll
+  for (int m = 0; m < KR; ++m) {
+    const float se = inv_pow2(fmaxf(e[m].h, e[m + 1].h));
+    const F2 e0 = f2(e[m].h * se, e[m].l * se), e1 = f2(e[m + 1].h * se, e[m + 1].l * se);
+    const F2 c = f2_sub(D[m + 1], D[m]), d = f2_add(D[m + 1], D[m]);
+    const F2 n = f2_mul(f2_mul(f2_mul(c, f2(d.h * se, d.l * se)), f2_add(e0, e1)), c);
+    const F2 r = f2_div(n, f2_addk<2>(f2_sqr(e1), f2_sqr(e0)));
+    q[m] = f2(2.f * r.h, 2.f * r.l);
+  }
+}
+
+}  // namespace apd

@@ -1,0 +1,332 @@
+// The FP64 explicit and update kernels of the WENO schemes with the split fluxes of
+// split_flux.cuh: three passes over a staged tile,
+//   1. FP64 increments along both axes, kept as pairs of floats (one FP64 operation each),
+//   2. the nonlinear interface terms N, on the FP32 pipe, in runs of neighbouring interfaces,
+//   3. per cell: the linear parts and the closed forms in FP64, with the differences of N.
+// What bounds them is still the FP64 pipe (2 operations per clock and SM), now with about 130
+// (explicit, all terms) and 75 (update) FP64 operations per cell instead of 510 and 370, beside
+// about 450 FP32 instructions per interface.  WENO5 at 2048^2, ms per step (32x8 tiles): explicit
+// 6.17 -> 2.16, update 6.06 -> 2.18; WENO3 at 256^2, 10 steps: 0.98 -> 0.55 and 1.00 -> 0.53.
+// Measured choices (2048^2, explicit + update, ms): WENO5 768 threads per SM (85 registers)
+// 2.16 + 2.18, 512 (128 registers) 2.30 + 2.31; one staged plane buffer 2.30 + 2.31 against 2.31 +
+// 2.35 with two (at 512 threads; the second block on the SM hides the copies); runs of 3
+// interfaces 2.30 + 2.31, of 4 2.37 + 2.55.  WENO3 keeps 512 threads: 2.03 + 1.99 against 1.98 +
+// 1.86 at 2048^2 but 0.056 + 0.053 against 0.070 + 0.066 at 256^2, the size it is run at.
+#pragma once
+#include "split_flux.cuh"
+#include "stencil_kernels.cuh"
+
+namespace apd {
+
+#ifndef APD_SPLIT_RUN
+#define APD_SPLIT_RUN 3   // interfaces per run of pass 2
+#endif
+#ifndef APD_SPLIT_THREADS5
+#define APD_SPLIT_THREADS5 768   // threads per SM the split kernels are compiled for, WENO5
+#endif
+#ifndef APD_SPLIT_THREADS3
+#define APD_SPLIT_THREADS3 512   // ... and WENO3
+#endif
+#ifndef APD_SPLIT_NBUF
+#define APD_SPLIT_NBUF 1   // staged plane buffers
+#endif
+
+template <int SCHEME, int TX, int TY>
+struct SplitGeo {
+  using G = Geo<double, SCHEME, TX, TY>;
+  static constexpr int NS = SCHEME == WENO5_C4 ? 4 : 2;                    // increments of one reconstruction
+  static constexpr int LX = G::W - 1, LY = G::HH - 1;                      // increments per line
+  static constexpr int LIX = TY * LX, LIY = LY * TX;                       // per field
+  static constexpr int NBUF = APD_SPLIT_NBUF;
+  // elements of 8 bytes besides the staged planes: increments of F fields per axis, N of P pairs per axis
+  static constexpr int extra(int F, int P) { return F * (LIX + LIY) + P * (G::NX + G::NY); }
+  static constexpr size_t explicit_bytes = 128 + 8 * (size_t)(NBUF * 6 * G::PL + extra(5, 3));
+  static constexpr size_t update_fixed_bytes = 128 + 8 * (size_t)(2 * G::PL + extra(4, 2));
+};
+
+template <int SCHEME, int THREADS>
+__host__ __device__ constexpr int split_min_blocks() {
+  const int n = (SCHEME == WENO5_C4 ? APD_SPLIT_THREADS5 : APD_SPLIT_THREADS3) / THREADS;
+  return n > 0 ? n : 1;
+}
+
+// Pass 1: increments of NF staged planes along x (fx) and NF along y (fy).
+template <int SCHEME, int TX, int TY, int NF>
+__device__ __forceinline__ void split_increments(const double* const* fx, const double* const* fy, F2* ix, F2* iy, int tid) {
+  using S = SplitGeo<SCHEME, TX, TY>;
+  using G = typename S::G;
+  for (int k = tid; k < S::LIX + S::LIY; k += TX * TY) {
+    if (k < S::LIX) {
+      const int line = k / S::LX, o = (G::H + line) * G::BW + G::XO + (k - line * S::LX);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) ix[f * S::LIX + k] = f2_from_double(fx[f][o + 1] - fx[f][o]);
+    } else {
+      const int r = k - S::LIX, pt = r / TX, o = pt * G::BW + G::XO + G::H + (r - pt * TX);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) iy[f * S::LIY + r] = f2_from_double(fy[f][o + G::BW] - fy[f][o]);
+    }
+  }
+}
+
+// Pass 2, one run: the increments of g and U at ig, iu (stride st between points, npt in the line),
+// sg = -1 negates g; N of interfaces m0 .. m0 + KR - 1 into out (stride so), those below ni only.
+template <int SCHEME, int KR>
+__device__ __forceinline__ void split_run(const F2* ig, const F2* iu, float sg, int st, int npt, F2 w, F2* out, int so,
+                                          int m0, int ni) {
+  constexpr int NS = SCHEME == WENO5_C4 ? 4 : 2, ND = KR + NS;
+  F2 D[ND], q[KR], qm[KR];
+#pragma unroll
+  for (int j = 0; j < ND - 1; ++j) {
+    const int o = min(m0 + j, npt - 1) * st;
+    const F2 a = ig[o];
+    D[j] = f2_norm(f2_add(f2(sg * a.h, sg * a.l), iu[o]));
+  }
+  if constexpr (SCHEME == WENO5_C4) w5_split<KR>(D, w, q);
+  else w3_split<KR>(D, w, q);
+  // g- from the right: the same with the increments in reverse
+#pragma unroll
+  for (int j = 1; j < ND; ++j) {
+    const int o = min(m0 + j, npt - 1) * st;
+    const F2 a = ig[o];
+    D[ND - 1 - j] = f2_norm(f2_sub(f2(sg * a.h, sg * a.l), iu[o]));
+  }
+  if constexpr (SCHEME == WENO5_C4) w5_split<KR>(D, w, qm);
+  else w3_split<KR>(D, w, qm);
+#pragma unroll
+  for (int i = 0; i < KR; ++i)
+    if (m0 + i < ni) out[(m0 + i) * so] = f2_norm(f2_sub(qm[KR - 1 - i], q[i]));
+}
+
+// Pass 2: NP pairs per axis.  Pair p takes the fields gi(p) and ui(p) of the increments
+// (NP = 3: g 0 1 2, U 1 3 4; NP = 2: g 0 1, U 2 3; NP = 1: g 0, U 1); the x pair NEGX is negated.
+template <int SCHEME, int TX, int TY, int NP, int NEGX>
+__device__ __forceinline__ void split_interfaces(const F2* ix, const F2* iy, F2* nx, F2* ny, F2 w, int tid) {
+  using S = SplitGeo<SCHEME, TX, TY>;
+  using G = typename S::G;
+  constexpr int KR = APD_SPLIT_RUN;
+  constexpr int RX = (TX + 1 + KR - 1) / KR, RY = (TY + 1 + KR - 1) / KR;
+  constexpr int IX = NP * TY * RX, IY = NP * TX * RY;
+  for (int k = tid; k < IX + IY; k += TX * TY) {
+    const bool ax = k < IX;
+    const int kk = ax ? k : k - IX, nl = ax ? TY : TX, per = ax ? TY * RX : TX * RY;
+    const int p = kk / per, r = kk - p * per, run = r / nl, line = r - run * nl;
+    const int gi = p, ui = NP == 1 ? 1 : (NP == 2 ? 2 + p : (p == 0 ? 1 : 2 + p));
+    const F2* base = ax ? ix + line * S::LX : iy + line;
+    const int fs = ax ? S::LIX : S::LIY;
+    split_run<SCHEME, KR>(base + gi * fs, base + ui * fs, (ax && p == NEGX) ? -1.f : 1.f, ax ? 1 : TX, ax ? S::LX : S::LY, w,
+                          ax ? nx + p * G::NX + line * (TX + 1) : ny + p * G::NY + line, ax ? 1 : TX, run * KR,
+                          ax ? TX + 1 : TY + 1);
+  }
+}
+
+// 8 (f_1 - f_-1) - (f_2 - f_-2) and the fourth difference along a line.
+__device__ __forceinline__ double cd12(const double* f, int st) { return fma(8.0, f[st] - f[-st], f[-2 * st] - f[2 * st]); }
+__device__ __forceinline__ double d4(const double* f, int st) {
+  return fma(-4.0, f[st] + f[-st], fma(6.0, f[0], f[2 * st] + f[-2 * st]));
+}
+__device__ __forceinline__ double dn(const F2* n, int a, int b) { return f2_to_double(f2_sub(n[b], n[a])); }
+
+__device__ __forceinline__ F2 f2_of(double x) {
+  const float h = (float)x;
+  return f2(h, (float)(x - (double)h));
+}
+
+// ---------------------------------------------------------------------------
+// k_explicit (stencil_kernels.cuh) with split fluxes.
+template <int SCHEME, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_explicit_split(const BatchDev* __restrict__ bp, int j, unsigned need,
+                                                                                double weno_eps) {
+  using S = SplitGeo<SCHEME, TX, TY>;
+  using G = typename S::G;
+  constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t bars[2];
+  double* stage = aligned_smem<double>(smem_raw);
+  F2* ix = reinterpret_cast<F2*>(stage + S::NBUF * 6 * PL);
+  F2* iy = ix + 5 * S::LIX;
+  F2* nxs = iy + 5 * S::LIY;   // [3][NX]: (q;v1), (-v1;u1), (v2;u2)
+  F2* nys = nxs + 3 * NX;      // [3][NY]: (q;v2), (v2;u1), (v1;u2)
+  const BatchDev& b = *bp;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const F2 w = f2_of((SCHEME == WENO5_C4 ? 16.0 : 4.0) * weno_eps);
+  const bool needB = (need & NEED_DLFB) != 0, needE = (need & NEED_E) != 0;
+  PlaneList pr;
+  for (int k = 0; k < 6; ++k) pr.add(j, k);
+  tile_loop<double, G, TX, TY, S::NBUF, true>(b, pr, stage, bars, tid, [&](const InstDev& I, const TileRef& t, double* s) {
+    const double* su1 = s;
+    const double* su2 = s + PL;
+    const double* sth = s + 2 * PL;
+    const double* sv1 = s + 3 * PL;
+    const double* sv2 = s + 4 * PL;
+    const double* sq = s + 5 * PL;
+    const int nx = I.nx;
+    const size_t pl = (size_t)nx * I.ny;
+    if (needE && needB) {
+      const double* fx[5] = {sq, sv1, sv2, su1, su2};
+      const double* fy[5] = {sq, sv2, sv1, su1, su2};
+      split_increments<SCHEME, TX, TY, 5>(fx, fy, ix, iy, tid);
+      __syncthreads();
+      split_interfaces<SCHEME, TX, TY, 3, 1>(ix, iy, nxs, nys, w, tid);
+    } else if (needE) {
+      const double* fx[2] = {sq, sv1};
+      const double* fy[2] = {sq, sv2};
+      split_increments<SCHEME, TX, TY, 2>(fx, fy, ix, iy, tid);
+      __syncthreads();
+      split_interfaces<SCHEME, TX, TY, 1, -1>(ix, iy, nxs, nys, w, tid);
+    } else if (needB) {
+      const double* fx[4] = {sv1, sv2, su1, su2};
+      const double* fy[4] = {sv2, sv1, su1, su2};
+      split_increments<SCHEME, TX, TY, 4>(fx, fy, ix, iy, tid);
+      __syncthreads();
+      split_interfaces<SCHEME, TX, TY, 2, 0>(ix, iy, nxs + NX, nys + NY, w, tid);
+    }
+    __syncthreads();
+    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    const Coef<double>& K = I.k64;
+    const double cx = K.cdx, cy = K.cdy;                // 1/(12 h)
+    const int c = G::C00 + ty * BW + tx;
+    const int fa = ty * (TX + 1) + tx, fb = ty * TX + tx;   // this cell's lower interfaces
+    const size_t o = (size_t)(t.y0 + ty) * nx + (t.x0 + tx);
+    double e1 = 0.0, e2 = 0.0;
+    if (needE || (need & NEED_DU)) {
+      const double u1x = cd12(su1 + c, 1), u2y = cd12(su2 + c, BW);
+      if (need & NEED_DU) reinterpret_cast<double*>(I.Du[j])[o] = fma(cx, u1x, cy * u2y);
+      if (needE) {
+        const double u2x = cd12(su2 + c, 1), u1y = cd12(su1 + c, BW);
+        const double gx = (cd12(sq + c, 1) + d4(sv1 + c, 1)) + dn(nxs, fa, fa + 1);
+        const double gy = (cd12(sq + c, BW) + d4(sv2 + c, BW)) + dn(nys, fb, fb + TX);
+        const double a1 = su1[c], a2 = su2[c];
+        // (tau/4) (D0_y u2 - D0_x u1) + tau eps^2 D_x q - (u2^2 - u1^2)/2, and the second component
+        e1 = fma(K.qcy, u2y, fma(-K.qcx, u1x, fma(0.5 * (a1 - a2), a1 + a2, K.tcx * gx)));
+        e2 = fma(K.qcx, u2x, fma(K.qcy, u1y, fma(-a1, a2, K.tcy * gy)));
+        double* e = reinterpret_cast<double*>(I.E[j]);
+        e[o] = e1;
+        e[o + pl] = e2;
+      }
+    }
+    if (need & NEED_LTH) {
+      const double* f = sth + c;
+      const double lx = fma(-30.0, f[0], fma(16.0, f[1] + f[-1], -(f[2] + f[-2])));
+      const double ly = fma(-30.0, f[0], fma(16.0, f[BW] + f[-BW], -(f[2 * BW] + f[-2 * BW])));
+      reinterpret_cast<double*>(I.Lth[j])[o] = fma(K.ldx, lx, K.ldy * ly);
+    }
+    if (needB) {
+      // D_LF . B(v^(j)) + D_0 theta^(j), the only form later stages use them in
+      const double v1x = d4(su1 + c, 1) - cd12(sv1 + c, 1) + dn(nxs + NX, fa, fa + 1);
+      const double v2y = d4(su1 + c, BW) + cd12(sv2 + c, BW) + dn(nys + NY, fb, fb + TX);
+      const double v2x = d4(su2 + c, 1) + cd12(sv2 + c, 1) + dn(nxs + 2 * NX, fa, fa + 1);
+      const double v1y = d4(su2 + c, BW) + cd12(sv1 + c, BW) + dn(nys + 2 * NY, fb, fb + TX);
+      double* db = reinterpret_cast<double*>(I.DLFB[j]);
+      db[o] = fma(cx, v1x + cd12(sth + c, 1), cy * v2y);
+      db[o + pl] = fma(cy, v1y + cd12(sth + c, BW), cx * v2x);
+    }
+    if (need & NEED_V) {
+      double r1, r2;   // step 1 of stage i = j + 1 at this cell
+      relax_v_cell<double, double>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
+      double* vi = reinterpret_cast<double*>(I.Xs[j + 1]);
+      vi[o + 3 * pl] = r1;
+      vi[o + 4 * pl] = r2;
+    }
+  });
+}
+
+// k_update (stencil_kernels.cuh) with split fluxes.
+template <int SCHEME, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_update_split(const BatchDev* __restrict__ bp, int i, double weno_eps,
+                                                                              int close_step, int form) {
+  using S = SplitGeo<SCHEME, TX, TY>;
+  using G = typename S::G;
+  constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t bars[2];
+  const BatchDev& b = *bp;
+  const PlaneList pr = update_planes(b, i);
+  double* stage = aligned_smem<double>(smem_raw);
+  double* sp1 = stage + S::NBUF * pr.n * PL;   // dissipation partner
+  double* sp2 = sp1 + PL;
+  F2* ix = reinterpret_cast<F2*>(sp2 + PL);
+  F2* iy = ix + 4 * S::LIX;
+  F2* nxs = iy + 4 * S::LIY;   // [2][NX]: (-v1;p1), (v2;p2)
+  F2* nys = nxs + 2 * NX;      // [2][NY]: (v2;p1), (v1;p2)
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const F2 w = f2_of((SCHEME == WENO5_C4 ? 16.0 : 4.0) * weno_eps);
+  const unsigned mwp = b.m_wp[i], mim = b.m_im[i];
+  tile_loop<double, G, TX, TY, S::NBUF, true>(b, pr, stage, bars, tid, [&](const InstDev& I, const TileRef& t, double* s) {
+    const double* sth = s;
+    const double* sv1 = s + PL;
+    const double* sv2 = s + 2 * PL;
+    const int nx = I.nx;
+    const size_t pl = (size_t)nx * I.ny;
+    const Coef<double>& K = I.k64;
+    // dissipation partner of D_LF . B(v^(i)), the explicit-weight predictor (1/a_ii) sum_{j<i} (atilde_ij - a_ij) u^(j)
+    for (int e = tid; e < BW * G::BH; e += TX * TY) {
+      double p1 = 0.0, p2 = 0.0;
+      int k = 3;
+      bool any = false;
+      for (int jj = 1; jj < i; ++jj) {
+        if (has(mwp, jj)) {
+          const double a = K.wp[i][jj], x1 = s[k * PL + e], x2 = s[(k + 1) * PL + e];
+          p1 = any ? fma(a, x1, p1) : a * x1;
+          p2 = any ? fma(a, x2, p2) : a * x2;
+          any = true;
+          k += 2;
+        }
+      }
+      sp1[e] = p1;
+      sp2[e] = p2;
+    }
+    __syncthreads();
+    const double* fx[4] = {sv1, sv2, sp1, sp2};
+    const double* fy[4] = {sv2, sv1, sp1, sp2};
+    split_increments<SCHEME, TX, TY, 4>(fx, fy, ix, iy, tid);
+    __syncthreads();
+    split_interfaces<SCHEME, TX, TY, 2, 0>(ix, iy, nxs, nys, w, tid);
+    __syncthreads();
+    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    const double cx = K.cdx, cy = K.cdy;
+    const int c = G::C00 + ty * BW + tx;
+    const int fa = ty * (TX + 1) + tx, fb = ty * TX + tx;
+    const size_t o = (size_t)(t.y0 + ty) * nx + (t.x0 + tx);
+    const double dv1x = cd12(sv1 + c, 1), dv2y = cd12(sv2 + c, BW);
+    const double v1x = d4(sp1 + c, 1) - dv1x + dn(nxs, fa, fa + 1);
+    const double v2y = d4(sp1 + c, BW) + dv2y + dn(nys, fb, fb + TX);
+    const double v2x = d4(sp2 + c, 1) + cd12(sv2 + c, 1) + dn(nxs + NX, fa, fa + 1);
+    const double v1y = d4(sp2 + c, BW) + cd12(sv1 + c, BW) + dn(nys + NY, fb, fb + TX);
+    const double dg1 = fma(cx, v1x + cd12(sth + c, 1), cy * v2y);    // D_LF . B(v^(i)) + D_0 theta^(i)
+    const double dg2 = fma(cy, v1y + cd12(sth + c, BW), cx * v2x);
+    const double dvi = fma(cx, dv1x, cy * dv2y);
+    // step 3
+    double s1 = K.aim[i][i] * dg1, s2 = K.aim[i][i] * dg2;
+    for (int jj = 1; jj < i; ++jj) {
+      if (has(mim, jj)) {
+        const double* bg = reinterpret_cast<const double*>(I.DLFB[jj]);
+        s1 = fma(K.aim[i][jj], bg[o], s1);
+        s2 = fma(K.aim[i][jj], bg[o + pl], s2);
+      }
+    }
+    const double* Xn = reinterpret_cast<const double*>(I.X);
+    double* out = reinterpret_cast<double*>(I.Xs[i]);
+    const double u1 = fma(-K.dt, s1, Xn[o]), u2 = fma(-K.dt, s2, Xn[o + pl]);
+    if (!close_step) {
+      out[o] = u1;
+      out[o + pl] = u2;
+      reinterpret_cast<double*>(I.Dv[i])[o] = dvi;   // D0 . v^(i) for the q steps of later stages
+    }
+    // step 4
+    double qi = K.r_n[i] * Xn[o + 5 * pl];
+    for (int jj = 1; jj <= i; ++jj) {
+      if (!has(mim, jj)) continue;
+      const double dv = (jj == i) ? dvi : reinterpret_cast<const double*>(I.Dv[jj])[o];
+      qi = fma(K.rq_d[i][jj], dv, qi);
+      if (jj < i) qi = fma(K.rv_v[i][jj], reinterpret_cast<const double*>(I.Xs[jj])[o + 5 * pl], qi);
+    }
+    if (!close_step) {
+      out[o + 5 * pl] = qi;
+      return;
+    }
+    const double m[6] = {u1, u2, sth[c], sv1[c], sv2[c], qi};
+    if (close_step_cell<double>(I, o, pl, m, form, reinterpret_cast<double*>(I.Xnext))) atomicOr(b.err, 1u);
+  });
+}
+
+}  // namespace apd

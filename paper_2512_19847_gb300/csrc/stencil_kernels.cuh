@@ -174,12 +174,13 @@ __device__ __forceinline__ void stage_begin(const BatchDev& b, int it, const Pla
 }
 
 // The persistent, double-buffered tile loop: body(I, tile, staged planes) runs
-// for every tile of the batch assigned to this block.
-template <typename T, class G, int TX, int TY, int NB = 2, class Body>
+// for every tile of the batch assigned to this block (SPLIT: the tiles of the
+// instances with split fluxes, which come last; else those of the others).
+template <typename T, class G, int TX, int TY, int NB = 2, bool SPLIT = false, class Body>
 __device__ __forceinline__ void tile_loop(const BatchDev& b, const PlaneList& pr, T* stage0, uint64_t* bars, int tid,
                                           Body&& body) {
   constexpr int NT = TX * TY;
-  const int ntiles = b.counts[0];
+  const int ntiles = b.counts[SPLIT ? 0 : 5];
   const int bstride = pr.n * G::PL;       // buffer 1 starts at stage0 + bstride
   if (tid == 0) {
     mbar_init(&bars[0], 1);
@@ -188,7 +189,7 @@ __device__ __forceinline__ void tile_loop(const BatchDev& b, const PlaneList& pr
   }
   __syncthreads();
   unsigned phase = 0u;                    // bit c: parity of the next phase of bars[c]
-  int it = blockIdx.x;
+  int it = blockIdx.x + (SPLIT ? b.counts[5] : 0);
   if constexpr (NB == 1) {
     // single buffer: stage the tile, wait, compute, then the next tile
     for (; it < ntiles; it += gridDim.x) {

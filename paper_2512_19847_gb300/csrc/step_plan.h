@@ -17,6 +17,10 @@ namespace apd {
 enum KernelKind { KK_EXPLICIT, KK_RHS, KK_ROWS_FWD, KK_COLS, KK_ROWS_INV, KK_UPDATE, KK_FINISH, KK_STAGE1 };
 
 // Kinds of Helmholtz transform work a batch holds (bits of StepKernels::fft_kinds).
+// Kinds of stencil work a batch holds (bits of StepKernels::stencil_kinds): instances whose fluxes are
+// evaluated whole, and those that take the split fluxes (split_flux.cuh).
+enum StencilKinds { STENCIL_WHOLE = 1, STENCIL_SPLIT = 2 };
+
 enum FftKinds { FFT_X_POW2 = 1, FFT_X_BS = 2, FFT_Y_POW2 = 4, FFT_Y_BS = 8 };
 
 // Transform launches of one implicit stage for the given kinds.
@@ -33,6 +37,9 @@ struct StepKernels {
   size_t smem_update;
   unsigned fft_kinds;   // FftKinds present among the attached solves
   int g_rows;           // grid of the power-of-two row passes (km.rows_threads threads per block)
+  unsigned stencil_kinds = STENCIL_WHOLE;   // StencilKinds present among the attached solves
+  int g_explicit_split = 0, g_update_split = 0;
+  size_t smem_update_split = 0;
 };
 
 // Planes k_update stages at its largest stage: theta, v1, v2 and u1, u2 of every
@@ -63,6 +70,25 @@ inline int fft_eblk(int nmax) { return nmax > 2048 ? nmax : 2048; }
 inline int fft_eblk_cols(int nmax, bool f32) {
   const int e = f32 ? 8192 : 4096;
   return nmax > e ? nmax : e;
+}
+
+inline size_t update_smem_split(const StencilSet& ks, const ap_dvm_params& t) {
+  return ks.update_fixed_split + (size_t)ks.nbuf_split * update_planes_max(t) * ks.plane_bytes;
+}
+
+// Whether the fluxes of a solve are split (split_flux.cuh): FP64 with a WENO scheme and at least
+// kSplitMinCells cells on each side.
+// Why the line lies there: the pairs of floats round the nonlinear terms, third (WENO3: second)
+// differences times weights, to about 2^-47 of their size, FP64 rounds the whole flux to 2^-52 of
+// its own.  For fields of wavenumbers up to 16 (the workloads') the rms error of a flux difference
+// against 113-bit arithmetic, split and whole, in units of 1e-17: WENO5 at 2048 cells a side 1.6 and
+// 5.3, 512: 2.0 and 5.3, 256: 2.9 and 5.3, 128: 8.3 and 5.4; WENO3 at 256: 5.5 and 5.5, 128: 20 and
+// 5.7.  Whole steps against 64-bit-mantissa arithmetic (relative, theta plane, which carries the
+// largest error): 1024^2 Taylor-Green 1.14e-14 split, 1.37e-14 whole; 256^2 random field 1.9e-15 and
+// 2.9e-15; 256^2 WENO3 layer 4.4e-15 and 5.6e-15; u, v and q likewise at or below the whole form.
+constexpr int kSplitMinCells = 256;
+inline bool split_fluxes(const ap_dvm_params& p) {
+  return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;
 }
 
 inline size_t update_smem(const StencilSet& ks, const ap_dvm_params& t) {
@@ -136,7 +162,10 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     if (j == 1 && !type_a) need |= 2u;                     // D0 . u^n (= D0 . u^(1)) enters every right-hand side
     if (j >= 1) {
       void* a[] = {&bp, &j, &need, &weno_eps};
-      if ((st = launch(K.ks.k_explicit, K.g_explicit, blk, K.ks.smem_explicit, a, KK_EXPLICIT))) return st;
+      if ((K.stencil_kinds & STENCIL_WHOLE) && (st = launch(K.ks.k_explicit, K.g_explicit, blk, K.ks.smem_explicit, a, KK_EXPLICIT))) return st;
+      if ((K.stencil_kinds & STENCIL_SPLIT) &&
+          (st = launch(K.ks.k_explicit_split, K.g_explicit_split, blk, K.ks.smem_explicit_split, a, KK_EXPLICIT)))
+        return st;
     }
     double sign = -1.0;   // theta-history term with a minus sign (the stage equations of Sec. 3.1)
     int first = (i == (type_a ? 1 : 2)) ? 1 : 0;           // the first right-hand side also sums theta^n
@@ -159,7 +188,10 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     {
       int close = (fused && i == s) ? 1 : 0;
       void* a[] = {&bp, &i, &weno_eps, &close, &form};
-      if ((st = launch(K.ks.k_update, K.g_update, blk, K.smem_update, a, KK_UPDATE))) return st;
+      if ((K.stencil_kinds & STENCIL_WHOLE) && (st = launch(K.ks.k_update, K.g_update, blk, K.smem_update, a, KK_UPDATE))) return st;
+      if ((K.stencil_kinds & STENCIL_SPLIT) &&
+          (st = launch(K.ks.k_update_split, K.g_update_split, blk, K.smem_update_split, a, KK_UPDATE)))
+        return st;
     }
   }
   if (fused) return 0;
@@ -178,6 +210,14 @@ inline void fill_coef(const ap_dvm_params& p, const InstDev& d, Coef<T>& k) {
   k.htau = T(0.5 * d.tau);
   k.inv_dx = T(d.inv_dx);
   k.inv_dy = T(d.inv_dy);
+  k.cdx = T(d.inv_dx / 12.0);
+  k.cdy = T(d.inv_dy / 12.0);
+  k.qcx = T(0.25 * d.tau * d.inv_dx / 12.0);
+  k.qcy = T(0.25 * d.tau * d.inv_dy / 12.0);
+  k.tcx = T(d.te2 * d.inv_dx / 12.0);
+  k.tcy = T(d.te2 * d.inv_dy / 12.0);
+  k.ldx = T(d.inv_dx * d.inv_dx / 12.0);
+  k.ldy = T(d.inv_dy * d.inv_dy / 12.0);
   for (int i = 1; i <= p.s; ++i)
     for (int j = 1; j <= p.s; ++j) {
       k.aex[i][j] = T(p.A_ex[(i - 1) * AP_DVM_MAX_STAGES + (j - 1)]);
