@@ -263,9 +263,9 @@ int auto_tile(const ap_dvm_handle* h) {
   for (const Slot& s : h->slots)
     if (s.attached) { minx = std::min(minx, s.p.nx); miny = std::min(miny, s.p.ny); }
   if (minx == (1 << 30)) { minx = h->tmpl.nx; miny = h->tmpl.ny; }
-  for (int t : {0, 1, 2, 3})
-    if (kTileX[t] <= minx && kTileY[t] <= miny) return t;
-  return 3;
+  return pick_tile(h->f32, minx, miny, h->capacity == 1 ? h->num_sms : 0, [&](int t) {
+    return (long long)((minx + kTileX[t] - 1) / kTileX[t]) * ((miny + kTileY[t] - 1) / kTileY[t]);
+  });
 }
 
 StencilSet stencil_for(int f32, int scheme, int tile) {

@@ -10,6 +10,33 @@ constexpr int kNumTiles = 6;
 constexpr int kTileX[kNumTiles] = {32, 32, 16, 8, 64, 32};
 constexpr int kTileY[kNumTiles] = {8, 4, 8, 8, 4, 16};
 
+// The automatic tile shape for grids of at least minx x miny cells.  tiles(t) is the number of
+// tiles of shape t over all of them, num_sms 0 when it is not to be looked at (a batch, whose
+// tiles come and go).
+//   FP32: 16x8 (7 blocks of 128 threads per SM); 2048^2, 4 steps, explicit + update: 1.55 + 2.00 ms
+//   against 1.82 + 2.65 with 32x8 and 1.99 + 2.31 with 8x8; 509x251: 0.14 + 0.16 against 0.20 +
+//   0.23 and 0.16 + 0.18; 24 uneven solves: 1.33 + 1.66 against 1.58 + 2.23 and 1.69 + 1.91.
+//   FP64: 32x8 while it gives two tiles per SM (2048^2: 2.16 + 2.18 against 2.12 + 2.31 with 16x8
+//   and 2.33 + 2.51 with 8x8), else the next smaller: a grid of fewer tiles leaves SMs, and with
+//   them FP64 pipes, idle (64^2, 10 steps: 0.78 + 0.78 ms with 16 tiles of 32x8, 0.55 + 0.57 with
+//   64 of 8x8; 384x192 LF1: 0.29 + 0.26 with 288 of 32x8, 0.26 + 0.24 with 576 of 16x8).
+template <class Tiles>
+inline int pick_tile(bool f32, int minx, int miny, int num_sms, Tiles&& tiles) {
+  static constexpr int order64[4] = {0, 1, 2, 3}, order32[2] = {2, 3}, small64[3] = {0, 2, 3};
+  auto fits = [&](int t) { return kTileX[t] <= minx && kTileY[t] <= miny; };
+  if (f32) {
+    for (int t : order32)
+      if (fits(t)) return t;
+  } else if (num_sms > 0) {
+    for (int t : small64)
+      if (fits(t) && tiles(t) >= 2LL * num_sms) return t;
+  } else {
+    for (int t : order64)
+      if (fits(t)) return t;
+  }
+  return 3;
+}
+
 struct StencilSet {
   const void* k_explicit;
   const void* k_rhs;

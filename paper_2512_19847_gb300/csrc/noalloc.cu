@@ -95,10 +95,8 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   int sms = 0;
   NA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
-  // kernels: the tile rule of the handle path (largest of 32x8, 32x4, 16x8, 8x8 that fits)
-  int tile = 3;
-  for (int t : {0, 1, 2, 3})
-    if (kTileX[t] <= p->nx && kTileY[t] <= p->ny) { tile = t; break; }
+  // kernels: the tile rule of the handle path for one solve
+  const int tile = pick_tile(false, p->nx, p->ny, sms, [&](int t) { return (long long)(p->nx / kTileX[t]) * (p->ny / kTileY[t]); });
   StencilSet ks = p->space_scheme == AP_DVM_LF1_C2 ? stencil_f64_lf1(tile)
                 : p->space_scheme == AP_DVM_WENO3_C4 ? stencil_f64_w3(tile) : stencil_f64_w5(tile);
   MiscSet km = misc_set(0, tile);
