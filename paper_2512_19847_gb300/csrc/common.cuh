@@ -74,6 +74,7 @@ struct InstDev {
   double inv_aii[APD_MAXS + 1];              // 1 / a_ii
   Coef<double> k64;             // the stage coefficients in FP64 ...
   Coef<float> k32;              // ... and rounded once to FP32
+  float wp_lo[APD_MAXS + 1][APD_MAXS + 1];   // k64.wp - k32.wp
   void* X;                      // 6 planes: state at t^n (moments)
   void* Xnext;                  // 6 planes the last stage's update writes the state at t^{n+1} to (the
                                 // other buffer of a double-buffered state; null: a separate finish kernel)

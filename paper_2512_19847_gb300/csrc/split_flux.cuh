@@ -8,21 +8,18 @@
 // it starts from are taken in FP64, so that the pair's relative rounding (2^-48)
 // applies to increments between neighbouring cells and not to the values.
 //
-// WENO5.  With g+- = g +- U (twice the Lax-Friedrichs split), interface i + 1/2,
-// D_k = f_{k+1} - f_k, third differences T_k = f_{k+2} - 3 f_{k+1} + 3 f_k - f_{k-1},
-// and the reconstruction about its centred candidate,
-//   6 (L(g+) + R(g-)) = [-g_{i-1} + 7 g_i + 7 g_{i+1} - g_{i+2}] + T_i(U) + N_{i+1/2},
-//   N = -(2 w0 T_{i-1} + w2 T_i)(g+) + (2 w0 T_{i+1} + w2 T_i)(g-),
+// With g+- = g +- U (twice the Lax-Friedrichs split), interface i + 1/2, increments
+// D_k = f_{k+1} - f_k, second differences c_k = D_k - D_{k-1} and third differences
+// T_k = c_{k+1} - c_k, the two reconstructions are (WENO5, about the centred candidate)
+//   6 L(g+) = 3 (g+_i + g+_{i+1}) - [c_i + 2 w0 T_{i-1} + w2 T_i](g+),
+//   6 R(g-) = 3 (g-_i + g-_{i+1}) - [c_{i+1} - 2 w0 T_{i+1} - w2 T_i](g-),
 // so that the flux difference of cell i is 1/(12 h) times
-//   8 (g_{i+1} - g_{i-1}) - (g_{i+2} - g_{i-2}) + (fourth difference of U) + N_{i+1/2} - N_{i-1/2}.
-// The smoothness indicators (times 4, plus 4 eps_W) are sums of squares of
-// increments: (13/3) (D_k - D_{k-1})^2 + l^2 + 4 eps_W with l = 3 D_k - D_{k-1},
-// D_{k-1} + D_k or D_k - 3 D_{k-1} for the three candidates.
-//
-// WENO3.  The same with w0 = 1/3 + (w0 - 1/3) for the weight of the outer candidate: the 1/3 gives
-// the linear part above, and
-//   N = -3 ((w0 - 1/3)(g+) c_i(g+) + (w0 - 1/3)(g-) c_{i+1}(g-))
-// with second differences c_k (taken whole, w0 c would be less exact than FP64 at 256 cells a side).
+//   6 (g_{i+1} - g_{i-1}) + N_{i+1/2} - N_{i-1/2},
+// N the two brackets, negated: the only term that is linear in the values and not in their
+// increments is a central difference of g, one FP64 operation.  The smoothness indicators (times 4,
+// plus 4 eps_W) are sums of squares of increments: (13/3) c_k^2 + l^2 + 4 eps_W with
+// l = 3 D_k - D_{k-1}, D_{k-1} + D_k or D_k - 3 D_{k-1} for the three candidates.
+// WENO3: the brackets are 3 w0 c_i (g+) and 3 w0 c_{i+1} (g-), taken as (1 + 3 (w0 - 1/3)) c.
 #pragma once
 #include "common.cuh"
 
@@ -101,8 +98,8 @@ __device__ __forceinline__ double f2_widen1(float x) {
 }
 __device__ __forceinline__ double f2_to_double(F2 a) { return f2_widen1(a.h) + f2_widen1(a.l); }
 
-// Nonlinear part of one WENO5 reconstruction for each of KR neighbouring interfaces:
-// q[m] = 2 w0 T_{out} + w2 T_{in} from the increments D[m .. m + 3] of its stencil (upwind
+// The bracket of one WENO5 reconstruction for each of KR neighbouring interfaces:
+// q[m] = c + 2 w0 T_{out} + w2 T_{in} from the increments D[m .. m + 3] of its stencil (upwind
 // to downwind; T_out = D[m+2] - 2 D[m+1] + D[m], T_in one further), w = 16 eps_W (the
 // indicators times 4, the doubled split).  With the e_k scaled by a power of two so that the
 // largest is about 1, and then their products likewise, every step stays in the float range
@@ -136,11 +133,11 @@ __device__ __forceinline__ void w5_split(const F2* D, F2 w, F2* q) {
     const F2 A = f2_sqr(pa), B = f2_scale(f2_sqr(pb), 6.f), E = f2_scale(f2_sqr(pc), 3.f);
     const F2 den = f2_add(f2_add(A, E), B);
     const F2 to = f2_sub(c[m + 2], c[m + 1]), ti = f2_sub(c[m + 3], c[m + 2]);
-    q[m] = f2_div(f2_addk<2>(f2_mul(E, ti), f2_mul(A, to)), den);
+    q[m] = f2_add(c[m + 2], f2_div(f2_addk<2>(f2_mul(E, ti), f2_mul(A, to)), den));
   }
 }
 
-// The same for WENO3: q[m] = 3 (w0 - 1/3) c with c = D[m+1] - D[m] (upwind, then downwind increment),
+// The same for WENO3: q[m] = c + 3 (w0 - 1/3) c with c = D[m+1] - D[m] (upwind, then downwind increment),
 // w = 4 eps_W, indicators e_k = D_k^2 + w: w0 = e1^2 / (e1^2 + 2 e0^2) and
 // 3 (w0 - 1/3) = 2 (e1 - e0)(e1 + e0) / (e1^2 + 2 e0^2), e1 - e0 = c (D[m] + D[m+1]).
 template <int KR>
@@ -155,7 +152,7 @@ __device__ __forceinline__ void w3_split(const F2* D, F2 w, F2* q) {
     const F2 c = f2_sub(D[m + 1], D[m]), d = f2_add(D[m + 1], D[m]);
     const F2 n = f2_mul(f2_mul(f2_mul(c, f2(d.h * se, d.l * se)), f2_add(e0, e1)), c);
     const F2 r = f2_div(n, f2_addk<2>(f2_sqr(e1), f2_sqr(e0)));
-    q[m] = f2(2.f * r.h, 2.f * r.l);
+    q[m] = f2_addk<2>(c, r);
   }
 }
 

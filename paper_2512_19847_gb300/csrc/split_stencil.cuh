@@ -3,15 +3,17 @@
 //   1. FP64 increments along both axes, kept as pairs of floats (one FP64 operation each),
 //   2. the nonlinear interface terms N, on the FP32 pipe, in runs of neighbouring interfaces,
 //   3. per cell: the linear parts and the closed forms in FP64, with the differences of N.
-// What bounds them is still the FP64 pipe (2 operations per clock and SM), now with about 130
-// (explicit, all terms) and 75 (update) FP64 operations per cell instead of 510 and 370, beside
+// What bounds them is still the FP64 pipe (2 operations per clock and SM), now with about 110
+// (explicit, all terms) and 70 (update) FP64 operations per cell instead of 510 and 370, beside
 // about 450 FP32 instructions per interface.  WENO5 at 2048^2, ms per step (32x8 tiles): explicit
-// 6.17 -> 2.16, update 6.06 -> 2.18; WENO3 at 256^2, 10 steps: 0.98 -> 0.55 and 1.00 -> 0.53.
-// Measured choices (2048^2, explicit + update, ms): WENO5 768 threads per SM (85 registers)
-// 2.16 + 2.18, 512 (128 registers) 2.30 + 2.31; one staged plane buffer 2.30 + 2.31 against 2.31 +
-// 2.35 with two (at 512 threads; the second block on the SM hides the copies); runs of 3
-// interfaces 2.30 + 2.31, of 4 2.37 + 2.55.  WENO3 keeps 512 threads: 2.03 + 1.99 against 1.98 +
-// 1.86 at 2048^2 but 0.056 + 0.053 against 0.070 + 0.066 at 256^2, the size it is run at.
+// 6.17 -> 1.77, update 6.06 -> 1.68 (2.16 and 2.18 with the fourth-order difference of g and the
+// fourth difference of U in FP64 and the partner as FP64 planes); WENO3 at 256^2, 10 steps:
+// 0.98 -> 0.47 and 1.00 -> 0.44.  Measured choices, with those earlier terms (2048^2, explicit +
+// update, ms): WENO5 768 threads per SM (85 registers) 2.16 + 2.18, 512 (128 registers) 2.30 + 2.31;
+// one staged plane buffer 2.30 + 2.31 against 2.31 + 2.35 with two (at 512 threads; the other blocks
+// on the SM hide the copies); runs of 3 interfaces 2.30 + 2.31, of 4 2.37 + 2.55.  WENO3 keeps 512
+// threads: 2.03 + 1.99 against 1.98 + 1.86 at 2048^2 but 0.056 + 0.053 against 0.070 + 0.066 at
+// 256^2, the size it is run at.
 #pragma once
 #include "split_flux.cuh"
 #include "stencil_kernels.cuh"
@@ -41,7 +43,7 @@ struct SplitGeo {
   // elements of 8 bytes besides the staged planes: increments of F fields per axis, N of P pairs per axis
   static constexpr int extra(int F, int P) { return F * (LIX + LIY) + P * (G::NX + G::NY); }
   static constexpr size_t explicit_bytes = 128 + 8 * (size_t)(NBUF * 6 * G::PL + extra(5, 3));
-  static constexpr size_t update_fixed_bytes = 128 + 8 * (size_t)(2 * G::PL + extra(4, 2));
+  static constexpr size_t update_fixed_bytes = 128 + 8 * (size_t)extra(4, 2);
 };
 
 template <int SCHEME, int THREADS>
@@ -65,6 +67,36 @@ __device__ __forceinline__ void split_increments(const double* const* fx, const 
 #pragma unroll
       for (int f = 0; f < NF; ++f) iy[f * S::LIY + r] = f2_from_double(fy[f][o + G::BW] - fy[f][o]);
     }
+  }
+}
+
+// Pass 1 of the update: increments of v1, v2 and of the dissipation partner
+// P = sum over the earlier stages' staged u planes (from plane 3 on) of weight (wh + wl) times u,
+// formed from the planes' increments.
+template <int SCHEME, int TX, int TY>
+__device__ __forceinline__ void split_increments_update(const double* s, int nw, const F2* wt, F2* ix, F2* iy, int tid) {
+  using S = SplitGeo<SCHEME, TX, TY>;
+  using G = typename S::G;
+  constexpr int PL = G::PL;
+  for (int k = tid; k < S::LIX + S::LIY; k += TX * TY) {
+    const bool ax = k < S::LIX;
+    const int r = ax ? k : k - S::LIX, line = ax ? r / S::LX : r % TX, pt = ax ? r - line * S::LX : r / TX;
+    const int o = ax ? (G::H + line) * G::BW + G::XO + pt : pt * G::BW + G::XO + G::H + line, st = ax ? 1 : G::BW;
+    F2* out = (ax ? ix : iy) + r;
+    const int fs = ax ? S::LIX : S::LIY;
+    const double* v = s + PL + o;
+    const F2 d1 = f2_from_double(v[st] - v[0]), d2 = f2_from_double(v[PL + st] - v[PL]);
+    out[0] = ax ? d1 : d2;
+    out[fs] = ax ? d2 : d1;
+    F2 p1 = f2(0.f, 0.f), p2 = p1;
+    const double* u = s + 3 * PL + o;
+    for (int m = 0; m < nw; ++m, u += 2 * PL) {
+      const F2 a1 = f2_mul(wt[m], f2_from_double(u[st] - u[0])), a2 = f2_mul(wt[m], f2_from_double(u[PL + st] - u[PL]));
+      p1 = m ? f2_add(p1, a1) : a1;
+      p2 = m ? f2_add(p2, a2) : a2;
+    }
+    out[2 * fs] = p1;
+    out[3 * fs] = p2;
   }
 }
 
@@ -127,10 +159,10 @@ __device__ __forceinline__ double cd12(const double* f, int st) { return fma(8.0
 __device__ __forceinline__ double cd12s(const double* f, int st) {
   return fma(-8.0, f[-st], fma(8.0, f[st], -f[2 * st])) + f[-2 * st];
 }
-__device__ __forceinline__ double d4(const double* f, int st) {
-  return fma(-4.0, f[st] + f[-st], fma(6.0, f[0], f[2 * st] + f[-2 * st]));
+// 12 h times the flux difference of g: 6 (g_1 - g_-1) and the difference of N.
+__device__ __forceinline__ double fd12(const double* g, int st, double sg6, const F2* n, int a, int b) {
+  return fma(sg6, g[st] - g[-st], f2_to_double(f2_sub(n[b], n[a])));
 }
-__device__ __forceinline__ double dn(const F2* n, int a, int b) { return f2_to_double(f2_sub(n[b], n[a])); }
 
 __device__ __forceinline__ F2 f2_of(double x) {
   const float h = (float)x;
@@ -199,8 +231,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
       if (need & NEED_DU) reinterpret_cast<double*>(I.Du[j])[o] = fma(cx, u1x, cy * u2y);
       if (needE) {
         const double u2x = cd12(su2 + c, 1), u1y = cd12(su1 + c, BW);
-        const double gx = (cd12(sq + c, 1) + d4(sv1 + c, 1)) + dn(nxs, fa, fa + 1);
-        const double gy = (cd12(sq + c, BW) + d4(sv2 + c, BW)) + dn(nys, fb, fb + TX);
+        const double gx = fd12(sq + c, 1, 6.0, nxs, fa, fa + 1), gy = fd12(sq + c, BW, 6.0, nys, fb, fb + TX);
         const double a1 = su1[c], a2 = su2[c];
         // (tau/4) (D0_y u2 - D0_x u1) + tau eps^2 D_x q - (u2^2 - u1^2)/2, and the second component
         e1 = fma(K.qcy, u2y, fma(-K.qcx, u1x, fma(0.5 * (a1 - a2), a1 + a2, K.tcx * gx)));
@@ -218,10 +249,8 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     }
     if (needB) {
       // D_LF . B(v^(j)) + D_0 theta^(j), the only form later stages use them in
-      const double v1x = d4(su1 + c, 1) - cd12(sv1 + c, 1) + dn(nxs + NX, fa, fa + 1);
-      const double v2y = d4(su1 + c, BW) + cd12(sv2 + c, BW) + dn(nys + NY, fb, fb + TX);
-      const double v2x = d4(su2 + c, 1) + cd12(sv2 + c, 1) + dn(nxs + 2 * NX, fa, fa + 1);
-      const double v1y = d4(su2 + c, BW) + cd12(sv1 + c, BW) + dn(nys + 2 * NY, fb, fb + TX);
+      const double v1x = fd12(sv1 + c, 1, -6.0, nxs + NX, fa, fa + 1), v2y = fd12(sv2 + c, BW, 6.0, nys + NY, fb, fb + TX);
+      const double v2x = fd12(sv2 + c, 1, 6.0, nxs + 2 * NX, fa, fa + 1), v1y = fd12(sv1 + c, BW, 6.0, nys + 2 * NY, fb, fb + TX);
       double* db = reinterpret_cast<double*>(I.DLFB[j]);
       db[o] = fma(cx, v1x + cd12(sth + c, 1), cy * v2y);
       db[o + pl] = fma(cy, v1y + cd12(sth + c, BW), cx * v2x);
@@ -248,9 +277,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
   const BatchDev& b = *bp;
   const PlaneList pr = update_planes(b, i);
   double* stage = aligned_smem<double>(smem_raw);
-  double* sp1 = stage + S::NBUF * pr.n * PL;   // dissipation partner
-  double* sp2 = sp1 + PL;
-  F2* ix = reinterpret_cast<F2*>(sp2 + PL);
+  F2* ix = reinterpret_cast<F2*>(stage + S::NBUF * pr.n * PL);
   F2* iy = ix + 4 * S::LIX;
   F2* nxs = iy + 4 * S::LIY;   // [2][NX]: (-v1;p1), (v2;p2)
   F2* nys = nxs + 2 * NX;      // [2][NY]: (v2;p1), (v1;p2)
@@ -264,27 +291,18 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     const int nx = I.nx;
     const size_t pl = (size_t)nx * I.ny;
     const Coef<double>& K = I.k64;
-    // dissipation partner of D_LF . B(v^(i)), the explicit-weight predictor (1/a_ii) sum_{j<i} (atilde_ij - a_ij) u^(j)
-    for (int e = tid; e < BW * G::BH; e += TX * TY) {
-      double p1 = 0.0, p2 = 0.0;
-      int k = 3;
-      bool any = false;
-      for (int jj = 1; jj < i; ++jj) {
-        if (has(mwp, jj)) {
-          const double a = K.wp[i][jj], x1 = s[k * PL + e], x2 = s[(k + 1) * PL + e];
-          p1 = any ? fma(a, x1, p1) : a * x1;
-          p2 = any ? fma(a, x2, p2) : a * x2;
-          any = true;
-          k += 2;
-        }
+    // weights of the dissipation partner of D_LF . B(v^(i)), the explicit-weight predictor
+    // (1/a_ii) sum_{j<i} (atilde_ij - a_ij) u^(j), as pairs (k32.wp and its remainder)
+    F2 wt[APD_MAXS - 1];
+    int nw = 0;
+#pragma unroll
+    for (int jj = 1; jj < APD_MAXS; ++jj)
+      if (jj < i && has(mwp, jj)) {
+        const F2 a = f2(I.k32.wp[i][jj], I.wp_lo[i][jj]);
+        if (nw == 0) wt[0] = a; else if (nw == 1) wt[1] = a; else wt[2] = a;
+        ++nw;
       }
-      sp1[e] = p1;
-      sp2[e] = p2;
-    }
-    __syncthreads();
-    const double* fx[4] = {sv1, sv2, sp1, sp2};
-    const double* fy[4] = {sv2, sv1, sp1, sp2};
-    split_increments<SCHEME, TX, TY, 4>(fx, fy, ix, iy, tid);
+    split_increments_update<SCHEME, TX, TY>(s, nw, wt, ix, iy, tid);
     __syncthreads();
     split_interfaces<SCHEME, TX, TY, 2, 0>(ix, iy, nxs, nys, w, tid);
     __syncthreads();
@@ -293,11 +311,11 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     const int c = G::C00 + ty * BW + tx;
     const int fa = ty * (TX + 1) + tx, fb = ty * TX + tx;
     const size_t o = (size_t)(t.y0 + ty) * nx + (t.x0 + tx);
-    const double dv1x = cd12(sv1 + c, 1), dv2y = cd12(sv2 + c, BW);
-    const double v1x = d4(sp1 + c, 1) - dv1x + dn(nxs, fa, fa + 1);
-    const double v2y = d4(sp1 + c, BW) + dv2y + dn(nys, fb, fb + TX);
-    const double v2x = d4(sp2 + c, 1) + cd12(sv2 + c, 1) + dn(nxs + NX, fa, fa + 1);
-    const double v1y = d4(sp2 + c, BW) + cd12(sv1 + c, BW) + dn(nys + NY, fb, fb + TX);
+    const double dv1 = sv1[c + 1] - sv1[c - 1], dv2 = sv2[c + BW] - sv2[c - BW];
+    const double dv1x = fma(8.0, dv1, sv1[c - 2] - sv1[c + 2]), dv2y = fma(8.0, dv2, sv2[c - 2 * BW] - sv2[c + 2 * BW]);
+    const double v1x = fma(-6.0, dv1, f2_to_double(f2_sub(nxs[fa + 1], nxs[fa])));
+    const double v2y = fma(6.0, dv2, f2_to_double(f2_sub(nys[fb + TX], nys[fb])));
+    const double v2x = fd12(sv2 + c, 1, 6.0, nxs + NX, fa, fa + 1), v1y = fd12(sv1 + c, BW, 6.0, nys + NY, fb, fb + TX);
     const double dg1 = fma(cx, v1x + cd12(sth + c, 1), cy * v2y);    // D_LF . B(v^(i)) + D_0 theta^(i)
     const double dg2 = fma(cy, v1y + cd12(sth + c, BW), cx * v2x);
     const double dvi = fma(cx, dv1x, cy * dv2y);

@@ -78,14 +78,15 @@ inline size_t update_smem_split(const StencilSet& ks, const ap_dvm_params& t) {
 
 // Whether the fluxes of a solve are split (split_flux.cuh): FP64 with a WENO scheme and at least
 // kSplitMinCells cells on each side.
-// Why the line lies there: the pairs of floats round the nonlinear terms, third (WENO3: second)
-// differences times weights, to about 2^-47 of their size, FP64 rounds the whole flux to 2^-52 of
-// its own.  For fields of wavenumbers up to 16 (the workloads') the rms error of a flux difference
-// against 113-bit arithmetic, split and whole, in units of 1e-17: WENO5 at 2048 cells a side 1.6 and
-// 5.3, 512: 2.0 and 5.3, 256: 2.9 and 5.3, 128: 8.3 and 5.4; WENO3 at 256: 5.5 and 5.5, 128: 20 and
-// 5.7.  Whole steps against 64-bit-mantissa arithmetic (relative, theta plane, which carries the
-// largest error): 1024^2 Taylor-Green 1.14e-14 split, 1.37e-14 whole; 256^2 random field 1.9e-15 and
-// 2.9e-15; 256^2 WENO3 layer 4.4e-15 and 5.6e-15; u, v and q likewise at or below the whole form.
+// Why the line lies there: the pairs of floats round second and third differences to about 2^-47 of
+// the increments, FP64 rounds the whole flux to 2^-52 of its own size.  For fields of wavenumbers up
+// to 16 (the workloads') the rms error of a flux difference against 113-bit arithmetic, split and
+// whole, in units of 1e-17: WENO5 at 2048 cells a side 0.4 and 5.3, 512: 1.6 and 5.3, 256: 3.2 and
+// 5.3, 128: 9.2 and 5.4; WENO3 at 512: 1.9 and 5.3, 256: 6.0 and 5.5, 128: 21 and 5.7.  Whole steps
+// against 64-bit-mantissa arithmetic (relative; u1, theta, v1): 512^2 Taylor-Green 0.80e-16, 5.7e-15,
+// 1.29e-16 split, 1.09e-16, 6.0e-15, 1.41e-16 whole; 256^2 WENO3 layer 0.87e-16, 4.3e-15, 1.6e-16 and
+// 1.48e-16, 5.6e-15, 2.3e-16; 256^2 random field 1.19e-16, 3.5e-15, 2.7e-16 and 1.16e-16, 2.9e-15,
+// 2.6e-16 (a plain FP64 evaluation: 1.57e-16, 3.7e-15, 2.4e-16).
 constexpr int kSplitMinCells = 256;
 inline bool split_fluxes(const ap_dvm_params& p) {
   return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;
@@ -290,6 +291,8 @@ inline void fill_constants(const ap_dvm_params& p, InstDev& d) {
   }
   fill_coef(p, d, d.k64);
   fill_coef(p, d, d.k32);
+  for (int i = 0; i <= APD_MAXS; ++i)
+    for (int j = 0; j <= APD_MAXS; ++j) d.wp_lo[i][j] = (float)(d.k64.wp[i][j] - (double)d.k32.wp[i][j]);
   const double ra = 1.0 / (p.rho0 * p.mach);
   d.sc_u = ra;
   d.sc_th = p.eps > 0 ? ra / (2.0 * p.eps) : 0.0;
