@@ -73,6 +73,7 @@ struct ap_dvm_handle {
   int num_sms = 0;
   int tile = 0;
   bool tile_auto = true;
+  bool dependent = false;            // launch a step's kernels as programmatic dependents
   int nmax = 0, lnmax = 0, eblk = 0, eblk_cols = 0;
   // batch workspace
   BatchDev* d_batch[2] = {nullptr, nullptr};   // per step parity (double-buffered state)
@@ -442,7 +443,8 @@ ap_dvm_status launch(ap_dvm_handle* h, cudaStream_t stream, const void* fn, int 
     h->ev_kind[h->ev_used] = kind;
     CUDA_TRY(h, cudaEventRecord(h->ev[h->ev_used], stream));
   }
-  CUDA_TRY(h, cudaLaunchKernel(fn, dim3(grid), block, args, smem, stream));
+  CUDA_TRY(h, kind >= 0 && !prof && h->dependent ? launch_dependent(fn, grid, block, smem, args, stream)
+                                 : cudaLaunchKernel(fn, dim3(grid), block, args, smem, stream));
   if (prof) {
     CUDA_TRY(h, cudaEventRecord(h->ev[h->ev_used + 1], stream));
     h->ev_used += 2;
@@ -562,6 +564,7 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   h->tmpl = *tmpl;
   h->capacity = capacity;
   h->f32 = tmpl->precision != AP_DVM_FP64;
+  h->dependent = capacity == 1 && (long long)tmpl->nx * tmpl->ny <= kDependentMaxCells;
   h->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   h->nmax = std::max(fft_length(tmpl->nx), fft_length(tmpl->ny));   // longest transform of the batch
   h->lnmax = ilog2(h->nmax);

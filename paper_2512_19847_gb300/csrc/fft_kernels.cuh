@@ -313,6 +313,7 @@ __host__ __device__ constexpr int rows_min_blocks() { return sizeof(T) == 4 ? 10
 
 template <typename T>
 __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_fwd(const BatchDev* __restrict__ bp) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -372,6 +373,7 @@ __host__ __device__ constexpr int cols_threads() { return sizeof(T) == 4 ? APD_C
 template <typename T>
 __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD_COLS_THREADS32 : 2)
     k_fft_cols(const BatchDev* __restrict__ bp, int i) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -427,6 +429,7 @@ __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD
 
 template <typename T>
 __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_inv(const BatchDev* __restrict__ bp, int i) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -590,6 +593,7 @@ __device__ __forceinline__ int stockham(typename Cplx<T>::type* x, int m, int n,
 
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs(const BatchDev* __restrict__ bp) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
@@ -666,6 +670,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs
 // so the division by the symbol applies to the convolution directly.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(const BatchDev* __restrict__ bp, int i) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
@@ -750,6 +755,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
 
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs(const BatchDev* __restrict__ bp, int i) {
+  grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);

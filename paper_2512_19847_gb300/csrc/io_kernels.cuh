@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(256) k_diagnostics(InstDev I, int c4, double* 
 // step 2, with the scheme's central difference (c4: 4th order, else 2nd).
 template <typename T, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY) k_stage1(const BatchDev* __restrict__ bp, int c4) {
+  grid_dependency();
   const BatchDev& b = *bp;
   const int ntiles = b.counts[0];
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
@@ -279,6 +280,7 @@ __global__ void __launch_bounds__(TX* TY) k_stage1(const BatchDev* __restrict__ 
 // theta is theta^(s) itself, not the one summed from the populations.
 template <typename T, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY) k_finish(const BatchDev* __restrict__ bp, int f32form) {
+  grid_dependency();
   const BatchDev& b = *bp;
   const int ntiles = b.counts[0];
   const int s = b.s;

@@ -174,7 +174,7 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   StepKernels K{ks, km, g_exp, g_rhs, g_upd, g_fin, g_fft, g2, km.cols_threads, fft_smem, cols_smem, smem_upd, FFT_X_POW2 | FFT_Y_POW2,
                 g_fft};
   auto ln = [&](const void* fn, int grid, dim3 block, size_t smem, void** args, int) -> int {
-    return cudaLaunchKernel(fn, dim3(grid), block, args, smem, stream) == cudaSuccess ? 0 : (int)AP_DVM_ERR_CUDA;
+    return launch_dependent(fn, grid, block, smem, args, stream) == cudaSuccess ? 0 : (int)AP_DVM_ERR_CUDA;
   };
   for (int step = 0; step < nsteps; ++step) {
     const int st = enqueue_imex_step(*p, K, bp, 0, ln);

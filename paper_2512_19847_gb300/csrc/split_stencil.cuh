@@ -174,6 +174,7 @@ __device__ __forceinline__ F2 f2_of(double x) {
 template <int SCHEME, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_explicit_split(const BatchDev* __restrict__ bp, int j, unsigned need,
                                                                                 double weno_eps) {
+  grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
   using G = typename S::G;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
@@ -269,6 +270,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
 template <int SCHEME, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_update_split(const BatchDev* __restrict__ bp, int i, double weno_eps,
                                                                               int close_step, int form) {
+  grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
   using G = typename S::G;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;

@@ -722,6 +722,7 @@ __device__ __forceinline__ T flux_scale(T inv_h) {
 // ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_explicit(const BatchDev* __restrict__ bp, int j, unsigned need, double weno_eps) {
+  grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -849,6 +850,7 @@ constexpr int RHS_THREADS = 32 * RHS_WARPS;
 template <typename T, int SCHEME>
 __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 : APD_RHS_MINB64)
     k_rhs(const BatchDev* __restrict__ bp, int i, double theta_sign, int first_stage) {
+  grid_dependency();
   constexpr int MAXT = 1 + 3 * (APD_MAXS - 1);
   constexpr int NR = 2 * rhs_pairs(sizeof(T) == 4);   // rows per item
   constexpr unsigned FULL = 0xffffffffu;
@@ -979,6 +981,7 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
 template <typename T, int SCHEME, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_update(const BatchDev* __restrict__ bp, int i, double weno_eps,
                                                                        int close_step, int form) {
+  grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -132,6 +132,27 @@ inline int encode_stage_maps(const ap_dvm_params& p, const InstDev& d, int bw, i
   return 1;
 }
 
+// Launch of a kernel of a step as a programmatic dependent of the work before it on the stream
+// (grid_dependency in common.cuh): the launch's own latency then overlaps the end of that work.  Taken
+// by single solves of at most kDependentMaxCells cells, whose kernels run for a few microseconds
+// each: 64^2 FP64, 10 steps, 2.15 -> 1.88 ms, 384x192 LF1 1.115 -> 0.936, 509x251 FP32 0.665 ->
+// 0.565, 512^2 FP64 1.96 -> 1.88, 1000^2 FP64 3.13 -> 3.08; beyond, it costs 0.2-0.7 % (2048^2 FP64
+// 5.85 -> 5.87, 24 uneven FP32 solves 4.67 -> 4.70).
+constexpr long long kDependentMaxCells = 3LL << 19;
+inline cudaError_t launch_dependent(const void* fn, int grid, dim3 block, size_t smem, void** args, cudaStream_t stream) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // launch(fn, grid, block, smem, args, kind) -> int status (0 = success); form = the precision form
 // (AP_DVM_FP64, AP_DVM_FP32_DEV, AP_DVM_FP32_DEV_TH), passed to the finish kernel
 // fused: the last stage's update closes the step into the other state buffer
