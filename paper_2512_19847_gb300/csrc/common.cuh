@@ -10,6 +10,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include "pairs.cuh"
+
 #define APD_MAXS 4          // maximum number of IMEX stages
 #define APD_NPLANES_STATE 6
 
@@ -70,11 +72,14 @@ struct InstDev {
   double inv_den[APD_MAXS + 1]; // 1 / (tau eps^2 + dt a_ii)
   double sc_u, sc_th, sc_v, sc_q;  // population view: 1/(rho0 A), 1/(2 eps rho0 A), 1/(eps rho0 A), 1/(eps^2 rho0 A)
   double pmc[8];                   // sc_u, sc_u/2, sqrt3 sc_u/2, sc_th, -sc_v/2, sc_v/4, sqrt3 sc_v/4, sc_q/4
+  // FP32 forms: sc_u, sqrt3 sc_u/2, sc_th, -sc_v/2, sqrt3 sc_v/4, sc_q/4 as (pmp_h + pmp_l) pms_a pms_b,
+  // the pair in [1, 2) and the scales powers of two (so that no eps takes a constant out of the float range)
+  float pmp_h[6], pmp_l[6], pms_a[6], pms_b[6];
   double inv_dx, inv_dy;
   double inv_aii[APD_MAXS + 1];              // 1 / a_ii
   Coef<double> k64;             // the stage coefficients in FP64 ...
   Coef<float> k32;              // ... and rounded once to FP32
-  float wp_lo[APD_MAXS + 1][APD_MAXS + 1];   // k64.wp - k32.wp
+  Coef<float> k32lo;            // k64 - k32: with k32 the coefficients as pairs of floats
   void* X;                      // 6 planes: state at t^n (moments)
   void* Xnext;                  // 6 planes the last stage's update writes the state at t^{n+1} to (the
                                 // other buffer of a double-buffered state; null: a separate finish kernel)
@@ -251,8 +256,8 @@ __device__ __forceinline__ double rcp_newton(double d) {
 // widening, narrowing rounded to nearest with ties to even (overflow to
 // infinity, subnormal results rounded likewise); a NaN stays a NaN
 // (ap_dvm_check_conversions compares them with the instructions bit for bit).
-// The FP32 forms use them where their FP64 arithmetic meets FP32 data: the
-// moment sums of the close and the closed-form relaxations at eps <= 1e-4.
+// ap_dvm_check_conversions is their self-check; the FP32 forms' own sums and relaxations
+// work in pairs of floats (pairs.cuh) and convert nothing.
 // Every class of input: zero, subnormal, infinity, NaN as well.
 static __device__ __noinline__ double widen_f32_any(float x) {
   const unsigned u = __float_as_uint(x), s = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;

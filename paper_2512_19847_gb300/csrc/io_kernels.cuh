@@ -50,20 +50,41 @@ __device__ __forceinline__ void mom_to_pop(const R* m, R eps, R rho0, R amp, R* 
   dF[2] = a * (S3 + D3); dF[5] = a * (S3 - D3);
 }
 
+// The same in pairs of floats, each moment rounded once to FP32: the pair sums s_k, d_k of two floats
+// are exact, what is summed and scaled after them keeps 2^-47 of its operands, far below the
+// moments' own rounding.  150 FP32 instructions; in FP64 the close took 22 FP64-pipe operations per
+// cell (and 84 integer ones to convert) and held that pipe 55 % busy in the FP32 update.
+template <class Put>
+__device__ __forceinline__ void pop_to_mom_pairs(const float* dF, const InstDev& I, Put&& put) {
+  auto scaled = [&](int k, F2 r) {
+    const F2 x = f2_mul(f2(I.pmp_h[k], I.pmp_l[k]), r);
+    put(k, (x.h + x.l) * I.pms_a[k] * I.pms_b[k]);
+  };
+  auto half = [](F2 a) { return f2(0.5f * a.h, 0.5f * a.l); };
+  {
+    const F2 d1 = f2_sum(dF[0], -dF[3]), d2 = f2_sum(dF[1], -dF[4]), d3 = f2_sum(dF[2], -dF[5]);
+    scaled(1, f2_add(d2, d3));
+    const F2 dm = f2_sub(d2, d3);
+    scaled(0, f2_add(d1, half(dm)));
+    scaled(5, f2_sub(dm, d1));
+  }
+  const F2 s1 = f2_sum(dF[0], dF[3]), s2 = f2_sum(dF[1], dF[4]), s3 = f2_sum(dF[2], dF[5]);
+  scaled(4, f2_sub(s2, s3));
+  const F2 sp = f2_add(s2, s3);
+  scaled(2, f2_add(s1, sp));
+  scaled(3, f2_sub(s1, half(sp)));
+}
+
 // FP32 form: store the deviation populations dF (the persistent state) and
 // the moments the next step starts from, summed from those FP32 values in
-// FP64 with the division by rho0 A (rounded once into the FP32 planes X, or
+// pairs of floats with the division by rho0 A (rounded once into the FP32 planes X, or
 // into dst when given).
 __device__ __forceinline__ void store_f32_state(const InstDev& I, size_t o, size_t pl, const float* d,
                                                 float* dst = nullptr) {
-  double dd[6], m[6];
-  for (int k = 0; k < 6; ++k) {
-    I.dF[o + k * pl] = d[k];
-    dd[k] = widen_f32(d[k]);
-  }
-  pop_to_mom(dd, I, m);
   float* X = dst ? dst : reinterpret_cast<float*>(I.X);
-  for (int k = 0; k < 6; ++k) X[o + k * pl] = narrow_f64_rn(m[k]);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) I.dF[o + k * pl] = d[k];
+  pop_to_mom_pairs(d, I, [&](int k, float m) { X[o + k * pl] = m; });
 }
 
 // The close of a step at one cell (GSA: X^{n+1} = X^(s)), given the last stage's

@@ -21,82 +21,9 @@
 // l = 3 D_k - D_{k-1}, D_{k-1} + D_k or D_k - 3 D_{k-1} for the three candidates.
 // WENO3: the brackets are 3 w0 c_i (g+) and 3 w0 c_{i+1} (g-), taken as (1 + 3 (w0 - 1/3)) c.
 #pragma once
-#include "common.cuh"
+#include "pairs.cuh"
 
 namespace apd {
-
-// h + l, |l| small against the operands it came from (not always against h).
-struct F2 { float h, l; };
-
-__device__ __forceinline__ F2 f2(float h, float l) { F2 r; r.h = h; r.l = l; return r; }
-
-// a + k b for k = 1, -1, 2, -2: the error of the leading sum kept exactly (Knuth's two-sum).
-template <int K>
-__device__ __forceinline__ F2 f2_addk(F2 a, F2 b) {
-  const float k = float(K);
-  const float s = __fmaf_rn(k, b.h, a.h), bb = __fsub_rn(s, a.h);
-  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fmaf_rn(k, b.h, -bb));
-  return f2(s, __fadd_rn(e, __fmaf_rn(k, b.l, a.l)));
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) { return f2_addk<1>(a, b); }
-__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) { return f2_addk<-1>(a, b); }
-// The same value with |l| <= ulp(h)/2.
-__device__ __forceinline__ F2 f2_norm(F2 a) {
-  const float h = __fadd_rn(a.h, a.l);
-  return f2(h, __fsub_rn(a.l, __fsub_rn(h, a.h)));
-}
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-  const float p = __fmul_rn(a.h, b.h);
-  return f2(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
-}
-__device__ __forceinline__ F2 f2_sqr(F2 a) {
-  const float p = __fmul_rn(a.h, a.h);
-  const float t = __fmul_rn(a.h, a.l);
-  return f2(p, __fadd_rn(t, __fadd_rn(t, __fmaf_rn(a.h, a.h, -p))));
-}
-// k a for an integer k that is a float.
-__device__ __forceinline__ F2 f2_scale(F2 a, float k) {
-  const float p = __fmul_rn(k, a.h);
-  return f2(p, __fmaf_rn(k, a.l, __fmaf_rn(k, a.h, -p)));
-}
-// n / d: one approximate quotient and the remainder's, with the same reciprocal.
-__device__ __forceinline__ F2 f2_div(F2 n, F2 d) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d.h));
-  const float q = __fmul_rn(n.h, r);
-  const float rem = __fadd_rn(__fmaf_rn(-q, d.h, n.h), __fmaf_rn(-q, d.l, n.l));
-  return f2(q, __fmul_rn(rem, r));
-}
-// 2^-(exponent of x) for 0 < x finite (0, infinity and NaN give something harmless or not finite).
-__device__ __forceinline__ float inv_pow2(float x) {
-  return __uint_as_float(0x7f000000u - (__float_as_uint(x) & 0x7f800000u));
-}
-
-// An FP64 increment as a pair, by integer operations (a conversion instruction takes a
-// slot of the FP64 pipe): h the leading 24 bits truncated, l the other 29 rounded to 24.
-__device__ __forceinline__ F2 f2_from_double(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned ea = (hi >> 20) & 0x7ffu;
-  if (ea - 949u <= 1150u - 949u) {   // 2^-74 <= |d| < 2^128
-    const unsigned s = hi & 0x80000000u;
-    const float h = __uint_as_float((__funnelshift_l(lo, hi, 3) - (384u << 23)) | s);   // 896 mod 512
-    const float m = __uint2float_rn(lo & 0x1fffffffu);
-    return f2(h, __fmul_rn(m, __uint_as_float(((ea - 948u) << 23) | s)));
-  }
-  if ((hi << 1 | lo) == 0u) return f2(0.f, 0.f);
-  const float h = __double2float_rn(d);
-  return f2(h, __double2float_rn(d - (double)h));
-}
-
-// h + l in FP64 (one FP64 operation; the widenings on the integer pipe).
-__device__ __forceinline__ double f2_widen1(float x) {
-  const unsigned u = __float_as_uint(x);
-  if (((u >> 23) & 0xffu) - 1u < 254u)
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-  if ((u << 1) == 0u) return 0.0;
-  return (double)x;
-}
-__device__ __forceinline__ double f2_to_double(F2 a) { return f2_widen1(a.h) + f2_widen1(a.l); }
 
 // The bracket of one WENO5 reconstruction for each of KR neighbouring interfaces:
 // q[m] = c + 2 w0 T_{out} + w2 T_{in} from the increments D[m .. m + 3] of its stencil (upwind

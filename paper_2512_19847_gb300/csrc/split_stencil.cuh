@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     }
     if (need & NEED_V) {
       double r1, r2;   // step 1 of stage i = j + 1 at this cell
-      relax_v_cell<double, double>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
+      relax_v_cell<false, double>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
       double* vi = reinterpret_cast<double*>(I.Xs[j + 1]);
       vi[o + 3 * pl] = r1;
       vi[o + 4 * pl] = r2;
@@ -294,13 +294,13 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     const size_t pl = (size_t)nx * I.ny;
     const Coef<double>& K = I.k64;
     // weights of the dissipation partner of D_LF . B(v^(i)), the explicit-weight predictor
-    // (1/a_ii) sum_{j<i} (atilde_ij - a_ij) u^(j), as pairs (k32.wp and its remainder)
+    // (1/a_ii) sum_{j<i} (atilde_ij - a_ij) u^(j), as pairs (k32 and k32lo)
     F2 wt[APD_MAXS - 1];
     int nw = 0;
 #pragma unroll
     for (int jj = 1; jj < APD_MAXS; ++jj)
       if (jj < i && has(mwp, jj)) {
-        const F2 a = f2(I.k32.wp[i][jj], I.wp_lo[i][jj]);
+        const F2 a = f2(I.k32.wp[i][jj], I.k32lo.wp[i][jj]);
         if (nw == 0) wt[0] = a; else if (nw == 1) wt[1] = a; else wt[2] = a;
         ++nw;
       }

@@ -639,64 +639,63 @@ __device__ __forceinline__ T* aligned_smem(unsigned char* raw) {
   return reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
 }
 
-// Widening of a transport value to the relaxation's arithmetic type R.  In the FP32
-// forms the closed-form relaxations run in FP64 (eps <= 1e-4): their FP32 inputs
-// are widened, and their results narrowed, with integer operations (widen_f32,
-// narrow_f64_rn: the instructions' results for every class of value) rather than by
-// the conversion instructions, which issue on the FP64 pipe, the pipe those kernels'
-// FP64 arithmetic already loads (APD_INT_WIDEN = 0 restores the instructions).
-#ifndef APD_INT_WIDEN
-#define APD_INT_WIDEN 1
-#endif
-template <typename R, typename T>
-__device__ __forceinline__ R widen(T x) {
-  if constexpr (APD_INT_WIDEN && std::is_same<R, double>::value && std::is_same<T, float>::value) return widen_f32(x);
-  else return R(x);
-}
-// and the relaxation's result back to the transport type, rounded to nearest
-template <typename T, typename R>
-__device__ __forceinline__ T narrow(R x) {
-  if constexpr (APD_INT_WIDEN && std::is_same<R, double>::value && std::is_same<T, float>::value) return narrow_f64_rn(x);
-  else return T(x);
-}
+// A closed form's sum of coefficient times value: in T, or (PAIRS, T = float) with the coefficient
+// as the pair c + lo and the sum in a pair, rounded once by value().
+template <bool PAIRS, typename T>
+struct RelaxSum {
+  T s;
+  __device__ __forceinline__ void start(T c, float, T x) { s = c * x; }
+  __device__ __forceinline__ void add(T c, float, T x) { s = s + c * x; }
+  __device__ __forceinline__ T value() const { return s; }
+};
+template <>
+struct RelaxSum<true, float> {
+  F2 s;
+  __device__ __forceinline__ void start(float c, float lo, float x) { s = f2_mulf(f2(c, lo), x); }
+  __device__ __forceinline__ void add(float c, float lo, float x) { s = f2_add(s, f2_mulf(f2(c, lo), x)); }
+  __device__ __forceinline__ float value() const { return s.h + s.l; }
+};
 
 // ---------------------------------------------------------------------------
 // Closed-form v^(i) at one cell (step 1):
 //   v^(i) = (tau eps^2 v^n - dt sum_j atilde_ij E^(j) - dt sum_j a_ij v^(j)) / (tau eps^2 + dt a_ii),
-// evaluated in R with the division folded into the coefficients.  E^(jcur)
-// and v^(jcur) may be given in registers (the values the kernel has just
-// computed or loaded).
-template <typename R, typename T>
+// with the division folded into the coefficients.  E^(jcur) and v^(jcur) may be given in
+// registers (the values the kernel has just computed or loaded).  PAIRS (FP32 form at
+// eps <= 1e-4): coefficients and sums in pairs of floats, rounded once.
+template <bool PAIRS, typename T>
 __device__ __forceinline__ void relax_v_cell(const BatchDev& b, const InstDev& I, int i, size_t o, size_t pl, int jcur,
                                              T ecur1, T ecur2, T vcur1, T vcur2, T& r1, T& r2) {
   const T* Xn = reinterpret_cast<const T*>(I.X);
-  const Coef<R>& K = coef<R>(I);
-  R a1 = K.r_n[i] * widen<R>(Xn[o + 3 * pl]), a2 = K.r_n[i] * widen<R>(Xn[o + 4 * pl]);
+  const Coef<T>& K = coef<T>(I);
+  RelaxSum<PAIRS, T> a1, a2;
+  a1.start(K.r_n[i], I.k32lo.r_n[i], Xn[o + 3 * pl]);
+  a2.start(K.r_n[i], I.k32lo.r_n[i], Xn[o + 4 * pl]);
   for (int jj = 1; jj < i; ++jj) {
     if (has(b.m_ex[i], jj)) {
       T e1, e2;
       if (jj == jcur) { e1 = ecur1; e2 = ecur2; }
       else { const T* e = reinterpret_cast<const T*>(I.E[jj]); e1 = e[o]; e2 = e[o + pl]; }
-      a1 = a1 + K.rv_e[i][jj] * widen<R>(e1);
-      a2 = a2 + K.rv_e[i][jj] * widen<R>(e2);
+      a1.add(K.rv_e[i][jj], I.k32lo.rv_e[i][jj], e1);
+      a2.add(K.rv_e[i][jj], I.k32lo.rv_e[i][jj], e2);
     }
     if (has(b.m_im[i], jj)) {
       T x1, x2;
       if (jj == jcur) { x1 = vcur1; x2 = vcur2; }
       else { const T* v = reinterpret_cast<const T*>(I.Xs[jj]); x1 = v[o + 3 * pl]; x2 = v[o + 4 * pl]; }
-      a1 = a1 + K.rv_v[i][jj] * widen<R>(x1);
-      a2 = a2 + K.rv_v[i][jj] * widen<R>(x2);
+      a1.add(K.rv_v[i][jj], I.k32lo.rv_v[i][jj], x1);
+      a2.add(K.rv_v[i][jj], I.k32lo.rv_v[i][jj], x2);
     }
   }
-  r1 = narrow<T>(a1);
-  r2 = narrow<T>(a2);
+  r1 = a1.value();
+  r2 = a2.value();
 }
 
 // Resident blocks per SM the explicit and update kernels are compiled for: threads worth
 // three 256-thread blocks in FP64 (the register budget that removes spills: 128 at 512
 // threads), APD_STENCIL_THREADS32 threads in the FP32 forms: 896 (seven 128-thread blocks of
-// the 16x8 tile at 72 registers, no spills) measured 8-9 % faster than 768 (six blocks, 80
-// registers); 1024 (64 registers) spills.
+// the 16x8 tile at 72 registers).  2048^2, ms per step, explicit + update: 0.358 + 0.457 at 896,
+// 0.378 + 0.440 at 768, 0.399 + 0.462 at 640; 509x251, whose 1024 tiles take one wave of 1064
+// blocks at 896 and two of 912 at 768, 0.565 against 0.588 ms for 4 steps.
 #ifndef APD_STENCIL_THREADS32
 #define APD_STENCIL_THREADS32 896
 #endif
@@ -810,8 +809,8 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_expl
     if (need & NEED_V) {
       // step 1 of stage i = j + 1 at this cell
       T r1, r2;
-      if (I.relax64) relax_v_cell<double, T>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
-      else relax_v_cell<T, T>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
+      if (sizeof(T) == 4 && I.relax64) relax_v_cell<sizeof(T) == 4, T>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
+      else relax_v_cell<false, T>(b, I, j + 1, o, pl, j, e1, e2, sv1[c], sv2[c], r1, r2);
       T* vi = reinterpret_cast<T*>(I.Xs[j + 1]);
       vi[o + 3 * pl] = r1;
       vi[o + 4 * pl] = r2;
@@ -909,6 +908,7 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
     const int y0 = NR * g, nrows = min(NR, ny - y0);
     const int seg0 = sg * RHS_SEG;                       // first column of this warp's segment
     double tsum = 0.0;
+    F2 tpair = f2(0.f, 0.f);   // FP32: the item's rows of this lane, exact to 2^-48
     if (task < rhs_tasks(nx, ny, sizeof(T) == 4)) {   // warp-uniform: past the instance's last task
       const int xs = seg0 + lane - 2;                 // this lane's column, unwrapped
       int x = xs % nx;
@@ -959,11 +959,13 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
           const size_t o = (size_t)(y0 + h) * nx + x;
           if (keep_db) DBi[o] = Bh;
           Rp[o] = R[h] - cdb * Bh;
-          tsum += double(thn[h]);
+          if constexpr (sizeof(T) == 4) tpair = f2_add(tpair, f2(float(thn[h]), 0.f));
+          else tsum += thn[h];
         }
       }
     }
     if (first_stage) {
+      if constexpr (sizeof(T) == 4) tsum = f2_to_double(tpair);
       for (int o = 16; o > 0; o >>= 1) tsum += __shfl_down_sync(FULL, tsum, o);
       if (lane == 0) red[warp] = tsum;
       __syncthreads();
@@ -1076,27 +1078,18 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_upda
       reinterpret_cast<T*>(I.Dv[i])[o] = dvi;   // D0 . v^(i) for the q steps of later stages
     }
     // step 4
+    auto step4 = [&](auto sum) {
+      sum.start(K.r_n[i], I.k32lo.r_n[i], Xn[o + 5 * pl]);
+      for (int jj = 1; jj <= i; ++jj) {
+        if (!has(mim, jj)) continue;
+        sum.add(K.rq_d[i][jj], I.k32lo.rq_d[i][jj], (jj == i) ? dvi : reinterpret_cast<const T*>(I.Dv[jj])[o]);
+        if (jj < i) sum.add(K.rv_v[i][jj], I.k32lo.rv_v[i][jj], reinterpret_cast<const T*>(I.Xs[jj])[o + 5 * pl]);
+      }
+      return sum.value();
+    };
     T qi;
-    if (I.relax64) {
-      const Coef<double>& K64 = I.k64;
-      double aq = K64.r_n[i] * widen<double>(Xn[o + 5 * pl]);
-      for (int jj = 1; jj <= i; ++jj) {
-        if (!has(mim, jj)) continue;
-        const double dv = widen<double>((jj == i) ? dvi : reinterpret_cast<const T*>(I.Dv[jj])[o]);
-        aq = aq + K64.rq_d[i][jj] * dv;
-        if (jj < i) aq = aq + K64.rv_v[i][jj] * widen<double>(reinterpret_cast<const T*>(I.Xs[jj])[o + 5 * pl]);
-      }
-      qi = narrow<T>(aq);
-    } else {
-      T aq = K.r_n[i] * Xn[o + 5 * pl];
-      for (int jj = 1; jj <= i; ++jj) {
-        if (!has(mim, jj)) continue;
-        const T dv = (jj == i) ? dvi : reinterpret_cast<const T*>(I.Dv[jj])[o];
-        aq = aq + K.rq_d[i][jj] * dv;
-        if (jj < i) aq = aq + K.rv_v[i][jj] * reinterpret_cast<const T*>(I.Xs[jj])[o + 5 * pl];
-      }
-      qi = aq;
-    }
+    if (sizeof(T) == 4 && I.relax64) qi = step4(RelaxSum<sizeof(T) == 4, T>());
+    else qi = step4(RelaxSum<false, T>());
     if (!close_step) {
       out[o + 5 * pl] = qi;
       return;

@@ -6,6 +6,8 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "../../include/ap_dvm.h"
@@ -312,8 +314,12 @@ inline void fill_constants(const ap_dvm_params& p, InstDev& d) {
   }
   fill_coef(p, d, d.k64);
   fill_coef(p, d, d.k32);
-  for (int i = 0; i <= APD_MAXS; ++i)
-    for (int j = 0; j <= APD_MAXS; ++j) d.wp_lo[i][j] = (float)(d.k64.wp[i][j] - (double)d.k32.wp[i][j]);
+  // every member of Coef is a T
+  const double* c64 = reinterpret_cast<const double*>(&d.k64);
+  const float* c32 = reinterpret_cast<const float*>(&d.k32);
+  float* lo = reinterpret_cast<float*>(&d.k32lo);
+  static_assert(sizeof(Coef<double>) == 2 * sizeof(Coef<float>), "Coef holds values of its type only");
+  for (size_t k = 0; k < sizeof(Coef<float>) / sizeof(float); ++k) lo[k] = (float)(c64[k] - (double)c32[k]);
   const double ra = 1.0 / (p.rho0 * p.mach);
   d.sc_u = ra;
   d.sc_th = p.eps > 0 ? ra / (2.0 * p.eps) : 0.0;
@@ -328,6 +334,17 @@ inline void fill_constants(const ap_dvm_params& p, InstDev& d) {
   d.pmc[5] = 0.25 * d.sc_v;
   d.pmc[6] = 0.25 * sq3 * d.sc_v;
   d.pmc[7] = 0.25 * d.sc_q;
+  const double pm[6] = {d.pmc[0], d.pmc[2], d.pmc[3], d.pmc[4], d.pmc[6], d.pmc[7]};
+  for (int k = 0; k < 6; ++k) {
+    int e = 0;
+    const double m = 2.0 * std::frexp(pm[k], &e);   // pm = m 2^(e - 1), |m| in [1, 2) (or 0)
+    d.pmp_h[k] = (float)m;
+    d.pmp_l[k] = (float)(m - (double)d.pmp_h[k]);
+    // two powers of two in the float range; a constant beyond it overflows as its narrowed result would
+    const int ea = std::max(-120, std::min(120, e - 1)), eb = std::max(-120, std::min(120, e - 1 - ea));
+    d.pms_a[k] = (float)std::ldexp(1.0, ea);
+    d.pms_b[k] = (float)std::ldexp(1.0, eb);
+  }
 }
 
 }  // namespace apd
