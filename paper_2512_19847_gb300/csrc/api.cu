@@ -81,6 +81,7 @@ struct ap_dvm_handle {
   int* d_tile_start = nullptr;
   int* d_row_start = nullptr;
   int* d_rhs_start = nullptr;
+  int* d_march_start[2] = {nullptr, nullptr};   // explicit, update
   int* d_col_start = nullptr;
   int* d_counts = nullptr;
   double2* d_tw = nullptr;
@@ -93,13 +94,13 @@ struct ap_dvm_handle {
   int n_active = 0;
   // upload staging (kept alive across async copies)
   std::vector<InstDev> up_inst[2];
-  std::vector<int> up_tiles, up_rows, up_cols, up_rhs;
-  int up_counts[6] = {0, 0, 0, 0, 0, 0};
+  std::vector<int> up_tiles, up_rows, up_cols, up_rhs, up_march[2];
+  int up_counts[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   // kernels
   StencilSet ks{};
   MiscSet km{};
   int grid_explicit = 0, grid_rhs = 0, grid_update = 0, grid_fft = 0, grid_cols = 0, grid_finish = 0, grid_rows = 0;
-  int grid_explicit_split = 0, grid_update_split = 0;
+  int grid_explicit_split = 0, grid_update_split = 0, grid_explicit_march = 0, grid_update_march = 0;
   unsigned fft_kinds = 0;   // FftKinds of the attached solves (the launches a step enqueues)
   unsigned stencil_kinds = 0;   // ... and their StencilKinds
   size_t smem_update = 0, smem_update_split = 0;
@@ -231,7 +232,9 @@ size_t batch_bytes(int capacity, int nmax) {
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
-  take(sizeof(int) * 6);
+  take(sizeof(int) * (capacity + 1));
+  take(sizeof(int) * (capacity + 1));
+  take(sizeof(int) * 8);
   take(sizeof(double2) * (nmax / 2));
   take(sizeof(float2) * (nmax / 2));
   take(sizeof(unsigned) * 4);
@@ -255,8 +258,8 @@ unsigned fft_kinds_of(const ap_dvm_handle* h) {
 unsigned stencil_kinds_of(const ap_dvm_handle* h) {
   unsigned k = 0;
   for (const Slot& s : h->slots)
-    if (s.attached) k |= split_fluxes(s.p) ? STENCIL_SPLIT : STENCIL_WHOLE;
-  return k ? k : (split_fluxes(h->tmpl) ? STENCIL_SPLIT : STENCIL_WHOLE);
+    if (s.attached) k |= stencil_kind(s.p);
+  return k ? k : stencil_kind(h->tmpl);
 }
 
 int auto_tile(const ap_dvm_handle* h) {
@@ -308,6 +311,18 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
     if ((st = occupancy_grid(h, h->ks.k_explicit_split, thr, h->ks.smem_explicit_split, &h->grid_explicit_split))) return st;
     if ((st = occupancy_grid(h, h->ks.k_update_split, thr, h->smem_update_split, &h->grid_update_split))) return st;
   }
+  if (h->ks.march_threads) {
+    h->grid_explicit_march = h->grid_update_march = 1 << 30;
+    int g = 0;
+    for (int n = 0; n < 3; ++n) {
+      for (int m = 0; m < 4; ++m) {
+        if ((st = occupancy_grid(h, h->ks.k_explicit_march[n][m], h->ks.march_threads, 0, &g))) return st;
+        h->grid_explicit_march = std::min(h->grid_explicit_march, g);
+      }
+      if ((st = occupancy_grid(h, h->ks.k_update_march[n], h->ks.march_threads, 0, &g))) return st;
+      h->grid_update_march = std::min(h->grid_update_march, g);
+    }
+  }
   if ((st = occupancy_grid(h, h->km.k_finish, thr, 0, &h->grid_finish))) return st;
   h->grid_fft = 1 << 30;
   for (const void* fn : {h->km.k_rows_fwd_bs, h->km.k_cols_bs, h->km.k_rows_inv_bs}) {
@@ -325,6 +340,23 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
   h->kernels_ready = true;
   h->graph_valid[0] = h->graph_valid[1] = false;
   return AP_DVM_OK;
+}
+
+// Rows per task of the marching kernels: the fewest rounds of tasks over the resident warps, a
+// task's start-up (the window's rows and curvature terms) counted as 5 rows.
+int march_rows(const std::vector<Slot*>& order, int grid) {
+  static constexpr int kRows[] = {8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 72, 80, 96, 112, 128};
+  const long long warps = 4LL * std::max(1, grid);
+  int best = 0;
+  long long best_cost = 0;
+  for (int rows : kRows) {
+    long long tasks = 0;
+    for (const Slot* s : order)
+      if (marching(s->p)) tasks += march_tasks(s->p.nx, s->p.ny, rows);
+    const long long cost = (tasks + warps - 1) / warps * (rows + 5);
+    if (!best || cost < best_cost) { best = rows; best_cost = cost; }
+  }
+  return best;
 }
 
 // Rebuild and upload the compacted instance table and work decomposition.
@@ -364,12 +396,16 @@ ap_dvm_status flush(ap_dvm_handle* h) {
   }
   const int row_share = (int)(row_elems / std::min(h->grid_rows, h->grid_fft));
   const int col_share = (int)(col_elems / std::min(h->grid_cols, h->grid_fft));
-  // the instances with split fluxes come last: a tile range for each kind of stencil kernel
+  // the instances that the tile kernels do not take with whole fluxes come last: a tile range for each kind
   std::vector<Slot*> order;
-  for (int split = 0; split < 2; ++split)
+  for (int other = 0; other < 2; ++other)
     for (Slot& s : h->slots)
-      if (s.attached && !s.paused && split_fluxes(s.p) == (split != 0)) order.push_back(&s);
+      if (s.attached && !s.paused && (stencil_kind(s.p) != STENCIL_WHOLE) == (other != 0)) order.push_back(&s);
   h->up_counts[5] = 0;
+  for (int m = 0; m < 2; ++m) {
+    h->up_march[m].assign(1, 0);
+    h->up_counts[6 + m] = march_rows(order, m ? h->grid_update_march : h->grid_explicit_march);
+  }
   for (Slot* sp : order) {
     Slot& s = *sp;
     if (s.p.nx < TX || s.p.ny < TY) return fail(h, AP_DVM_ERR_ARG, "grid %dx%d smaller than the tile %dx%d", s.p.nx, s.p.ny, TX, TY);
@@ -398,7 +434,9 @@ ap_dvm_status flush(ap_dvm_handle* h) {
       h->up_inst[par].push_back(v);
     }
     h->up_tiles.push_back(h->up_tiles.back() + d.tiles_x * d.tiles_y);
-    if (!split_fluxes(s.p)) h->up_counts[5] = h->up_tiles.back();
+    if (stencil_kind(s.p) == STENCIL_WHOLE) h->up_counts[5] = h->up_tiles.back();
+    for (int m = 0; m < 2; ++m)
+      h->up_march[m].push_back(h->up_march[m].back() + (marching(s.p) ? march_tasks(s.p.nx, s.p.ny, h->up_counts[6 + m]) : 0));
     h->up_rows.push_back(h->up_rows.back() + (pairs + d.row_pairs - 1) / d.row_pairs);
     h->up_rhs.push_back(h->up_rhs.back() + rhs_items(s.p.nx, s.p.ny, h->f32));
     h->up_cols.push_back(h->up_cols.back() + (s.p.nx / 2 + 1 + d.col_group - 1) / d.col_group);
@@ -417,9 +455,11 @@ ap_dvm_status flush(ap_dvm_handle* h) {
     CUDA_TRY(h, cudaMemcpyAsync(h->d_tile_start, h->up_tiles.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(h->d_row_start, h->up_rows.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(h->d_rhs_start, h->up_rhs.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
+    for (int m = 0; m < 2; ++m)
+      CUDA_TRY(h, cudaMemcpyAsync(h->d_march_start[m], h->up_march[m].data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(h->d_col_start, h->up_cols.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream));
   }
-  CUDA_TRY(h, cudaMemcpyAsync(h->d_counts, h->up_counts, sizeof(int) * 6, cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(h->d_counts, h->up_counts, sizeof(int) * 8, cudaMemcpyHostToDevice, h->stream));
   h->dirty = false;
   return AP_DVM_OK;
 }
@@ -470,7 +510,8 @@ ap_dvm_status profile_collect(ap_dvm_handle* h) {
 ap_dvm_status enqueue_step(ap_dvm_handle* h, cudaStream_t stream, int parity) {
   StepKernels K{h->ks,       h->km,         h->grid_explicit, h->grid_rhs,   h->grid_update, h->grid_finish,
                 h->grid_fft, h->grid_cols, h->km.cols_threads, fft_smem(h), cols_smem(h), h->smem_update, h->fft_kinds,
-                h->grid_rows, h->stencil_kinds, h->grid_explicit_split, h->grid_update_split, h->smem_update_split};
+                h->grid_rows, h->stencil_kinds, h->grid_explicit_split, h->grid_update_split, h->smem_update_split,
+                h->grid_explicit_march, h->grid_update_march};
   auto ln = [&](const void* fn, int grid, dim3 block, size_t smem, void** args, int kind) -> int {
     return (int)launch(h, stream, fn, grid, block, smem, args, kind);
   };
@@ -588,7 +629,8 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   h->d_row_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   h->d_col_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   h->d_rhs_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
-  h->d_counts = reinterpret_cast<int*>(take(sizeof(int) * 6));
+  for (int*& m : h->d_march_start) m = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
+  h->d_counts = reinterpret_cast<int*>(take(sizeof(int) * 8));
   h->d_tw = reinterpret_cast<double2*>(take(sizeof(double2) * (h->nmax / 2)));
   h->d_tw32 = reinterpret_cast<float2*>(take(sizeof(float2) * (h->nmax / 2)));
   h->d_err = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 4));
@@ -609,6 +651,7 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   hb.row_start = h->d_row_start;
   hb.col_start = h->d_col_start;
   hb.rhs_start = h->d_rhs_start;
+  for (int m = 0; m < 2; ++m) hb.march_start[m] = h->d_march_start[m];
   hb.counts = h->d_counts;
   hb.tw = h->d_tw;
   hb.tw32 = h->d_tw32;
@@ -625,7 +668,7 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   for (int par = 0; par < 2; ++par)
     CUDA_TRY(h, cudaMemcpyAsync(h->d_batch[par], &h->hb[par], sizeof(BatchDev), cudaMemcpyHostToDevice, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned) * 4, h->stream));
-  CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, sizeof(int) * 6, h->stream));
+  CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, sizeof(int) * 8, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->slots.resize(capacity);
   h->dirty = true;
@@ -935,7 +978,7 @@ int ap_dvm_launches_per_step(const ap_dvm_handle* h) {
   const ap_dvm_params& t = h->tmpl;
   const int f = fft_launches(fft_kinds_of(h));   // transform launches per implicit stage
   const unsigned sk = stencil_kinds_of(h);
-  const int n = ((sk & STENCIL_WHOLE) ? 1 : 0) + ((sk & STENCIL_SPLIT) ? 1 : 0);   // explicit, and update, launches per stage
+  const int n = ((sk & STENCIL_WHOLE) ? 1 : 0) + ((sk & STENCIL_SPLIT) ? 1 : 0) + ((sk & STENCIL_MARCH) ? 1 : 0);   // explicit, and update, launches per stage
   // the last stage's update closes the step (no finish kernel)
   return t.A_im[0] != 0.0 ? 1 + (1 + n + f) + (1 + 2 * n + f) * (t.s - 1) : (1 + 2 * n + f) * (t.s - 1);
 }

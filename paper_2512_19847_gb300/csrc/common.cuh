@@ -123,8 +123,10 @@ struct BatchDev {
   int* row_start;        // [n+1]
   int* col_start;        // [n+1]
   int* rhs_start;        // [n+1]
+  int* march_start[2];   // [n+1] (FP32: tasks of the marching explicit and update kernels; null without them)
   int* counts;           // [0] tiles, [1] row items, [2] column items, [3] instances, [4] k_rhs items,
-                         // [5] tiles of the instances whose fluxes are not split (they come first)
+                         // [5] tiles of the instances taken by the tile kernels with whole fluxes (they come
+                         // first), [6], [7] rows per task of the marching explicit and update kernels
   double2* tw;           // twiddles exp(-2 pi i k / nmax), k < nmax/2
   float2* tw32;          // the same, rounded once to FP32 (FP32 form)
   int lnmax;             // log2 of the largest transform length
@@ -162,6 +164,9 @@ __host__ __device__ constexpr int rhs_items(int nx, int ny, bool f32) {
 __device__ __forceinline__ void grid_dependency() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+
+// Columns one warp of the marching stencil kernels (march_kernels.cuh) puts out.
+constexpr int MARCH_OUT = 26;
 
 // Instance owning work item `item`: the last k with start[k] <= item.
 __device__ __forceinline__ int find_inst(const int* __restrict__ start, int n, int item) {

@@ -45,7 +45,7 @@ Layout layout(const ap_dvm_params& p, int nmax) {
   L.row_start = take(2 * sizeof(int));
   L.col_start = take(2 * sizeof(int));
   L.rhs_start = take(2 * sizeof(int));
-  L.counts = take(6 * sizeof(int));
+  L.counts = take(8 * sizeof(int));
   L.tw = take(sizeof(double2) * (nmax / 2));
   L.err = take(4 * sizeof(unsigned));
   L.ws = take(carve_instance(p, nullptr, nullptr));
@@ -142,7 +142,7 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   const int ncols = (p->nx / 2 + 1 + I.col_group - 1) / I.col_group;
   const int nrhs = rhs_items(p->nx, p->ny, false);
   const int ts[2] = {0, ntiles}, rs[2] = {0, nrows}, cs[2] = {0, ncols}, hs[2] = {0, nrhs};
-  const int counts[6] = {ntiles, nrows, ncols, 1, nrhs, ntiles};
+  const int counts[8] = {ntiles, nrows, ncols, 1, nrhs, ntiles, 0, 0};
   double2 tw[64];                                   // nmax/2 <= 64 for grids of at most 128 cells a side
   double lx[65], ly[128];
   const long double pi = 3.141592653589793238462643383279502884L;

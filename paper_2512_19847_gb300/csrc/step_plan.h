@@ -19,9 +19,10 @@ namespace apd {
 enum KernelKind { KK_EXPLICIT, KK_RHS, KK_ROWS_FWD, KK_COLS, KK_ROWS_INV, KK_UPDATE, KK_FINISH, KK_STAGE1 };
 
 // Kinds of Helmholtz transform work a batch holds (bits of StepKernels::fft_kinds).
-// Kinds of stencil work a batch holds (bits of StepKernels::stencil_kinds): instances whose fluxes are
-// evaluated whole, and those that take the split fluxes (split_flux.cuh).
-enum StencilKinds { STENCIL_WHOLE = 1, STENCIL_SPLIT = 2 };
+// Kinds of stencil work a batch holds (bits of StepKernels::stencil_kinds): instances taken by the tile
+// kernels with whole fluxes, those with split fluxes (FP64, split_flux.cuh), and those taken by the
+// marching kernels (FP32, march_kernels.cuh).
+enum StencilKinds { STENCIL_WHOLE = 1, STENCIL_SPLIT = 2, STENCIL_MARCH = 4 };
 
 enum FftKinds { FFT_X_POW2 = 1, FFT_X_BS = 2, FFT_Y_POW2 = 4, FFT_Y_BS = 8 };
 
@@ -42,6 +43,7 @@ struct StepKernels {
   unsigned stencil_kinds = STENCIL_WHOLE;   // StencilKinds present among the attached solves
   int g_explicit_split = 0, g_update_split = 0;
   size_t smem_update_split = 0;
+  int g_explicit_march = 0, g_update_march = 0;
 };
 
 // Planes k_update stages at its largest stage: theta, v1, v2 and u1, u2 of every
@@ -93,6 +95,22 @@ constexpr int kSplitMinCells = 256;
 inline bool split_fluxes(const ap_dvm_params& p) {
   return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;
 }
+
+// Whether a solve is taken by the marching kernels: FP32 WENO5, enough cells for their warps (each holds
+// a row of 26 columns) to fill the chip, and a width that does not leave over a quarter of their
+// columns beyond the grid.  Explicit + update, us per step, marching against tiles: 256^2 57 and 48,
+// 320^2 62 and 54, 384^2 61 and 65, 512^2 69 and 81, 1024^2 148 and 227, 2048^2 489 and 817,
+// 4096^2 1787 and 3165.  A property of the solve alone, so that a batch does not change its result.
+constexpr long long kMarchMinCells = 384LL * 384;
+inline bool marching(const ap_dvm_params& p) {
+  const int covered = (p.nx + MARCH_OUT - 1) / MARCH_OUT * MARCH_OUT;
+  return p.precision != AP_DVM_FP64 && p.space_scheme == AP_DVM_WENO5_C4 && (long long)p.nx * p.ny >= kMarchMinCells &&
+         4LL * covered <= 5LL * p.nx;
+}
+inline unsigned stencil_kind(const ap_dvm_params& p) {
+  return split_fluxes(p) ? STENCIL_SPLIT : (marching(p) ? STENCIL_MARCH : STENCIL_WHOLE);
+}
+inline int march_tasks(int nx, int ny, int rows) { return ((nx + MARCH_OUT - 1) / MARCH_OUT) * ((ny + rows - 1) / rows); }
 
 inline size_t update_smem(const StencilSet& ks, const ap_dvm_params& t) {
   return ks.update_fixed + (size_t)ks.nbuf * update_planes_max(t) * ks.plane_bytes;
@@ -190,6 +208,12 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
       if ((K.stencil_kinds & STENCIL_SPLIT) &&
           (st = launch(K.ks.k_explicit_split, K.g_explicit_split, blk, K.ks.smem_explicit_split, a, KK_EXPLICIT)))
         return st;
+      if (K.stencil_kinds & STENCIL_MARCH) {
+        int terms = 1;   // of v^(i): v^n and the stages before j
+        for (int k = 1; k < j; ++k) terms += (AEX(i, k) != 0.0) + (AIM(i, k) != 0.0);
+        const void* fn = K.ks.k_explicit_march[std::min(terms, 3) - 1][(need & 1u) | ((need & 16u) >> 3)];
+        if ((st = launch(fn, K.g_explicit_march, dim3(K.ks.march_threads), 0, a, KK_EXPLICIT))) return st;
+      }
     }
     double sign = -1.0;   // theta-history term with a minus sign (the stage equations of Sec. 3.1)
     int first = (i == (type_a ? 1 : 2)) ? 1 : 0;           // the first right-hand side also sums theta^n
@@ -216,6 +240,15 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
       if ((K.stencil_kinds & STENCIL_SPLIT) &&
           (st = launch(K.ks.k_update_split, K.g_update_split, blk, K.smem_update_split, a, KK_UPDATE)))
         return st;
+      if (K.stencil_kinds & STENCIL_MARCH) {
+        int nw = 0, nt = 0;
+        for (int k = 1; k < i; ++k) {
+          nw += AEX(i, k) - AIM(i, k) != 0.0;
+          nt += AIM(i, k) != 0.0;
+        }
+        const void* fn = K.ks.k_update_march[nw == 1 && nt == 0 ? 0 : (nw == 2 && nt == 1 ? 1 : 2)];
+        if ((st = launch(fn, K.g_update_march, dim3(K.ks.march_threads), 0, a, KK_UPDATE))) return st;
+      }
     }
   }
   if (fused) return 0;
