@@ -300,7 +300,7 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
   if (h->tile_auto) h->tile = auto_tile(h);
   h->ks = stencil_for(h->f32, h->tmpl.space_scheme, h->tile);
   h->km = misc_set(h->f32, h->tile);
-  const int thr = h->ks.tx * h->ks.ty;
+  const int cells = h->ks.tx * h->ks.ty, thr = cells * h->ks.tz;
   ap_dvm_status st;
   if ((st = occupancy_grid(h, h->ks.k_explicit, thr, h->ks.smem_explicit, &h->grid_explicit))) return st;
   if ((st = occupancy_grid(h, h->ks.k_rhs, h->ks.rhs_threads, 0, &h->grid_rhs))) return st;
@@ -323,7 +323,7 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
       h->grid_update_march = std::min(h->grid_update_march, g);
     }
   }
-  if ((st = occupancy_grid(h, h->km.k_finish, thr, 0, &h->grid_finish))) return st;
+  if ((st = occupancy_grid(h, h->km.k_finish, cells, 0, &h->grid_finish))) return st;
   h->grid_fft = 1 << 30;
   for (const void* fn : {h->km.k_rows_fwd_bs, h->km.k_cols_bs, h->km.k_rows_inv_bs}) {
     int g = 0;

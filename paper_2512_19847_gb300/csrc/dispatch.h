@@ -55,7 +55,7 @@ struct StencilSet {
   int rhs_threads;                     // k_rhs: threads per block (no dynamic shared memory)
   size_t plane_bytes, update_fixed;   // k_update: update_fixed + nbuf * (planes staged) * plane_bytes
   int nbuf;                            // staged plane buffers of k_update (1 or 2)
-  int tx, ty;
+  int tx, ty, tz;                      // tile, and threads per cell (explicit and update kernels)
   int bw, bh;                          // staged box: (tx + 8) x (ty + 2 * halo)
 };
 

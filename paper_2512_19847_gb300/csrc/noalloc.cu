@@ -102,13 +102,13 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   MiscSet km = misc_set(0, tile);
   const int eblk = fft_eblk(nmax), eblk_cols = fft_eblk_cols(nmax, false);
   const size_t fft_smem = fft_block_bytes(eblk, false), cols_smem = fft_block_bytes(eblk_cols, false);
-  const int thr = ks.tx * ks.ty;
+  const int cells = ks.tx * ks.ty, thr = cells * ks.tz;
   int g_exp = 0, g_rhs = 0, g_upd = 0, g_fin = 0, g1 = 0, g2 = 0, g3 = 0;
   NA_TRY(grid_of(ks.k_explicit, thr, ks.smem_explicit, sms, &g_exp));
   NA_TRY(grid_of(ks.k_rhs, ks.rhs_threads, 0, sms, &g_rhs));
   const size_t smem_upd = update_smem(ks, *p);
   NA_TRY(grid_of(ks.k_update, thr, smem_upd, sms, &g_upd));
-  NA_TRY(grid_of(km.k_finish, thr, 0, sms, &g_fin));
+  NA_TRY(grid_of(km.k_finish, cells, 0, sms, &g_fin));
   NA_TRY(grid_of(km.k_rows_fwd, km.rows_threads, fft_smem, sms, &g1));
   NA_TRY(grid_of(km.k_cols, km.cols_threads, cols_smem, sms, &g2));
   NA_TRY(grid_of(km.k_rows_inv, km.rows_threads, fft_smem, sms, &g3));

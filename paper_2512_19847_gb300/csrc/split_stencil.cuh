@@ -57,7 +57,7 @@ template <int SCHEME, int TX, int TY, int NF>
 __device__ __forceinline__ void split_increments(const double* const* fx, const double* const* fy, F2* ix, F2* iy, int tid) {
   using S = SplitGeo<SCHEME, TX, TY>;
   using G = typename S::G;
-  for (int k = tid; k < S::LIX + S::LIY; k += TX * TY) {
+  for (int k = tid; k < S::LIX + S::LIY; k += G::NT) {
     if (k < S::LIX) {
       const int line = k / S::LX, o = (G::H + line) * G::BW + G::XO + (k - line * S::LX);
 #pragma unroll
@@ -78,7 +78,7 @@ __device__ __forceinline__ void split_increments_update(const double* s, int nw,
   using S = SplitGeo<SCHEME, TX, TY>;
   using G = typename S::G;
   constexpr int PL = G::PL;
-  for (int k = tid; k < S::LIX + S::LIY; k += TX * TY) {
+  for (int k = tid; k < S::LIX + S::LIY; k += G::NT) {
     const bool ax = k < S::LIX;
     const int r = ax ? k : k - S::LIX, line = ax ? r / S::LX : r % TX, pt = ax ? r - line * S::LX : r / TX;
     const int o = ax ? (G::H + line) * G::BW + G::XO + pt : pt * G::BW + G::XO + G::H + line, st = ax ? 1 : G::BW;
@@ -138,7 +138,7 @@ __device__ __forceinline__ void split_interfaces(const F2* ix, const F2* iy, F2*
   constexpr int KR = APD_SPLIT_RUN;
   constexpr int RX = (TX + 1 + KR - 1) / KR, RY = (TY + 1 + KR - 1) / KR;
   constexpr int IX = NP * TY * RX, IY = NP * TX * RY;
-  for (int k = tid; k < IX + IY; k += TX * TY) {
+  for (int k = tid; k < IX + IY; k += G::NT) {
     const bool ax = k < IX;
     const int kk = ax ? k : k - IX, nl = ax ? TY : TX, per = ax ? TY * RX : TX * RY;
     const int p = kk / per, r = kk - p * per, run = r / nl, line = r - run * nl;
@@ -172,7 +172,7 @@ __device__ __forceinline__ F2 f2_of(double x) {
 // ---------------------------------------------------------------------------
 // k_explicit (stencil_kernels.cuh) with split fluxes.
 template <int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_explicit_split(const BatchDev* __restrict__ bp, int j, unsigned need,
+__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_explicit_split(const BatchDev* __restrict__ bp, int j, unsigned need,
                                                                                 double weno_eps) {
   grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
   F2* nxs = iy + 5 * S::LIY;   // [3][NX]: (q;v1), (-v1;u1), (v2;u2)
   F2* nys = nxs + 3 * NX;      // [3][NY]: (q;v2), (v2;u1), (v1;u2)
   const BatchDev& b = *bp;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const F2 w = f2_of((SCHEME == WENO5_C4 ? 16.0 : 4.0) * weno_eps);
   const bool needB = (need & NEED_DLFB) != 0, needE = (need & NEED_E) != 0;
   PlaneList pr;
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
       split_interfaces<SCHEME, TX, TY, 2, 0>(ix, iy, nxs + NX, nys + NY, w, tid);
     }
     __syncthreads();
-    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    if (threadIdx.z > 0 || t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // no cell, or beyond the grid (ragged edge tile)
     const Coef<double>& K = I.k64;
     const double cx = K.cdx, cy = K.cdy;                // 1/(12 h)
     const int c = G::C00 + ty * BW + tx;
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
 
 // k_update (stencil_kernels.cuh) with split fluxes.
 template <int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k_update_split(const BatchDev* __restrict__ bp, int i, double weno_eps,
+__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_update_split(const BatchDev* __restrict__ bp, int i, double weno_eps,
                                                                               int close_step, int form) {
   grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
   F2* iy = ix + 4 * S::LIX;
   F2* nxs = iy + 4 * S::LIY;   // [2][NX]: (-v1;p1), (v2;p2)
   F2* nys = nxs + 2 * NX;      // [2][NY]: (v2;p1), (v1;p2)
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const F2 w = f2_of((SCHEME == WENO5_C4 ? 16.0 : 4.0) * weno_eps);
   const unsigned mwp = b.m_wp[i], mim = b.m_im[i];
   tile_loop<double, G, TX, TY, S::NBUF, true>(b, pr, stage, bars, tid, [&](const InstDev& I, const TileRef& t, double* s) {
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(TX* TY, split_min_blocks<SCHEME, TX * TY>()) k
     __syncthreads();
     split_interfaces<SCHEME, TX, TY, 2, 0>(ix, iy, nxs, nys, w, tid);
     __syncthreads();
-    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    if (threadIdx.z > 0 || t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // no cell, or beyond the grid (ragged edge tile)
     const double cx = K.cdx, cy = K.cdy;
     const int c = G::C00 + ty * BW + tx;
     const int fa = ty * (TX + 1) + tx, fb = ty * TX + tx;

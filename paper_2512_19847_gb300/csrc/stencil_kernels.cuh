@@ -46,6 +46,13 @@ struct Geo {
   static constexpr unsigned PLANE_BYTES = (unsigned)(BW * BH * sizeof(T));
   static constexpr int C00 = H * BW + 4;                // interior cell (0, 0)
   static constexpr int NX = TY * (TX + 1), NY = (TY + 1) * TX;
+  // threads per block: one per cell, four on the smallest tile of the FP64 WENO kernels (taken by grids
+  // of few tiles, whose passes are chains of FP64 operations in too few warps), the cells being
+  // those of threadIdx.z = 0.  64^2, us per launch with the launch gap: explicit 27.2 -> 18.6, update
+  // 28.5 -> 19.4; the LF1 kernels have one short pass and lose by it (384x192, 12 launches each: 0.24 +
+  // 0.22 -> 0.28 + 0.29 ms).
+  static constexpr int TZ = (sizeof(T) == 8 && TX * TY <= 64 && SCHEME != LF1_C2) ? 4 : 1;
+  static constexpr int NT = TX * TY * TZ;
   static constexpr int LS = (TY * W > HH * TX) ? TY * W : HH * TX;
   // FP32 WENO5 computes its fluxes in register runs: no split scratch, no partner planes
   static constexpr bool RUNS = SCHEME == WENO5_C4 && sizeof(T) == 4;
@@ -179,7 +186,7 @@ __device__ __forceinline__ void stage_begin(const BatchDev& b, int it, const Pla
 template <typename T, class G, int TX, int TY, int NB = 2, bool SPLIT = false, class Body>
 __device__ __forceinline__ void tile_loop(const BatchDev& b, const PlaneList& pr, T* stage0, uint64_t* bars, int tid,
                                           Body&& body) {
-  constexpr int NT = TX * TY;
+  constexpr int NT = G::NT;
   const int ntiles = b.counts[SPLIT ? 0 : 5];
   const int bstride = pr.n * G::PL;       // buffer 1 starts at stage0 + bstride
   if (tid == 0) {
@@ -320,7 +327,7 @@ __device__ __forceinline__ void axis_fluxes(const T* const* g, const T* const* U
   constexpr int NI = AX == 0 ? TX + 1 : TY + 1;   // interfaces per line
   constexpr int LS = NL * LL;
   constexpr int PS = AX == 0 ? 1 : NL;            // split stride between points of a line
-  constexpr int NT = TX * TY;
+  constexpr int NT = G::NT;
   // index r of the split scratch -> (line, point), and of the interfaces -> (line, m)
   auto pt_line = [&](int r, int& line, int& pt) {
     if (AX == 0) { line = r / LL; pt = r - line * LL; }
@@ -521,7 +528,7 @@ template <typename T, int TX, int TY, int NP, unsigned NEGX, unsigned NEGY>
 __device__ __forceinline__ void w5_fluxes_xy(const T* const* gx, const T* const* ux, const T* const* gy,
                                              const T* const* uy, T* split, T* fx, T* fy, T ew, int tid) {
   using G = Geo<T, WENO5_C4, TX, TY>;
-  constexpr int H = G::H, W = G::W, HH = G::HH, SW = G::BW, XO = G::XO, NT = TX * TY;
+  constexpr int H = G::H, W = G::W, HH = G::HH, SW = G::BW, XO = G::XO, NT = G::NT;
   constexpr int LSX = G::LSX, LSY = G::LSY, NIX = TX + 1, NIY = TY + 1;
   T* spx = split;                    // [4 NP][LSX]: (row, point)
   T* spy = split + 4 * NP * LSX;     // [4 NP][LSY]: (point, column)
@@ -720,7 +727,7 @@ __device__ __forceinline__ T flux_scale(T inv_h) {
 
 // ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_explicit(const BatchDev* __restrict__ bp, int j, unsigned need, double weno_eps) {
+__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_explicit(const BatchDev* __restrict__ bp, int j, unsigned need, double weno_eps) {
   grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
@@ -731,7 +738,7 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_expl
   T* fx = split + 3 * G::SPLIT_PER_PAIR;  // [3][NX]: (q;v1), (-v1;u1), (v2;u2)
   T* fy = fx + 3 * NX;                    // [3][NY]: (q;v2), (v2;u1), (v1;u2)
   const BatchDev& b = *bp;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const T ew = T(weno_eps);
   const bool needB = (need & NEED_DLFB) != 0, needE = (need & NEED_E) != 0;
   PlaneList pr;
@@ -766,7 +773,7 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_expl
       both_axes<T, SCHEME, TX, TY, 2, 1u, 0u>(gx, ux, gy, uy, split, fx + NX, fy + NY, ew, tid);
     }
     __syncthreads();
-    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    if (threadIdx.z > 0 || t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // no cell, or beyond the grid (ragged edge tile)
     const Coef<T>& K = coef<T>(I);
     const T idx = K.inv_dx, idy = K.inv_dy;
     const T fidx = flux_scale<T, SCHEME>(idx), fidy = flux_scale<T, SCHEME>(idy);
@@ -981,7 +988,7 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
 
 // ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_update(const BatchDev* __restrict__ bp, int i, double weno_eps,
+__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_update(const BatchDev* __restrict__ bp, int i, double weno_eps,
                                                                        int close_step, int form) {
   grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
@@ -997,7 +1004,7 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_upda
   T* split = G::RUNS ? sp1 : sp2 + PL;     // 2 pairs
   T* fx = split + 2 * G::SPLIT_U_PER_PAIR; // [2][NX]: (-v1;p1), (v2;p2)
   T* fy = fx + 2 * NX;                     // [2][NY]: (v2;p1), (v1;p2)
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const T ew = T(weno_eps);
   const unsigned mwp = b.m_wp[i], mim = b.m_im[i];
   tile_loop<T, G, TX, TY, G::NBUF_U>(b, pr, stage, bars, tid, [&](const InstDev& I, const TileRef& t, T* s) {
@@ -1026,7 +1033,7 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_upda
       const PlaneSum uy[2] = {P1, P2};
       w5_runs_both_axes<TX, TY, 2, 1u, 0u>(gx, ux, gy, uy, fx, fy, ew, tid);
     } else {
-      for (int e = tid; e < G::BW * G::BH; e += TX * TY) {
+      for (int e = tid; e < G::BW * G::BH; e += G::NT) {
         T p1 = T(0), p2 = T(0);
         int k = 3;
         for (int jj = 1; jj < i; ++jj) {
@@ -1047,7 +1054,7 @@ __global__ void __launch_bounds__(TX* TY, stencil_min_blocks<T>(TX * TY)) k_upda
       both_axes<T, SCHEME, TX, TY, 2, 1u, 0u, G::MERGED>(gx, ux, gy, uy, split, fx, fy, ew, tid);
     }
     __syncthreads();
-    if (t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // beyond the grid (ragged edge tile)
+    if (threadIdx.z > 0 || t.x0 + tx >= nx || t.y0 + ty >= I.ny) return;   // no cell, or beyond the grid (ragged edge tile)
     const T idx = K.inv_dx, idy = K.inv_dy;
     const T fidx = flux_scale<T, SCHEME>(idx), fidy = flux_scale<T, SCHEME>(idy);
     const int c = G::C00 + ty * BW + tx;

@@ -182,7 +182,7 @@ template <class Launch>
 int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp, int form, Launch&& launch,
                       bool fused = false) {
   const int s = t.s;
-  const dim3 blk(K.ks.tx, K.ks.ty);
+  const dim3 blk(K.ks.tx, K.ks.ty, K.ks.tz), cells(K.ks.tx, K.ks.ty);
   double weno_eps = t.weno_eps;
   int st;
   auto AEX = [&](int i, int j) { return t.A_ex[(i - 1) * AP_DVM_MAX_STAGES + (j - 1)]; };
@@ -192,7 +192,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
   if (type_a) {
     int c4 = t.space_scheme != AP_DVM_LF1_C2;
     void* a[] = {&bp, &c4};
-    if ((st = launch(K.km.k_stage1, K.g_finish, blk, 0, a, KK_STAGE1))) return st;
+    if ((st = launch(K.km.k_stage1, K.g_finish, cells, 0, a, KK_STAGE1))) return st;
   }
   for (int i = type_a ? 1 : 2; i <= s; ++i) {
     int j = i - 1;
@@ -253,7 +253,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
   }
   if (fused) return 0;
   void* a[] = {&bp, &form};
-  return launch(K.km.k_finish, K.g_finish, blk, 0, a, KK_FINISH);
+  return launch(K.km.k_finish, K.g_finish, cells, 0, a, KK_FINISH);
 }
 
 // Fill the derived per-instance constants of a descriptor from its parameters.
