@@ -235,8 +235,8 @@ size_t batch_bytes(int capacity, int nmax) {
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * 8);
-  take(sizeof(double2) * (nmax / 2));
-  take(sizeof(float2) * (nmax / 2));
+  take(sizeof(double2) * nmax);
+  take(sizeof(float2) * nmax);
   take(sizeof(unsigned) * 4);
   return align_up(off, 256);
 }
@@ -631,20 +631,15 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   h->d_rhs_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   for (int*& m : h->d_march_start) m = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
   h->d_counts = reinterpret_cast<int*>(take(sizeof(int) * 8));
-  h->d_tw = reinterpret_cast<double2*>(take(sizeof(double2) * (h->nmax / 2)));
-  h->d_tw32 = reinterpret_cast<float2*>(take(sizeof(float2) * (h->nmax / 2)));
+  h->d_tw = reinterpret_cast<double2*>(take(sizeof(double2) * h->nmax));
+  h->d_tw32 = reinterpret_cast<float2*>(take(sizeof(float2) * h->nmax));
   h->d_err = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 4));
-  // twiddles exp(-2 pi i k / nmax) from long double
-  std::vector<double2> tw(h->nmax / 2);
-  std::vector<float2> tw32(h->nmax / 2);
-  const long double pi = 3.141592653589793238462643383279502884L;
-  for (int k = 0; k < h->nmax / 2; ++k) {
-    const long double a = -2.0L * pi * (long double)k / (long double)h->nmax;
-    tw[k].x = (double)std::cos(a);
-    tw[k].y = (double)std::sin(a);
-    tw32[k].x = (float)std::cos(a);
-    tw32[k].y = (float)std::sin(a);
-  }
+  std::vector<double2> tw(h->nmax);
+  std::vector<float2> tw32(h->nmax);
+  twiddle_table(h->nmax, [&](int k, long double c, long double sn) {
+    tw[k] = make_double2((double)c, (double)sn);
+    tw32[k] = make_float2((float)c, (float)sn);
+  }, [&](int k, int j) { tw[k] = tw[j]; tw32[k] = tw32[j]; });
   BatchDev& hb = h->hb[0];
   hb.inst = h->d_inst[0];
   hb.tile_start = h->d_tile_start;

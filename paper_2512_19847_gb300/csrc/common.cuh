@@ -100,6 +100,7 @@ struct InstDev {
   float* lamx32;                // FP32 form: the same tables rounded once (null in the FP64 form)
   float* lamy32;
   float hscale32;               // FP32 form: 1/(nx ny) rounded once
+  double hscale;                // 1/(nx ny)
   double* th_part;              // partial sums of theta^n, one per k_rhs item (rhs_items)
   float* dF;                    // FP32 form: deviation populations (6 planes)
   unsigned mr_plan[2];          // axes whose n is not a power of two but factors into 2, 3, 5, 7 (x, y):
@@ -127,7 +128,7 @@ struct BatchDev {
   int* counts;           // [0] tiles, [1] row items, [2] column items, [3] instances, [4] k_rhs items,
                          // [5] tiles of the instances taken by the tile kernels with whole fluxes (they come
                          // first), [6], [7] rows per task of the marching explicit and update kernels
-  double2* tw;           // twiddles exp(-2 pi i k / nmax), k < nmax/2
+  double2* tw;           // twiddles exp(-2 pi i k / nmax), k < nmax/2, then as many in bit-reversed order (fft_rev)
   float2* tw32;          // the same, rounded once to FP32 (FP32 form)
   int lnmax;             // log2 of the largest transform length
   int s;                 // stages

@@ -9,9 +9,8 @@
 //                    symbol (mode k = 0 set to mean(theta^n): every other term of R has zero mean),
 //                    inverse DFT along y, scaled by 1/(nx ny);
 //   k_fft_rows_inv : inverse real row DFTs into theta^(i).
-// Power-of-two lengths: radix-2^3 passes in shared memory, decimation in time
-// from bit-reversed order for the forward transforms, decimation in frequency
-// (natural in, bit-reversed out) for the inverse ones, so no permutation pass
+// Power-of-two lengths: radix-2^3 passes in shared memory, from bit-reversed to natural
+// order (fft_dit) or from natural to bit-reversed (fft_rev), so no permutation pass
 // is needed.  Other lengths that factor into 2, 3, 5 and 7: a self-sorting
 // mixed-radix transform (below).  Any other length n is transformed by
 // Bluestein's chirp-z identity (L. I. Bluestein, 1970): with
@@ -63,19 +62,41 @@ __device__ __forceinline__ C mul_j(C a, bool inv) {
   return r;
 }
 
-// Multiplication by the eighth roots W_8^1 = (1 - i)/sqrt2 and W_8^3 = W_8^1 W_8^2
-// (conjugated when inv), the constant twiddles inside a radix-2^3 step.
+// Butterfly with the twiddle on the second input: (a, b) -> (a + w b, a - w b) in six FMAs, the
+// difference as 2 a - (a + w b).  Multiplying first and adding after takes eight operations.
 template <typename C>
-__device__ __forceinline__ C mul_w8(C a, bool inv) {
+__device__ __forceinline__ void bfly(C& a, C& b, C w) {
   using T = decltype(a.x);
-  const T r = T(0.70710678118654752440);
-  C b;
-  if (inv) { b.x = r * (a.x - a.y); b.y = r * (a.x + a.y); }
-  else { b.x = r * (a.x + a.y); b.y = r * (a.y - a.x); }
-  return b;
+  const T sx = fma(-w.y, b.y, fma(w.x, b.x, a.x)), sy = fma(w.y, b.x, fma(w.x, b.y, a.y));
+  b.x = fma(T(2), a.x, -sx);
+  b.y = fma(T(2), a.y, -sy);
+  a.x = sx;
+  a.y = sy;
 }
 template <typename C>
-__device__ __forceinline__ C mul_w83(C a, bool inv) { return mul_j(mul_w8(a, inv), inv); }
+__device__ __forceinline__ void bfly1(C& a, C& b) {   // w = 1
+  const C s = cadd(a, b), d = csub(a, b);
+  a = s;
+  b = d;
+}
+template <typename C>
+__device__ __forceinline__ void bflyj(C& a, C& b, bool inv) {   // w = W_4
+  b = mul_j(b, inv);
+  bfly1(a, b);
+}
+// Twiddle of a table, conjugated for the inverse transform, and times W_4 (likewise).
+template <typename C>
+__device__ __forceinline__ C tw_of(C w, bool inv) { if (inv) w.y = -w.y; return w; }
+template <typename C>
+__device__ __forceinline__ C tw_j(C w, bool inv) { return mul_j(w, inv); }
+template <typename C>
+__device__ __forceinline__ C tw_8(bool inv) {
+  using T = decltype(C().x);
+  C w;
+  w.x = T(0.70710678118654752440);
+  w.y = inv ? T(0.70710678118654752440) : T(-0.70710678118654752440);
+  return w;
+}
 
 // Shared-memory index with padding: one spare element after every 2^PS
 // elements (PS = 31: none), so that the strided accesses of the butterfly
@@ -93,10 +114,15 @@ __host__ __device__ constexpr int padded_len(int n, int ps) { return ps >= 31 ? 
 // x[pidx<PS>(i)]), input in bit-reversed order, output natural.  Twiddle
 // W_m^p = tw[p * nmax/m].  Stages are taken three at a time (radix-2^3): each
 // thread loads eight elements p0 + k h (k = 0..7, h = 2^(s-1)), applies stage s
-// (half h, twiddle W_{2h}^pos), stage s+1 (half 2h, W_{4h}^pos and W_{4h}^pos W_4)
-// and stage s+2 (half 4h, W_{8h}^pos W_8^k) in registers, and stores them: one
-// table twiddle per stage, the rest constant roots.  One or two stages left over
-// take a radix-2^2 or radix-2 step; the first step has only constant twiddles.
+// (half h, twiddle W_{2h}^pos), stage s+1 (half 2h, W_{4h}^pos times 1 and W_4)
+// and stage s+2 (half 4h, W_{8h}^pos times 1, W_8, W_4, W_4 W_8) in registers, and stores
+// them: every butterfly takes its whole twiddle (bfly), read from the table or that times W_4,
+// which exchanges its parts.  One or two stages left over take a radix-2^2 or radix-2 step; the
+// first step has only constant twiddles.
+// FP64 transforms are bound by the FP64 pipe: 72 operations per eight elements and step against
+// 104 with twiddles and constant roots multiplied separately.  2048^2, FP64, ms per step: columns
+// 0.944 -> 0.652, rows 0.417 -> 0.312 (forward) and 0.406 -> 0.290 (inverse); FP32, which is not: 0.098
+// -> 0.095, 0.050 -> 0.052 and 0.049 -> 0.047.
 template <typename T, int PS = 31>
 __device__ __forceinline__ void fft_dit(typename Cplx<T>::type* x, int ln, int ntr,
                                         const typename Cplx<T>::type* __restrict__ tw, int lnmax,
@@ -112,145 +138,109 @@ __device__ __forceinline__ void fft_dit(typename Cplx<T>::type* x, int ln, int n
       const int q = t * n + grp * 8 * h + pos;
       C v0 = x[pidx<PS>(q)], v1 = x[pidx<PS>(q + h)], v2 = x[pidx<PS>(q + 2 * h)], v3 = x[pidx<PS>(q + 3 * h)];
       C v4 = x[pidx<PS>(q + 4 * h)], v5 = x[pidx<PS>(q + 5 * h)], v6 = x[pidx<PS>(q + 6 * h)], v7 = x[pidx<PS>(q + 7 * h)];
-      if (s > 1) {   // stage s: W_{2h}^pos on the odd elements
-        const C w1 = tw[pos << (lnmax - s)];
-        v1 = cmul_tw(w1, v1, inv); v3 = cmul_tw(w1, v3, inv); v5 = cmul_tw(w1, v5, inv); v7 = cmul_tw(w1, v7, inv);
+      if (s == 1) {
+        bfly1(v0, v1); bfly1(v2, v3); bfly1(v4, v5); bfly1(v6, v7);
+        bfly1(v0, v2); bflyj(v1, v3, inv); bfly1(v4, v6); bflyj(v5, v7, inv);
+        const C w8 = tw_8<C>(inv);
+        bfly1(v0, v4); bfly(v1, v5, w8); bflyj(v2, v6, inv); bfly(v3, v7, tw_j(w8, inv));
+      } else {
+        const C w1 = tw_of(tw[pos << (lnmax - s)], inv), w2 = tw_of(tw[pos << (lnmax - s - 1)], inv);
+        const C w3 = tw_of(tw[pos << (lnmax - s - 2)], inv), w4 = tw_of(tw[(pos + h) << (lnmax - s - 2)], inv);
+        bfly(v0, v1, w1); bfly(v2, v3, w1); bfly(v4, v5, w1); bfly(v6, v7, w1);
+        const C w2j = tw_j(w2, inv);
+        bfly(v0, v2, w2); bfly(v1, v3, w2j); bfly(v4, v6, w2); bfly(v5, v7, w2j);
+        bfly(v0, v4, w3); bfly(v1, v5, w4); bfly(v2, v6, tw_j(w3, inv)); bfly(v3, v7, tw_j(w4, inv));
       }
-      C a0 = cadd(v0, v1), a1 = csub(v0, v1), a2 = cadd(v2, v3), a3 = csub(v2, v3);
-      C a4 = cadd(v4, v5), a5 = csub(v4, v5), a6 = cadd(v6, v7), a7 = csub(v6, v7);
-      if (s > 1) {   // stage s+1: W_{4h}^pos (and W_4 below)
-        const C w2 = tw[pos << (lnmax - s - 1)];
-        a2 = cmul_tw(w2, a2, inv); a3 = cmul_tw(w2, a3, inv); a6 = cmul_tw(w2, a6, inv); a7 = cmul_tw(w2, a7, inv);
-      }
-      a3 = mul_j(a3, inv);
-      a7 = mul_j(a7, inv);
-      C b0 = cadd(a0, a2), b2 = csub(a0, a2), b1 = cadd(a1, a3), b3 = csub(a1, a3);
-      C b4 = cadd(a4, a6), b6 = csub(a4, a6), b5 = cadd(a5, a7), b7 = csub(a5, a7);
-      if (s > 1) {   // stage s+2: W_{8h}^pos (and W_8^k below)
-        const C w3 = tw[pos << (lnmax - s - 2)];
-        b4 = cmul_tw(w3, b4, inv); b5 = cmul_tw(w3, b5, inv); b6 = cmul_tw(w3, b6, inv); b7 = cmul_tw(w3, b7, inv);
-      }
-      b5 = mul_w8(b5, inv);
-      b6 = mul_j(b6, inv);
-      b7 = mul_w83(b7, inv);
-      x[pidx<PS>(q)] = cadd(b0, b4); x[pidx<PS>(q + 4 * h)] = csub(b0, b4);
-      x[pidx<PS>(q + h)] = cadd(b1, b5); x[pidx<PS>(q + 5 * h)] = csub(b1, b5);
-      x[pidx<PS>(q + 2 * h)] = cadd(b2, b6); x[pidx<PS>(q + 6 * h)] = csub(b2, b6);
-      x[pidx<PS>(q + 3 * h)] = cadd(b3, b7); x[pidx<PS>(q + 7 * h)] = csub(b3, b7);
+      x[pidx<PS>(q)] = v0; x[pidx<PS>(q + h)] = v1; x[pidx<PS>(q + 2 * h)] = v2; x[pidx<PS>(q + 3 * h)] = v3;
+      x[pidx<PS>(q + 4 * h)] = v4; x[pidx<PS>(q + 5 * h)] = v5; x[pidx<PS>(q + 6 * h)] = v6; x[pidx<PS>(q + 7 * h)] = v7;
     }
     __syncthreads();
   }
   if (s + 1 == ln) {   // two stages left: radix-2^2
     const int h = 1 << (s - 1), nq = n >> 2, nb = ntr * nq;
     for (int k = tid; k < nb; k += nthr) {
-      const int t = k >> (ln - 2), bi = k & (nq - 1);
-      const int pos = bi & (h - 1), grp = bi >> (s - 1);
-      const int p0 = t * n + grp * 4 * h + pos;
+      const int t = k >> (ln - 2), pos = k & (nq - 1);   // one group: h = n / 4
+      const int p0 = t * n + pos;
       C x0 = x[pidx<PS>(p0)], x1 = x[pidx<PS>(p0 + h)], x2 = x[pidx<PS>(p0 + 2 * h)], x3 = x[pidx<PS>(p0 + 3 * h)];
-      if (s > 1) {
-        const C w1 = tw[pos << (lnmax - s)];
-        x1 = cmul_tw(w1, x1, inv);
-        x3 = cmul_tw(w1, x3, inv);
-      }
-      const C a0 = cadd(x0, x1), a1 = csub(x0, x1);
-      C a2 = cadd(x2, x3), a3 = csub(x2, x3);
-      if (s > 1) {
-        const C w2 = tw[pos << (lnmax - s - 1)];
-        a2 = cmul_tw(w2, a2, inv);
-        a3 = cmul_tw(w2, a3, inv);
-      }
-      a3 = mul_j(a3, inv);
-      x[pidx<PS>(p0)] = cadd(a0, a2);
-      x[pidx<PS>(p0 + 2 * h)] = csub(a0, a2);
-      x[pidx<PS>(p0 + h)] = cadd(a1, a3);
-      x[pidx<PS>(p0 + 3 * h)] = csub(a1, a3);
+      const C w1 = tw_of(tw[pos << (lnmax - s)], inv), w2 = tw_of(tw[pos << (lnmax - s - 1)], inv);
+      bfly(x0, x1, w1); bfly(x2, x3, w1);
+      bfly(x0, x2, w2); bfly(x1, x3, tw_j(w2, inv));
+      x[pidx<PS>(p0)] = x0; x[pidx<PS>(p0 + h)] = x1; x[pidx<PS>(p0 + 2 * h)] = x2; x[pidx<PS>(p0 + 3 * h)] = x3;
     }
     __syncthreads();
   } else if (s == ln) {   // one stage left: radix-2
     const int half = 1 << (s - 1), sh = lnmax - s, nb = ntr * (n >> 1);
     for (int k = tid; k < nb; k += nthr) {
-      const int t = k >> (ln - 1), bi = k & ((n >> 1) - 1);
-      const int pos = bi & (half - 1), grp = bi >> (s - 1);
-      const int i0 = t * n + grp * 2 * half + pos, i1 = i0 + half;
-      const C a = x[pidx<PS>(i0)], tb = cmul_tw(tw[pos << sh], x[pidx<PS>(i1)], inv);
-      x[pidx<PS>(i0)] = cadd(a, tb);
-      x[pidx<PS>(i1)] = csub(a, tb);
+      const int t = k >> (ln - 1), pos = k & ((n >> 1) - 1);
+      const int i0 = t * n + pos, i1 = i0 + half;
+      C a = x[pidx<PS>(i0)], c = x[pidx<PS>(i1)];
+      bfly(a, c, tw_of(tw[pos << sh], inv));
+      x[pidx<PS>(i0)] = a;
+      x[pidx<PS>(i1)] = c;
     }
     __syncthreads();
   }
 }
 
-// Natural-order input, bit-reversed output (decimation in frequency), three
-// stages at a time as in fft_dit, mirrored: stage s (half 4h, W_{8h}^pos W_8^k
-// on the differences), stage s-1 (half 2h, W_{4h}^pos and W_{4h}^pos W_4),
-// stage s-2 (half h, W_{2h}^pos), h = 2^(s-3); leftovers as radix-2^2 or radix-2.
+// Natural-order input, bit-reversed output, with the same butterflies: splitting the polynomial
+// sum_i x_i z^i modulo z^n - 1 into its remainders modulo z^t - c and z^t + c, level by level, block j
+// of a level of m blocks takes c = W_{2m}^{rev(j)} (rev: j's log2 m bits reversed) for all its pairs.
+// rev(j) / (2m) is half the fraction with j's bits after the point in reverse, for every m, so
+// one table in that order, tr[j] = exp(-pi i 0.b0 b1 b2 ...), serves all levels: block j of three
+// successive levels takes tr[j], tr[2j] (times 1 and W_4) and tr[4j], tr[4j + 2] = W_8 tr[4j].
+// tr follows the nmax / 2 values of tw.
 template <typename T, int PS = 31>
-__device__ __forceinline__ void fft_dif(typename Cplx<T>::type* x, int ln, int ntr,
+__device__ __forceinline__ void fft_rev(typename Cplx<T>::type* x, int ln, int ntr,
                                         const typename Cplx<T>::type* __restrict__ tw, int lnmax,
                                         bool inv, int tid, int nthr) {
   using C = typename Cplx<T>::type;
+  const C* __restrict__ tr = tw + (1 << (lnmax - 1));
   const int n = 1 << ln;
-  int s = ln;
+  int s = ln;   // levels of size 2^s and below are left
   for (; s >= 3; s -= 3) {
     const int h = 1 << (s - 3), ne = n >> 3, nb = ntr * ne;
     for (int k = tid; k < nb; k += nthr) {
       const int t = k >> (ln - 3), bi = k & (ne - 1);
-      const int pos = bi & (h - 1), grp = bi >> (s - 3);
-      const int q = t * n + grp * 8 * h + pos;
-      const C v0 = x[pidx<PS>(q)], v1 = x[pidx<PS>(q + h)], v2 = x[pidx<PS>(q + 2 * h)], v3 = x[pidx<PS>(q + 3 * h)];
-      const C v4 = x[pidx<PS>(q + 4 * h)], v5 = x[pidx<PS>(q + 5 * h)], v6 = x[pidx<PS>(q + 6 * h)], v7 = x[pidx<PS>(q + 7 * h)];
-      // stage s: pairs (k, k+4), differences times W_{8h}^pos W_8^k
-      C a0 = cadd(v0, v4), a1 = cadd(v1, v5), a2 = cadd(v2, v6), a3 = cadd(v3, v7);
-      C a4 = csub(v0, v4), a5 = csub(v1, v5), a6 = csub(v2, v6), a7 = csub(v3, v7);
-      a5 = mul_w8(a5, inv);
-      a6 = mul_j(a6, inv);
-      a7 = mul_w83(a7, inv);
-      if (s > 3) {
-        const C w3 = tw[pos << (lnmax - s)];
-        a4 = cmul_tw(w3, a4, inv); a5 = cmul_tw(w3, a5, inv); a6 = cmul_tw(w3, a6, inv); a7 = cmul_tw(w3, a7, inv);
+      const int pos = bi & (h - 1), j = bi >> (s - 3);
+      const int q = t * n + j * 8 * h + pos;
+      C v0 = x[pidx<PS>(q)], v1 = x[pidx<PS>(q + h)], v2 = x[pidx<PS>(q + 2 * h)], v3 = x[pidx<PS>(q + 3 * h)];
+      C v4 = x[pidx<PS>(q + 4 * h)], v5 = x[pidx<PS>(q + 5 * h)], v6 = x[pidx<PS>(q + 6 * h)], v7 = x[pidx<PS>(q + 7 * h)];
+      if (s == ln) {   // one block: constant twiddles
+        bfly1(v0, v4); bfly1(v1, v5); bfly1(v2, v6); bfly1(v3, v7);
+        bfly1(v0, v2); bfly1(v1, v3); bflyj(v4, v6, inv); bflyj(v5, v7, inv);
+        const C w8 = tw_8<C>(inv);
+        bfly1(v0, v1); bflyj(v2, v3, inv); bfly(v4, v5, w8); bfly(v6, v7, tw_j(w8, inv));
+      } else {
+        const C w1 = tw_of(tr[j], inv), w2 = tw_of(tr[2 * j], inv), w3 = tw_of(tr[4 * j], inv), w4 = tw_of(tr[4 * j + 2], inv);
+        bfly(v0, v4, w1); bfly(v1, v5, w1); bfly(v2, v6, w1); bfly(v3, v7, w1);
+        const C w2j = tw_j(w2, inv);
+        bfly(v0, v2, w2); bfly(v1, v3, w2); bfly(v4, v6, w2j); bfly(v5, v7, w2j);
+        bfly(v0, v1, w3); bfly(v2, v3, tw_j(w3, inv)); bfly(v4, v5, w4); bfly(v6, v7, tw_j(w4, inv));
       }
-      // stage s-1: pairs (k, k+2), differences times W_{4h}^pos (W_4 for the odd ones)
-      C b0 = cadd(a0, a2), b1 = cadd(a1, a3), b2 = csub(a0, a2), b3 = csub(a1, a3);
-      C b4 = cadd(a4, a6), b5 = cadd(a5, a7), b6 = csub(a4, a6), b7 = csub(a5, a7);
-      b3 = mul_j(b3, inv);
-      b7 = mul_j(b7, inv);
-      if (s > 3) {
-        const C w2 = tw[pos << (lnmax - s + 1)];
-        b2 = cmul_tw(w2, b2, inv); b3 = cmul_tw(w2, b3, inv); b6 = cmul_tw(w2, b6, inv); b7 = cmul_tw(w2, b7, inv);
-      }
-      // stage s-2: pairs (k, k+1), differences times W_{2h}^pos
-      C c1 = csub(b0, b1), c3 = csub(b2, b3), c5 = csub(b4, b5), c7 = csub(b6, b7);
-      if (s > 3) {
-        const C w1 = tw[pos << (lnmax - s + 2)];
-        c1 = cmul_tw(w1, c1, inv); c3 = cmul_tw(w1, c3, inv); c5 = cmul_tw(w1, c5, inv); c7 = cmul_tw(w1, c7, inv);
-      }
-      x[pidx<PS>(q)] = cadd(b0, b1); x[pidx<PS>(q + h)] = c1;
-      x[pidx<PS>(q + 2 * h)] = cadd(b2, b3); x[pidx<PS>(q + 3 * h)] = c3;
-      x[pidx<PS>(q + 4 * h)] = cadd(b4, b5); x[pidx<PS>(q + 5 * h)] = c5;
-      x[pidx<PS>(q + 6 * h)] = cadd(b6, b7); x[pidx<PS>(q + 7 * h)] = c7;
+      x[pidx<PS>(q)] = v0; x[pidx<PS>(q + h)] = v1; x[pidx<PS>(q + 2 * h)] = v2; x[pidx<PS>(q + 3 * h)] = v3;
+      x[pidx<PS>(q + 4 * h)] = v4; x[pidx<PS>(q + 5 * h)] = v5; x[pidx<PS>(q + 6 * h)] = v6; x[pidx<PS>(q + 7 * h)] = v7;
     }
     __syncthreads();
   }
-  if (s == 2) {   // two stages left: radix-2^2 with trivial table twiddles (h = 1)
+  if (s == 2) {   // two levels left: radix-2^2
     const int nq = n >> 2, nb = ntr * nq;
     for (int k = tid; k < nb; k += nthr) {
-      const int p0 = 4 * k;
-      const C x0 = x[pidx<PS>(p0)], x1 = x[pidx<PS>(p0 + 1)], x2 = x[pidx<PS>(p0 + 2)], x3 = x[pidx<PS>(p0 + 3)];
-      const C b0 = cadd(x0, x2), b1 = cadd(x1, x3), b2 = csub(x0, x2);
-      const C b3 = mul_j(csub(x1, x3), inv);
-      x[pidx<PS>(p0)] = cadd(b0, b1);
-      x[pidx<PS>(p0 + 1)] = csub(b0, b1);
-      x[pidx<PS>(p0 + 2)] = cadd(b2, b3);
-      x[pidx<PS>(p0 + 3)] = csub(b2, b3);
+      const int j = k & (nq - 1), p0 = 4 * k;
+      C x0 = x[pidx<PS>(p0)], x1 = x[pidx<PS>(p0 + 1)], x2 = x[pidx<PS>(p0 + 2)], x3 = x[pidx<PS>(p0 + 3)];
+      const C w1 = tw_of(tr[j], inv), w2 = tw_of(tr[2 * j], inv);
+      bfly(x0, x2, w1); bfly(x1, x3, w1);
+      bfly(x0, x1, w2); bfly(x2, x3, tw_j(w2, inv));
+      x[pidx<PS>(p0)] = x0; x[pidx<PS>(p0 + 1)] = x1; x[pidx<PS>(p0 + 2)] = x2; x[pidx<PS>(p0 + 3)] = x3;
     }
     __syncthreads();
-  } else if (s == 1) {   // last radix-2 stage: all twiddles are 1
+  } else if (s == 1) {   // one level left
     const int nb = ntr * (n >> 1);
     for (int k = tid; k < nb; k += nthr) {
       const int i0 = 2 * k, i1 = i0 + 1;
-      const C a = x[pidx<PS>(i0)], b = x[pidx<PS>(i1)];
-      x[pidx<PS>(i0)] = cadd(a, b);
-      x[pidx<PS>(i1)] = csub(a, b);
+      C a = x[pidx<PS>(i0)], c = x[pidx<PS>(i1)];
+      bfly(a, c, tw_of(tr[k & ((n >> 1) - 1)], inv));
+      x[pidx<PS>(i0)] = a;
+      x[pidx<PS>(i1)] = c;
     }
     __syncthreads();
   }
@@ -266,7 +256,7 @@ __device__ __forceinline__ void bluestein_conv(typename Cplx<T>::type* x, int lm
                                                const typename Cplx<T>::type* __restrict__ filt,
                                                const typename Cplx<T>::type* __restrict__ tw, int lnmax, bool inv,
                                                int tid, int nthr) {
-  fft_dif<T>(x, lm, ntr, tw, lnmax, false, tid, nthr);
+  fft_rev<T>(x, lm, ntr, tw, lnmax, false, tid, nthr);
   const int m = 1 << lm;
   for (int e = tid; e < ntr * m; e += nthr) x[e] = cmul_tw(filt[e & (m - 1)], x[e], inv);
   __syncthreads();
@@ -294,7 +284,7 @@ __device__ __forceinline__ void theta_mean(const InstDev& I, int nt, double* red
   if (tid == 0) {
     double sum = 0.0;
     for (int w = 0; w < (nthr + 31) / 32; ++w) sum += red[w];
-    *mean = sum / ((double)I.nx * (double)I.ny);
+    *mean = sum * I.hscale;
   }
   __syncthreads();
 }
@@ -355,9 +345,8 @@ __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft
 
 // Column pass: a work item is a group of col_group (a power of two) adjacent
 // spectral columns, loaded and stored row by row (adjacent threads take
-// adjacent columns of one row); the forward transform runs by decimation in
-// frequency (natural order in, bit-reversed out) and the inverse by decimation
-// in time (bit-reversed in, natural out), so the symbol division takes the
+// adjacent columns of one row); the forward transform runs from natural to
+// bit-reversed order and the inverse back, so the symbol division takes the
 // spectrum in bit-reversed order and no permutation pass is needed.  The FP32
 // form runs it with blocks of 512 threads, two per SM (cols_threads<T>; at 2048^2
 // its 257 items of four columns then run in one wave: 0.098 ms per step against
@@ -398,9 +387,9 @@ __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD
       if (g < ntr) x[pidx<PS>(g * n + y)] = S[(size_t)y * ss + col0 + g];
     }
     __syncthreads();
-    fft_dif<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, false, tid, nthr);
+    fft_rev<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, false, tid, nthr);
     const double kap = I.kappa[i];
-    const double scale = 1.0 / ((double)I.nx * (double)I.ny);
+    const double scale = I.hscale;
     for (int e = tid; e < ntr * n; e += nthr) {
       const int g = e >> ln, ky = brev(e & (n - 1), ln), kx = col0 + g;
       C v = x[pidx<PS>(e)];
@@ -463,7 +452,7 @@ __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft
       x[pidx<PS>(e)] = z;
     }
     __syncthreads();
-    fft_dif<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr);
+    fft_rev<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr);
     T* th = reinterpret_cast<T*>(I.Xs[i]) + 2 * (size_t)I.nx * I.ny;
     for (int e = tid; e < ntr * n; e += nthr) {
       const int p = e >> ln, m = e & (n - 1);
@@ -495,52 +484,40 @@ __device__ __forceinline__ constexpr double root_sin(int R, int q) {
        : (q == 1 ? 0.7818314824680298087084445 : q == 2 ? 0.9749279121818236070181317 : 0.4338837391175581204757683);
 }
 
-// R-point DFT of v in place (exp(-2 pi i ab/R); conjugate roots when inv).  Odd R:
+// R-point DFT of v in place, R odd (exp(-2 pi i ab/R); conjugate roots when inv):
 // opposite inputs are paired, y_a = v_0 + sum_b [(v_b + v_{R-b}) cos - i (v_b - v_{R-b}) sin](2 pi ab/R).
 template <int R, typename C>
 __device__ __forceinline__ void small_dft(C* v, bool inv) {
   using T = decltype(v[0].x);
-  if constexpr (R == 2) {
-    const C a = v[0];
-    v[0] = cadd(a, v[1]);
-    v[1] = csub(a, v[1]);
-  } else if constexpr (R == 4) {
-    const C t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]), t2 = cadd(v[1], v[3]), t3 = mul_j(csub(v[1], v[3]), inv);
-    v[0] = cadd(t0, t2);
-    v[2] = csub(t0, t2);
-    v[1] = cadd(t1, t3);
-    v[3] = csub(t1, t3);
-  } else {
-    constexpr int H = (R - 1) / 2;
-    C sp[H], dm[H], out[R];
-    C y0 = v[0];
+  constexpr int H = (R - 1) / 2;
+  C sp[H], dm[H], out[R];
+  C y0 = v[0];
+#pragma unroll
+  for (int b = 1; b <= H; ++b) {
+    sp[b - 1] = cadd(v[b], v[R - b]);
+    dm[b - 1] = csub(v[b], v[R - b]);
+    y0 = cadd(y0, sp[b - 1]);
+  }
+  out[0] = y0;
+#pragma unroll
+  for (int a = 1; a <= H; ++a) {
+    C re = v[0], im;
+    im.x = T(0); im.y = T(0);
 #pragma unroll
     for (int b = 1; b <= H; ++b) {
-      sp[b - 1] = cadd(v[b], v[R - b]);
-      dm[b - 1] = csub(v[b], v[R - b]);
-      y0 = cadd(y0, sp[b - 1]);
+      const int q = (a * b) % R, qq = q <= H ? q : R - q;
+      const T c = T(root_cos(R, qq)), sn = q <= H ? T(root_sin(R, qq)) : -T(root_sin(R, qq));
+      re.x += c * sp[b - 1].x; re.y += c * sp[b - 1].y;
+      im.x += sn * dm[b - 1].x; im.y += sn * dm[b - 1].y;
     }
-    out[0] = y0;
-#pragma unroll
-    for (int a = 1; a <= H; ++a) {
-      C re = v[0], im;
-      im.x = T(0); im.y = T(0);
-#pragma unroll
-      for (int b = 1; b <= H; ++b) {
-        const int q = (a * b) % R, qq = q <= H ? q : R - q;
-        const T c = T(root_cos(R, qq)), sn = q <= H ? T(root_sin(R, qq)) : -T(root_sin(R, qq));
-        re.x += c * sp[b - 1].x; re.y += c * sp[b - 1].y;
-        im.x += sn * dm[b - 1].x; im.y += sn * dm[b - 1].y;
-      }
-      C ya, yb;   // re -+ i im (forward), re +- i im (inverse)
-      if (!inv) { ya.x = re.x + im.y; ya.y = re.y - im.x; yb.x = re.x - im.y; yb.y = re.y + im.x; }
-      else { ya.x = re.x - im.y; ya.y = re.y + im.x; yb.x = re.x + im.y; yb.y = re.y - im.x; }
-      out[a] = ya;
-      out[R - a] = yb;
-    }
-#pragma unroll
-    for (int a = 0; a < R; ++a) v[a] = out[a];
+    C ya, yb;   // re -+ i im (forward), re +- i im (inverse)
+    if (!inv) { ya.x = re.x + im.y; ya.y = re.y - im.x; yb.x = re.x - im.y; yb.y = re.y + im.x; }
+    else { ya.x = re.x - im.y; ya.y = re.y + im.x; yb.x = re.x + im.y; yb.y = re.y - im.x; }
+    out[a] = ya;
+    out[R - a] = yb;
   }
+#pragma unroll
+  for (int a = 0; a < R; ++a) v[a] = out[a];
 }
 
 template <typename T, int R>
@@ -555,9 +532,27 @@ __device__ __forceinline__ void stockham_pass(typename Cplx<T>::type* x, int m, 
     C* dst = x + p * m + dst_off;
     C v[R];
     v[0] = src[j];
+    if constexpr (R == 4) {
+      // two levels of butterflies with their whole twiddles: W^{2k}, then W^k times 1 and W_4
+      v[1] = src[j + nr];
+      v[2] = src[j + 2 * nr];
+      v[3] = src[j + 3 * nr];
+      const C w1 = tw_of(tw[k * tws], inv), w2 = tw_of(tw[2 * k * tws], inv);
+      bfly(v[0], v[2], w2);
+      bfly(v[1], v[3], w2);
+      bfly(v[0], v[1], w1);
+      bfly(v[2], v[3], tw_j(w1, inv));
+      const C y1 = v[2];
+      v[2] = v[1];
+      v[1] = y1;
+    } else if constexpr (R == 2) {
+      v[1] = src[j + nr];
+      bfly(v[0], v[1], tw_of(tw[k * tws], inv));
+    } else {
 #pragma unroll
-    for (int r = 1; r < R; ++r) v[r] = cmul_tw(tw[k * r * tws], src[j + r * nr], inv);
-    small_dft<R>(v, inv);
+      for (int r = 1; r < R; ++r) v[r] = cmul_tw(tw[k * r * tws], src[j + r * nr], inv);
+      small_dft<R>(v, inv);
+    }
     const int d0 = (j - k) * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) dst[d0 + r * Ns] = v[r];
@@ -665,6 +660,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs
   }
 }
 
+// v times a real factor given in FP64, rounded once: FP32 values by the factor as a pair of floats.
+__device__ __forceinline__ void apply_factor(double2& v, double f) { v.x *= f; v.y *= f; }
+__device__ __forceinline__ void apply_factor(float2& v, double f) {
+  const F2 p = f2_from_double(f), a = f2_mulf(p, v.x), c = f2_mulf(p, v.y);
+  v.x = a.h + a.l;
+  v.y = c.h + c.l;
+}
+
 // The forward Bluestein convolution differs from the spectrum along y by the
 // factor conj(w_ky), which the inverse transform's input chirp w_ky cancels,
 // so the division by the symbol applies to the convolution directly.
@@ -698,7 +701,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
       __syncthreads();
       const int off = stockham<T>(x, m, n, ntr, I.mr_plan[1], I.mr_npass[1], tw, false, 0, tid, nthr);
       const double kap = I.kappa[i];
-      const double scale = 1.0 / ((double)I.nx * (double)I.ny);
+      const double scale = I.hscale;
       for (int e = tid; e < ntr * n; e += nthr) {
         const int g = e / n, ky = e - g * n, kx = col0 + g;
         C v = x[g * m + off + ky];
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
           v.x = T(s_mean); v.y = T(0);
         } else {
           const double f = scale * rcp_newton(I.lamx[kx] + I.lamy[ky] - kap);
-          v.x = T(double(v.x) * f); v.y = T(double(v.y) * f);
+          apply_factor(v, f);
         }
         x[g * m + off + ky] = v;
       }
@@ -729,7 +732,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
     __syncthreads();
     bluestein_conv<T>(x, ln, ntr, filt, twiddles<T>(b), b.lnmax, false, tid, nthr);
     const double kap = I.kappa[i];
-    const double scale = 1.0 / ((double)I.nx * (double)I.ny);
+    const double scale = I.hscale;
     for (int e = tid; e < ntr * m; e += nthr) {
       const int g = e >> ln, ky = e & (m - 1), kx = col0 + g;
       C v = x[e];
@@ -739,7 +742,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
         v.x = T(s_mean); v.y = T(0);
       } else {
         const double f = scale * rcp_newton(I.lamx[kx] + I.lamy[ky] - kap);
-        v.x = T(double(v.x) * f); v.y = T(double(v.y) * f);
+        apply_factor(v, f);
       }
       x[e] = v;
     }

@@ -46,7 +46,7 @@ Layout layout(const ap_dvm_params& p, int nmax) {
   L.col_start = take(2 * sizeof(int));
   L.rhs_start = take(2 * sizeof(int));
   L.counts = take(8 * sizeof(int));
-  L.tw = take(sizeof(double2) * (nmax / 2));
+  L.tw = take(sizeof(double2) * nmax);
   L.err = take(4 * sizeof(unsigned));
   L.ws = take(carve_instance(p, nullptr, nullptr));
   L.total = align_up(off, 256);
@@ -143,14 +143,10 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   const int nrhs = rhs_items(p->nx, p->ny, false);
   const int ts[2] = {0, ntiles}, rs[2] = {0, nrows}, cs[2] = {0, ncols}, hs[2] = {0, nrhs};
   const int counts[8] = {ntiles, nrows, ncols, 1, nrhs, ntiles, 0, 0};
-  double2 tw[64];                                   // nmax/2 <= 64 for grids of at most 128 cells a side
+  double2 tw[128];                                  // nmax <= 128: grids of at most 128 cells a side
   double lx[65], ly[128];
-  const long double pi = 3.141592653589793238462643383279502884L;
-  for (int k = 0; k < nmax / 2; ++k) {
-    const long double a = -2.0L * pi * (long double)k / (long double)nmax;
-    tw[k].x = (double)std::cos(a);
-    tw[k].y = (double)std::sin(a);
-  }
+  twiddle_table(nmax, [&](int k, long double c, long double sn) { tw[k] = make_double2((double)c, (double)sn); },
+                [&](int k, int j) { tw[k] = tw[j]; });
   laplacian_symbol(p->nx, I.dx, p->space_scheme, lx, p->nx / 2 + 1);
   laplacian_symbol(p->ny, I.dy, p->space_scheme, ly, p->ny);
   NA_TRY(cudaMemcpyAsync(base + L.batch, &B, sizeof(B), cudaMemcpyHostToDevice, stream));
@@ -160,7 +156,7 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   NA_TRY(cudaMemcpyAsync(B.col_start, cs, sizeof(cs), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(B.rhs_start, hs, sizeof(hs), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(B.counts, counts, sizeof(counts), cudaMemcpyHostToDevice, stream));
-  NA_TRY(cudaMemcpyAsync(B.tw, tw, sizeof(double2) * (nmax / 2), cudaMemcpyHostToDevice, stream));
+  NA_TRY(cudaMemcpyAsync(B.tw, tw, sizeof(double2) * nmax, cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(I.lamx, lx, sizeof(double) * (p->nx / 2 + 1), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(I.lamy, ly, sizeof(double) * p->ny, cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemsetAsync(B.err, 0, 4 * sizeof(unsigned), stream));

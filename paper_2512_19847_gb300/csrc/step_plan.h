@@ -340,7 +340,8 @@ inline void fill_constants(const ap_dvm_params& p, InstDev& d) {
   }
   d.inv_dx = 1.0 / d.dx;
   d.inv_dy = 1.0 / d.dy;
-  d.hscale32 = (float)(1.0 / ((double)p.nx * (double)p.ny));
+  d.hscale = 1.0 / ((double)p.nx * (double)p.ny);
+  d.hscale32 = (float)d.hscale;
   for (int i = 1; i <= p.s; ++i) {
     const double a = p.A_im[(i - 1) * AP_DVM_MAX_STAGES + (i - 1)];
     d.inv_aii[i] = a != 0.0 ? 1.0 / a : 0.0;

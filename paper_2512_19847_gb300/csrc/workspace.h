@@ -103,6 +103,26 @@ inline size_t carve_instance(const ap_dvm_params& p, char* base, InstDev* d, boo
   return align_up(off, 256);
 }
 
+// Twiddles of transforms up to length nmax (a power of two): exp(-2 pi i k / nmax) for k < nmax / 2, then the
+// same in bit-reversed order (exp(-pi i f_j), f_j the fraction with j's bits after the point in reverse).
+// put(k, cos, sin) sets value k, copy(k, j) sets it to value j.
+template <class Put, class Copy>
+inline void twiddle_table(int nmax, Put&& put, Copy&& copy) {
+  const long double pi = 3.141592653589793238462643383279502884L;
+  const int half = nmax / 2;
+  for (int k = 0; k < half; ++k) {
+    const long double a = -2.0L * pi * (long double)k / (long double)nmax;
+    put(k, std::cos(a), std::sin(a));
+  }
+  for (int k = 0, r = 0; k < half; ++k) {
+    copy(half + k, r);
+    for (int bit = half >> 1; bit; bit >>= 1) {   // r: k's bits in reverse
+      r ^= bit;
+      if (r & bit) break;
+    }
+  }
+}
+
 // 1D symbol of the Laplacian stencil on DFT mode k (compact 3-point or 4th-order
 // 5-point second difference, Sec. 3.2), without cancellation for small k.
 inline void laplacian_symbol(int n, double h, int scheme, double* out, int count) {
