@@ -303,7 +303,12 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
   const int cells = h->ks.tx * h->ks.ty, thr = cells * h->ks.tz;
   ap_dvm_status st;
   if ((st = occupancy_grid(h, h->ks.k_explicit, thr, h->ks.smem_explicit, &h->grid_explicit))) return st;
-  if ((st = occupancy_grid(h, h->ks.k_rhs, h->ks.rhs_threads, 0, &h->grid_rhs))) return st;
+  h->grid_rhs = 1 << 30;
+  for (const void* fn : h->ks.k_rhs) {
+    int g = 0;
+    if ((st = occupancy_grid(h, fn, h->ks.rhs_threads, 0, &g))) return st;
+    h->grid_rhs = std::min(h->grid_rhs, g);
+  }
   h->smem_update = update_smem(h->ks, h->tmpl);
   if ((st = occupancy_grid(h, h->ks.k_update, thr, h->smem_update, &h->grid_update))) return st;
   if (h->ks.k_explicit_split) {

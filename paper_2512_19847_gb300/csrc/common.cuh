@@ -218,18 +218,21 @@ __device__ __forceinline__ T cdiff2(const T* f, int st, T inv_h2) {
 }
 
 // The same two differences from the values at offsets -2 .. 2 along a line, without
-// their scale (fm2 and fp2 unused by the second-order scheme): the first difference is
-// d1_scale(inv_h) * d1_sum(...), the second d2_scale(inv_h) * d2_sum(...).
+// their scale (fm2 and fp2 unused by the second-order scheme) and, the second, without its centre
+// value: the first difference is d1_scale(inv_h) * d1_sum(...), the second
+// d2_scale(inv_h) * (d2_sum(...) + d2_centre() * f0).
 template <typename T, int SCHEME>
 __device__ __forceinline__ T d1_sum(T fm2, T fm1, T fp1, T fp2) {
   if (SCHEME == LF1_C2) return fp1 - fm1;
   return T(8) * (fp1 - fm1) - (fp2 - fm2);
 }
 template <typename T, int SCHEME>
-__device__ __forceinline__ T d2_sum(T fm2, T fm1, T f0, T fp1, T fp2) {
-  if (SCHEME == LF1_C2) return (fp1 + fm1) - T(2) * f0;
-  return T(16) * (fp1 + fm1) - T(30) * f0 - (fp2 + fm2);
+__device__ __forceinline__ T d2_sum(T fm2, T fm1, T fp1, T fp2) {
+  if (SCHEME == LF1_C2) return fp1 + fm1;
+  return T(16) * (fp1 + fm1) - (fp2 + fm2);
 }
+template <typename T, int SCHEME>
+__device__ __forceinline__ constexpr T d2_centre() { return SCHEME == LF1_C2 ? T(-2) : T(-30); }
 template <typename T, int SCHEME>
 __device__ __forceinline__ T d1_scale(T inv_h) { return SCHEME == LF1_C2 ? T(0.5) * inv_h : inv_h * T(1.0 / 12.0); }
 template <typename T, int SCHEME>

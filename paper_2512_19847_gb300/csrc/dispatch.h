@@ -39,7 +39,7 @@ inline int pick_tile(bool f32, int minx, int miny, int num_sms, Tiles&& tiles) {
 
 struct StencilSet {
   const void* k_explicit;
-  const void* k_rhs;
+  const void* k_rhs[3];                // 1, 4, or up to the most terms of earlier stages
   const void* k_update;
   const void* k_explicit_split;        // FP64 WENO: the same with split fluxes (null otherwise)
   const void* k_update_split;

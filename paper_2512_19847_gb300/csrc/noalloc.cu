@@ -105,7 +105,12 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   const int cells = ks.tx * ks.ty, thr = cells * ks.tz;
   int g_exp = 0, g_rhs = 0, g_upd = 0, g_fin = 0, g1 = 0, g2 = 0, g3 = 0;
   NA_TRY(grid_of(ks.k_explicit, thr, ks.smem_explicit, sms, &g_exp));
-  NA_TRY(grid_of(ks.k_rhs, ks.rhs_threads, 0, sms, &g_rhs));
+  g_rhs = 1 << 30;
+  for (const void* fn : ks.k_rhs) {
+    int g = 0;
+    NA_TRY(grid_of(fn, ks.rhs_threads, 0, sms, &g));
+    g_rhs = std::min(g_rhs, g);
+  }
   const size_t smem_upd = update_smem(ks, *p);
   NA_TRY(grid_of(ks.k_update, thr, smem_upd, sms, &g_upd));
   NA_TRY(grid_of(km.k_finish, cells, 0, sms, &g_fin));

@@ -219,7 +219,10 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     int first = (i == (type_a ? 1 : 2)) ? 1 : 0;           // the first right-hand side also sums theta^n
     {
       void* a[] = {&bp, &i, &sign, &first};
-      if ((st = launch(K.ks.k_rhs, K.g_rhs, dim3(K.ks.rhs_threads), 0, a, KK_RHS))) return st;
+      int terms = 1;   // D_0 . u^n, and three planes of every earlier stage with a_ij
+      for (int k = 1; k < i; ++k) terms += AIM(i, k) != 0.0 ? 3 : 0;
+      const void* fn = K.ks.k_rhs[terms == 1 ? 0 : (terms == 4 ? 1 : 2)];
+      if ((st = launch(fn, K.g_rhs, dim3(K.ks.rhs_threads), 0, a, KK_RHS))) return st;
     }
     {
       // each pass: the power-of-two kernel and/or the Bluestein kernel, as the batch needs
