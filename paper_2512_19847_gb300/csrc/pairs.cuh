@@ -20,6 +20,12 @@ __device__ __forceinline__ F2 f2_addk(F2 a, F2 b) {
 }
 __device__ __forceinline__ F2 f2_add(F2 a, F2 b) { return f2_addk<1>(a, b); }
 __device__ __forceinline__ F2 f2_sub(F2 a, F2 b) { return f2_addk<-1>(a, b); }
+// a + k b for k = 1 or -1 given at run time.
+__device__ __forceinline__ F2 f2_addr(F2 a, F2 b, float k) {
+  const float s = __fmaf_rn(k, b.h, a.h), bb = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fmaf_rn(k, b.h, -bb));
+  return f2(s, __fadd_rn(e, __fmaf_rn(k, b.l, a.l)));
+}
 // The same value with |l| <= ulp(h)/2.
 __device__ __forceinline__ F2 f2_norm(F2 a) {
   const float h = __fadd_rn(a.h, a.l);
@@ -31,8 +37,7 @@ __device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
 }
 __device__ __forceinline__ F2 f2_sqr(F2 a) {
   const float p = __fmul_rn(a.h, a.h);
-  const float t = __fmul_rn(a.h, a.l);
-  return f2(p, __fadd_rn(t, __fadd_rn(t, __fmaf_rn(a.h, a.h, -p))));
+  return f2(p, __fmaf_rn(a.h, a.l, __fmaf_rn(a.h, a.l, __fmaf_rn(a.h, a.h, -p))));
 }
 // k a for an integer k that is a float.
 __device__ __forceinline__ F2 f2_scale(F2 a, float k) {

@@ -29,8 +29,8 @@ namespace apd {
 // q[m] = c + 2 w0 T_{out} + w2 T_{in} from the increments D[m .. m + 3] of its stencil (upwind
 // to downwind; T_out = D[m+2] - 2 D[m+1] + D[m], T_in one further), w = 16 eps_W (the
 // indicators times 4, the doubled split).  With the e_k scaled by a power of two so that the
-// largest is about 1, and then their products likewise, every step stays in the float range
-// whatever the data and eps_W: what underflows is below 2^-60 of the sum it belongs to.
+// largest is about 1, and their products likewise where even the largest is small, every step stays in
+// the float range whatever the data and eps_W: what underflows is below 2^-60 of the sum it belongs to.
 template <int KR>
 __device__ __forceinline__ void w5_split(const F2* D, F2 w, F2* q) {
   F2 c[KR + 3], C[KR + 3];
@@ -43,6 +43,7 @@ __device__ __forceinline__ void w5_split(const F2* D, F2 w, F2* q) {
     const float pl = __fmaf_rn(kl, s.h, __fmaf_rn(kh, s.l, __fmaf_rn(kh, s.h, -p)));
     C[k] = f2_add(w, f2(p, pl));
   }
+  F2 to = f2_sub(c[2], c[1]);
 #pragma unroll
   for (int m = 0; m < KR; ++m) {
     F2 e0 = f2_add(C[m + 1], f2_sqr(f2_addk<2>(c[m + 1], D[m + 1])));
@@ -53,14 +54,18 @@ __device__ __forceinline__ void w5_split(const F2* D, F2 w, F2* q) {
     e1 = f2(e1.h * se, e1.l * se);
     e2 = f2(e2.h * se, e2.l * se);
     F2 pa = f2_mul(e1, e2), pb = f2_mul(e0, e2), pc = f2_mul(e0, e1);
-    const float sp = inv_pow2(fmaxf(fmaxf(pa.h, pb.h), pc.h));
-    pa = f2(pa.h * sp, pa.l * sp);
-    pb = f2(pb.h * sp, pb.l * sp);
-    pc = f2(pc.h * sp, pc.l * sp);
+    const float pm = fmaxf(fmaxf(pa.h, pb.h), pc.h);
+    if (pm < 9.09e-13f) {   // 2^-40
+      const float sp = inv_pow2(pm);
+      pa = f2(pa.h * sp, pa.l * sp);
+      pb = f2(pb.h * sp, pb.l * sp);
+      pc = f2(pc.h * sp, pc.l * sp);
+    }
     const F2 A = f2_sqr(pa), B = f2_scale(f2_sqr(pb), 6.f), E = f2_scale(f2_sqr(pc), 3.f);
     const F2 den = f2_add(f2_add(A, E), B);
-    const F2 to = f2_sub(c[m + 2], c[m + 1]), ti = f2_sub(c[m + 3], c[m + 2]);
+    const F2 ti = f2_sub(c[m + 3], c[m + 2]);
     q[m] = f2_add(c[m + 2], f2_div(f2_addk<2>(f2_mul(E, ti), f2_mul(A, to)), den));
+    to = ti;
   }
 }
 

@@ -100,33 +100,35 @@ __device__ __forceinline__ void split_increments_update(const double* s, int nw,
   }
 }
 
-// Pass 2, one run: the increments of g and U at ig, iu (stride st between points, npt in the line),
-// sg = -1 negates g; N of interfaces m0 .. m0 + KR - 1 into out (stride so), those below ni only.
-template <int SCHEME, int KR>
+// Pass 2, one run: the increments of g and U at ig, iu (stride st between points, npt in the line);
+// N of interfaces m0 .. m0 + KR - 1 into out (stride so), those below ni only.  sg = -1 negates g, by
+// exchanging the two reconstructions (-g + U = -(g - U)).  CLAMP: runs may reach past the line.
+template <int SCHEME, int KR, bool CLAMP>
 __device__ __forceinline__ void split_run(const F2* ig, const F2* iu, float sg, int st, int npt, F2 w, F2* out, int so,
                                           int m0, int ni) {
   constexpr int NS = SCHEME == WENO5_C4 ? 4 : 2, ND = KR + NS;
   F2 D[ND], q[KR], qm[KR];
 #pragma unroll
   for (int j = 0; j < ND - 1; ++j) {
-    const int o = min(m0 + j, npt - 1) * st;
-    const F2 a = ig[o];
-    D[j] = f2_norm(f2_add(f2(sg * a.h, sg * a.l), iu[o]));
+    const int o = (CLAMP ? min(m0 + j, npt - 1) : m0 + j) * st;
+    D[j] = f2_norm(f2_addr(ig[o], iu[o], sg));
   }
   if constexpr (SCHEME == WENO5_C4) w5_split<KR>(D, w, q);
   else w3_split<KR>(D, w, q);
-  // g- from the right: the same with the increments in reverse
+  // from the right: the same with the increments in reverse
 #pragma unroll
   for (int j = 1; j < ND; ++j) {
-    const int o = min(m0 + j, npt - 1) * st;
-    const F2 a = ig[o];
-    D[ND - 1 - j] = f2_norm(f2_sub(f2(sg * a.h, sg * a.l), iu[o]));
+    const int o = (CLAMP ? min(m0 + j, npt - 1) : m0 + j) * st;
+    D[ND - 1 - j] = f2_norm(f2_addr(ig[o], iu[o], -sg));
   }
   if constexpr (SCHEME == WENO5_C4) w5_split<KR>(D, w, qm);
   else w3_split<KR>(D, w, qm);
 #pragma unroll
   for (int i = 0; i < KR; ++i)
-    if (m0 + i < ni) out[(m0 + i) * so] = f2_norm(f2_sub(qm[KR - 1 - i], q[i]));
+    if (!CLAMP || m0 + i < ni) {
+      const F2 r = f2_norm(f2_sub(qm[KR - 1 - i], q[i]));
+      out[(m0 + i) * so] = f2(sg * r.h, sg * r.l);
+    }
 }
 
 // Pass 2: NP pairs per axis.  Pair p takes the fields gi(p) and ui(p) of the increments
@@ -138,6 +140,7 @@ __device__ __forceinline__ void split_interfaces(const F2* ix, const F2* iy, F2*
   constexpr int KR = APD_SPLIT_RUN;
   constexpr int RX = (TX + 1 + KR - 1) / KR, RY = (TY + 1 + KR - 1) / KR;
   constexpr int IX = NP * TY * RX, IY = NP * TX * RY;
+  constexpr bool CLAMP = (TX + 1) % KR != 0 || (TY + 1) % KR != 0;
   for (int k = tid; k < IX + IY; k += G::NT) {
     const bool ax = k < IX;
     const int kk = ax ? k : k - IX, nl = ax ? TY : TX, per = ax ? TY * RX : TX * RY;
@@ -145,7 +148,7 @@ __device__ __forceinline__ void split_interfaces(const F2* ix, const F2* iy, F2*
     const int gi = p, ui = NP == 1 ? 1 : (NP == 2 ? 2 + p : (p == 0 ? 1 : 2 + p));
     const F2* base = ax ? ix + line * S::LX : iy + line;
     const int fs = ax ? S::LIX : S::LIY;
-    split_run<SCHEME, KR>(base + gi * fs, base + ui * fs, (ax && p == NEGX) ? -1.f : 1.f, ax ? 1 : TX, ax ? S::LX : S::LY, w,
+    split_run<SCHEME, KR, CLAMP>(base + gi * fs, base + ui * fs, (ax && p == NEGX) ? -1.f : 1.f, ax ? 1 : TX, ax ? S::LX : S::LY, w,
                           ax ? nx + p * G::NX + line * (TX + 1) : ny + p * G::NY + line, ax ? 1 : TX, run * KR,
                           ax ? TX + 1 : TY + 1);
   }
