@@ -76,7 +76,6 @@ struct ap_dvm_handle {
   bool dependent = false;            // launch a step's kernels as programmatic dependents
   int nmax = 0, lnmax = 0, eblk = 0, eblk_cols = 0;
   // batch workspace
-  BatchDev* d_batch[2] = {nullptr, nullptr};   // per step parity (double-buffered state)
   InstDev* d_inst[2] = {nullptr, nullptr};
   int* d_tile_start = nullptr;
   int* d_row_start = nullptr;
@@ -87,7 +86,7 @@ struct ap_dvm_handle {
   double2* d_tw = nullptr;
   float2* d_tw32 = nullptr;
   unsigned* d_err = nullptr;
-  BatchDev hb[2]{};
+  BatchDev hb[2]{};                  // per step parity (double-buffered state)
   int parity = 0;                    // parity of the next step: which state buffer it reads
   std::vector<Slot> slots;
   bool dirty = true;
@@ -226,7 +225,6 @@ bool same_method(const ap_dvm_params& a, const ap_dvm_params& b) {
 size_t batch_bytes(int capacity, int nmax) {
   size_t off = 0;
   auto take = [&](size_t b) { off = align_up(off, 256); off += b; };
-  take(sizeof(BatchDev) * 2);
   take(sizeof(InstDev) * capacity * 2);
   take(sizeof(int) * (capacity + 1));
   take(sizeof(int) * (capacity + 1));
@@ -520,7 +518,7 @@ ap_dvm_status enqueue_step(ap_dvm_handle* h, cudaStream_t stream, int parity) {
   auto ln = [&](const void* fn, int grid, dim3 block, size_t smem, void** args, int kind) -> int {
     return (int)launch(h, stream, fn, grid, block, smem, args, kind);
   };
-  return (ap_dvm_status)enqueue_imex_step(h->tmpl, K, h->d_batch[parity], h->tmpl.precision, ln, true);
+  return (ap_dvm_status)enqueue_imex_step(h->tmpl, K, h->hb[parity], h->tmpl.precision, ln, true);
 }
 
 // A CUDA graph of graph_steps steps starting at the given parity.
@@ -624,10 +622,8 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   char* base = reinterpret_cast<char*>(d_workspace);
   size_t off = 0;
   auto take = [&](size_t b) { off = align_up(off, 256); char* r = base + off; off += b; return r; };
-  BatchDev* batches = reinterpret_cast<BatchDev*>(take(sizeof(BatchDev) * 2));
   InstDev* insts = reinterpret_cast<InstDev*>(take(sizeof(InstDev) * capacity * 2));
   for (int par = 0; par < 2; ++par) {
-    h->d_batch[par] = batches + par;
     h->d_inst[par] = insts + (size_t)par * capacity;
   }
   h->d_tile_start = reinterpret_cast<int*>(take(sizeof(int) * (capacity + 1)));
@@ -665,8 +661,6 @@ ap_dvm_status ap_dvm_batch_create(const ap_dvm_params* tmpl, int capacity, void*
   CUDA_TRY(h, cudaMemcpyAsync(h->d_tw32, tw32.data(), sizeof(float2) * tw32.size(), cudaMemcpyHostToDevice, h->stream));
   h->hb[1] = hb;
   h->hb[1].inst = h->d_inst[1];
-  for (int par = 0; par < 2; ++par)
-    CUDA_TRY(h, cudaMemcpyAsync(h->d_batch[par], &h->hb[par], sizeof(BatchDev), cudaMemcpyHostToDevice, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned) * 4, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, sizeof(int) * 8, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));

@@ -116,7 +116,8 @@ struct InstDev {
   int pad1;
 };
 
-// Work decomposition of the active instances: item ranges per instance are
+// Work decomposition of the active instances, passed by value to the kernels of a step (its pointers and
+// tableau are the handle's for good; what changes with the set of solves lies behind the pointers): item ranges per instance are
 // prefix sums (start[k] .. start[k+1]); an item is decoded by binary search.
 struct BatchDev {
   InstDev* inst;         // active instances, compacted

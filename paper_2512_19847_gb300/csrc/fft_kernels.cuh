@@ -302,13 +302,12 @@ template <typename T>
 __host__ __device__ constexpr int rows_min_blocks() { return sizeof(T) == 4 ? 1024 / APD_ROWS_THREADS32 : 3; }
 
 template <typename T>
-__global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_fwd(const BatchDev* __restrict__ bp) {
+__global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_fwd(const __grid_constant__ BatchDev b) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
-  const BatchDev& b = *bp;
   const int nitems = b.counts[1], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.row_start, b.counts[3], it);
@@ -361,7 +360,7 @@ __host__ __device__ constexpr int cols_threads() { return sizeof(T) == 4 ? APD_C
 
 template <typename T>
 __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD_COLS_THREADS32 : 2)
-    k_fft_cols(const BatchDev* __restrict__ bp, int i) {
+    k_fft_cols(const __grid_constant__ BatchDev b, int i) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
@@ -369,7 +368,6 @@ __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD
   C* x = reinterpret_cast<C*>(smem_raw);
   __shared__ double red[32];
   __shared__ double s_mean;
-  const BatchDev& b = *bp;
   const int nitems = b.counts[2], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.col_start, b.counts[3], it);
@@ -417,13 +415,12 @@ __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD
 }
 
 template <typename T>
-__global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_inv(const BatchDev* __restrict__ bp, int i) {
+__global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft_rows_inv(const __grid_constant__ BatchDev b, int i) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   constexpr int PS = pad_shift<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
-  const BatchDev& b = *bp;
   const int nitems = b.counts[1], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.row_start, b.counts[3], it);
@@ -587,12 +584,11 @@ __device__ __forceinline__ int stockham(typename Cplx<T>::type* x, int m, int n,
 // buffers as well) back to back
 
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs(const BatchDev* __restrict__ bp) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs(const __grid_constant__ BatchDev b) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
-  const BatchDev& b = *bp;
   const int nitems = b.counts[1], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.row_start, b.counts[3], it);
@@ -672,14 +668,13 @@ __device__ __forceinline__ void apply_factor(float2& v, double f) {
 // factor conj(w_ky), which the inverse transform's input chirp w_ky cancels,
 // so the division by the symbol applies to the convolution directly.
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(const BatchDev* __restrict__ bp, int i) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(const __grid_constant__ BatchDev b, int i) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
   __shared__ double red[8];
   __shared__ double s_mean;
-  const BatchDev& b = *bp;
   const int nitems = b.counts[2], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.col_start, b.counts[3], it);
@@ -757,12 +752,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs(const BatchDev* __restrict__ bp, int i) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs(const __grid_constant__ BatchDev b, int i) {
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* x = reinterpret_cast<C*>(smem_raw);
-  const BatchDev& b = *bp;
   const int nitems = b.counts[1], tid = threadIdx.x, nthr = blockDim.x;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int k_inst = find_inst(b.row_start, b.counts[3], it);

@@ -257,9 +257,8 @@ __global__ void __launch_bounds__(256) k_diagnostics(InstDev I, int c4, double* 
 // over j < 1 are empty), into X^(1), and D_0 . u^n for the right-hand sides of
 // step 2, with the scheme's central difference (c4: 4th order, else 2nd).
 template <typename T, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) k_stage1(const BatchDev* __restrict__ bp, int c4) {
+__global__ void __launch_bounds__(TX* TY) k_stage1(const __grid_constant__ BatchDev b, int c4) {
   grid_dependency();
-  const BatchDev& b = *bp;
   const int ntiles = b.counts[0];
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
     const int k_inst = find_inst(b.tile_start, b.counts[3], it);
@@ -300,9 +299,8 @@ __global__ void __launch_bounds__(TX* TY) k_stage1(const BatchDev* __restrict__ 
 // as the next step's X; with theta carried (f32form = 2) the next step's
 // theta is theta^(s) itself, not the one summed from the populations.
 template <typename T, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) k_finish(const BatchDev* __restrict__ bp, int f32form) {
+__global__ void __launch_bounds__(TX* TY) k_finish(const __grid_constant__ BatchDev b, int f32form) {
   grid_dependency();
-  const BatchDev& b = *bp;
   const int ntiles = b.counts[0];
   const int s = b.s;
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {

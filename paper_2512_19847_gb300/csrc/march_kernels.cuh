@@ -155,10 +155,9 @@ struct MarchTerms {
 // D_LF . B(v^(j)) + D_0 theta^(j) are needed; NT: terms of v^(j+1) read from memory
 // (v^n and the earlier stages' E and v; 5: up to that many).
 template <bool E, bool B, int NT>
-__global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_march(const BatchDev* __restrict__ bp, int j, unsigned need,
+__global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_march(const __grid_constant__ BatchDev b, int j, unsigned need,
                                                                                   double weno_eps) {
   grid_dependency();
-  const BatchDev& b = *bp;
   const int lane = threadIdx.x & 31;
   const int ntasks = b.march_start[0][b.counts[3]];
   const float ew4 = 16.f * float(weno_eps);
@@ -306,12 +305,11 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
 // k_update (stencil_kernels.cuh) for stage i.  NW: stages in the dissipation partner, NT: earlier
 // stages in the sums of steps 3 and 4 (NT = 3: up to NW and NT of them).
 template <int NW, int NT>
-__global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_march(const BatchDev* __restrict__ bp, int i, double weno_eps,
+__global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_march(const __grid_constant__ BatchDev b, int i, double weno_eps,
                                                                                 int close_step, int form) {
   grid_dependency();
   constexpr bool GEN = NT == 3;
   constexpr int MT = NT > 0 ? NT : 1;
-  const BatchDev& b = *bp;
   const int lane = threadIdx.x & 31;
   const int ntasks = b.march_start[1][b.counts[3]];
   const float ew4 = 16.f * float(weno_eps);

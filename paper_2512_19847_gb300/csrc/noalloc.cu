@@ -31,7 +31,7 @@ void* g_scratch_ptr[kMaxDevices] = {nullptr};
 
 // Layout of the scratch: batch tables, then the instance's planes.
 struct Layout {
-  size_t batch, inst, tile_start, row_start, col_start, rhs_start, counts, tw, err, ws;
+  size_t inst, tile_start, row_start, col_start, rhs_start, counts, tw, err, ws;
   size_t total;
 };
 
@@ -39,7 +39,6 @@ Layout layout(const ap_dvm_params& p, int nmax) {
   Layout L{};
   size_t off = 0;
   auto take = [&](size_t b) { off = align_up(off, 256); size_t r = off; off += b; return r; };
-  L.batch = take(sizeof(BatchDev));
   L.inst = take(sizeof(InstDev));
   L.tile_start = take(2 * sizeof(int));
   L.row_start = take(2 * sizeof(int));
@@ -154,7 +153,6 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
                 [&](int k, int j) { tw[k] = tw[j]; });
   laplacian_symbol(p->nx, I.dx, p->space_scheme, lx, p->nx / 2 + 1);
   laplacian_symbol(p->ny, I.dy, p->space_scheme, ly, p->ny);
-  NA_TRY(cudaMemcpyAsync(base + L.batch, &B, sizeof(B), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(base + L.inst, &I, sizeof(I), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(B.tile_start, ts, sizeof(ts), cudaMemcpyHostToDevice, stream));
   NA_TRY(cudaMemcpyAsync(B.row_start, rs, sizeof(rs), cudaMemcpyHostToDevice, stream));
@@ -171,14 +169,13 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   NA_TRY(cudaStreamSynchronize(stream));            // the host-stack sources above go out of scope
 
   // the steps: the launch sequence of one IMEX step shared with the handle path
-  BatchDev* bp = reinterpret_cast<BatchDev*>(base + L.batch);
   StepKernels K{ks, km, g_exp, g_rhs, g_upd, g_fin, g_fft, g2, km.cols_threads, fft_smem, cols_smem, smem_upd, FFT_X_POW2 | FFT_Y_POW2,
                 g_fft};
   auto ln = [&](const void* fn, int grid, dim3 block, size_t smem, void** args, int) -> int {
     return launch_dependent(fn, grid, block, smem, args, stream) == cudaSuccess ? 0 : (int)AP_DVM_ERR_CUDA;
   };
   for (int step = 0; step < nsteps; ++step) {
-    const int st = enqueue_imex_step(*p, K, bp, 0, ln);
+    const int st = enqueue_imex_step(*p, K, B, 0, ln);
     if (st) return (ap_dvm_status)st;
   }
   NA_TRY(cudaMemcpyAsync(d_state6, I.X, 6 * sizeof(double) * p->nx * p->ny, cudaMemcpyDeviceToDevice, stream));

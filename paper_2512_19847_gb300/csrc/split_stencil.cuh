@@ -175,7 +175,7 @@ __device__ __forceinline__ F2 f2_of(double x) {
 // ---------------------------------------------------------------------------
 // k_explicit (stencil_kernels.cuh) with split fluxes.
 template <int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_explicit_split(const BatchDev* __restrict__ bp, int j, unsigned need,
+__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_explicit_split(const __grid_constant__ BatchDev b, int j, unsigned need,
                                                                                 double weno_eps) {
   grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
@@ -188,7 +188,6 @@ __global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blo
   F2* iy = ix + 5 * S::LIX;
   F2* nxs = iy + 5 * S::LIY;   // [3][NX]: (q;v1), (-v1;u1), (v2;u2)
   F2* nys = nxs + 3 * NX;      // [3][NY]: (q;v2), (v2;u1), (v1;u2)
-  const BatchDev& b = *bp;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const F2 w = f2_of((SCHEME == WENO5_C4 ? 16.0 : 4.0) * weno_eps);
   const bool needB = (need & NEED_DLFB) != 0, needE = (need & NEED_E) != 0;
@@ -271,7 +270,7 @@ __global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blo
 
 // k_update (stencil_kernels.cuh) with split fluxes.
 template <int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_update_split(const BatchDev* __restrict__ bp, int i, double weno_eps,
+__global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blocks<SCHEME, SplitGeo<SCHEME, TX, TY>::G::NT>()) k_update_split(const __grid_constant__ BatchDev b, int i, double weno_eps,
                                                                               int close_step, int form) {
   grid_dependency();
   using S = SplitGeo<SCHEME, TX, TY>;
@@ -279,7 +278,6 @@ __global__ void __launch_bounds__(SplitGeo<SCHEME, TX, TY>::G::NT, split_min_blo
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t bars[2];
-  const BatchDev& b = *bp;
   const PlaneList pr = update_planes(b, i);
   double* stage = aligned_smem<double>(smem_raw);
   F2* ix = reinterpret_cast<F2*>(stage + S::NBUF * pr.n * PL);

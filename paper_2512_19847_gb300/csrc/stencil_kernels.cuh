@@ -727,7 +727,7 @@ __device__ __forceinline__ T flux_scale(T inv_h) {
 
 // ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_explicit(const BatchDev* __restrict__ bp, int j, unsigned need, double weno_eps) {
+__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_explicit(const __grid_constant__ BatchDev b, int j, unsigned need, double weno_eps) {
   grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
@@ -737,7 +737,6 @@ __global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks
   T* split = stage + 2 * 6 * PL;          // 3 pairs
   T* fx = split + 3 * G::SPLIT_PER_PAIR;  // [3][NX]: (q;v1), (-v1;u1), (v2;u2)
   T* fy = fx + 3 * NX;                    // [3][NY]: (q;v2), (v2;u1), (v1;u2)
-  const BatchDev& b = *bp;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * TX + threadIdx.z * TX * TY;
   const T ew = T(weno_eps);
   const bool needB = (need & NEED_DLFB) != 0, needE = (need & NEED_E) != 0;
@@ -858,7 +857,7 @@ constexpr int RHS_THREADS = 32 * RHS_WARPS;
 constexpr int RHS_MAXT = 1 + 3 * (APD_MAXS - 1);
 template <typename T, int SCHEME, int NT>
 __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 : APD_RHS_MINB64)
-    k_rhs(const BatchDev* __restrict__ bp, int i, double theta_sign, int first_stage) {
+    k_rhs(const __grid_constant__ BatchDev b, int i, double theta_sign, int first_stage) {
   grid_dependency();
   constexpr int MAXT = RHS_MAXT;
   constexpr int NR = 2 * rhs_pairs(sizeof(T) == 4);   // rows per item
@@ -867,7 +866,6 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
   __shared__ T tc[MAXT];
   __shared__ int s_nt;
   __shared__ double red[RHS_WARPS];
-  const BatchDev& b = *bp;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nitems = b.counts[4];
   int cur = -1;   // instance whose coefficient list is in tp, tc
@@ -990,14 +988,13 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
 
 // ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
-__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_update(const BatchDev* __restrict__ bp, int i, double weno_eps,
+__global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_update(const __grid_constant__ BatchDev b, int i, double weno_eps,
                                                                        int close_step, int form) {
   grid_dependency();
   using G = Geo<T, SCHEME, TX, TY>;
   constexpr int BW = G::BW, PL = G::PL, NX = G::NX, NY = G::NY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t bars[2];
-  const BatchDev& b = *bp;
   const PlaneList pr = update_planes(b, i);
   const int np = pr.n;
   T* stage = aligned_smem<T>(smem_raw);    // 2 x np planes

@@ -179,9 +179,10 @@ inline cudaError_t launch_dependent(const void* fn, int grid, dim3 block, size_t
 // (I.Xnext; the handle path's double-buffered state), else a finish kernel
 // closes it in place.
 template <class Launch>
-int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp, int form, Launch&& launch,
+int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, const BatchDev& batch, int form, Launch&& launch,
                       bool fused = false) {
   const int s = t.s;
+  void* bp = const_cast<BatchDev*>(&batch);   // copied into each launch's parameters
   const dim3 blk(K.ks.tx, K.ks.ty, K.ks.tz), cells(K.ks.tx, K.ks.ty);
   double weno_eps = t.weno_eps;
   int st;
@@ -191,7 +192,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
   const bool type_a = AIM(1, 1) != 0.0;
   if (type_a) {
     int c4 = t.space_scheme != AP_DVM_LF1_C2;
-    void* a[] = {&bp, &c4};
+    void* a[] = {bp, &c4};
     if ((st = launch(K.km.k_stage1, K.g_finish, cells, 0, a, KK_STAGE1))) return st;
   }
   for (int i = type_a ? 1 : 2; i <= s; ++i) {
@@ -203,7 +204,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     }
     if (j == 1 && !type_a) need |= 2u;                     // D0 . u^n (= D0 . u^(1)) enters every right-hand side
     if (j >= 1) {
-      void* a[] = {&bp, &j, &need, &weno_eps};
+      void* a[] = {bp, &j, &need, &weno_eps};
       if ((K.stencil_kinds & STENCIL_WHOLE) && (st = launch(K.ks.k_explicit, K.g_explicit, blk, K.ks.smem_explicit, a, KK_EXPLICIT))) return st;
       if ((K.stencil_kinds & STENCIL_SPLIT) &&
           (st = launch(K.ks.k_explicit_split, K.g_explicit_split, blk, K.ks.smem_explicit_split, a, KK_EXPLICIT)))
@@ -218,7 +219,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     double sign = -1.0;   // theta-history term with a minus sign (the stage equations of Sec. 3.1)
     int first = (i == (type_a ? 1 : 2)) ? 1 : 0;           // the first right-hand side also sums theta^n
     {
-      void* a[] = {&bp, &i, &sign, &first};
+      void* a[] = {bp, &i, &sign, &first};
       int terms = 1;   // D_0 . u^n, and three planes of every earlier stage with a_ij
       for (int k = 1; k < i; ++k) terms += AIM(i, k) != 0.0 ? 3 : 0;
       const void* fn = K.ks.k_rhs[terms == 1 ? 0 : (terms == 4 ? 1 : 2)];
@@ -226,8 +227,8 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     }
     {
       // each pass: the power-of-two kernel and/or the Bluestein kernel, as the batch needs
-      void* a[] = {&bp};
-      void* b[] = {&bp, &i};
+      void* a[] = {bp};
+      void* b[] = {bp, &i};
       const unsigned kk = K.fft_kinds;
       if ((kk & FFT_X_POW2) && (st = launch(K.km.k_rows_fwd, K.g_rows, dim3(K.km.rows_threads), K.fft_smem, a, KK_ROWS_FWD))) return st;
       if ((kk & FFT_X_BS) && (st = launch(K.km.k_rows_fwd_bs, K.g_fft, dim3(256), K.fft_smem, a, KK_ROWS_FWD))) return st;
@@ -238,7 +239,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     }
     {
       int close = (fused && i == s) ? 1 : 0;
-      void* a[] = {&bp, &i, &weno_eps, &close, &form};
+      void* a[] = {bp, &i, &weno_eps, &close, &form};
       if ((K.stencil_kinds & STENCIL_WHOLE) && (st = launch(K.ks.k_update, K.g_update, blk, K.smem_update, a, KK_UPDATE))) return st;
       if ((K.stencil_kinds & STENCIL_SPLIT) &&
           (st = launch(K.ks.k_update_split, K.g_update_split, blk, K.smem_update_split, a, KK_UPDATE)))
@@ -255,7 +256,7 @@ int enqueue_imex_step(const ap_dvm_params& t, const StepKernels& K, BatchDev* bp
     }
   }
   if (fused) return 0;
-  void* a[] = {&bp, &form};
+  void* a[] = {bp, &form};
   return launch(K.km.k_finish, K.g_finish, cells, 0, a, KK_FINISH);
 }
 
