@@ -45,7 +45,7 @@ struct StencilSet {
   const void* k_update_split;
   size_t smem_explicit_split, update_fixed_split;
   int nbuf_split;
-  // FP32 WENO5: by marching warps (null otherwise).  Explicit: [terms of v read from memory: 1, 2, up to
+  // FP32: by marching warps (null otherwise).  Explicit: [terms of v read from memory: 1, 2, up to
   // 5][bit 0: E, bit 1: D_LF . B(v)]; update: [(stages in the partner, earlier stages in the sums):
   // (1, 0), (2, 1), up to (3, 3)]
   const void* k_explicit_march[3][4];

@@ -1,16 +1,17 @@
-// The FP32 WENO5 explicit and update kernels for large grids, by marching warps.
+// The FP32 explicit and update kernels for large grids, by marching warps.
 //
 // A warp takes MARCH_OUT columns (its 32 lanes hold them and 3 halo columns on each side) and a
 // segment of rows, and walks down the rows: the fluxes along y come from a register window of six
 // rows, each interface evaluated once, those along x from the neighbouring lanes by shuffles.
 // No shared memory, no barrier, no staged halo; a row is read once per warp (the 6 halo
 // columns and rows again by the neighbours, from L1 and L2).  Same flux arithmetic as the
-// tile kernels (w5_rec_f32).
+// tile kernels (w5_rec_f32, weno3, LF1); the narrower schemes keep the same window and columns.
 //
-// What bounds the tile kernels here is the instruction issue (60 % active) and the latency
+// What bounds the tile kernels here (figures of WENO5) is the instruction issue (60 % active) and the latency
 // of their phases: 1314 (explicit) and 1463 (update) thread instructions per cell, half of
 // them not flux arithmetic (indices, staging, the runs' overlap).  2048^2, ms per step: explicit
-// 0.359 -> 0.235, update 0.458 -> 0.254.  What the closed forms read beside the window is loaded at
+// 0.359 -> 0.235, update 0.458 -> 0.254 (WENO3 0.399 -> 0.240 and 0.489 -> 0.224, LF1 0.261 -> 0.184 and
+// 0.343 -> 0.199).  What the closed forms read beside the window is loaded at
 // the head of a row, before its fluxes: with those loads where they are used (and their pointers
 // read from the descriptor each row) 0.295 and 0.456.  Measured choices: explicit 3 blocks per SM
 // and 3 rows per loop body 0.235 (1 row 0.240, 6 rows 0.273, 4 blocks 0.241, 5 blocks 0.39);
@@ -61,8 +62,19 @@ __device__ __forceinline__ float march_curv(float a, float b, float c, float ew4
   return fmaf(13.f / 3.f * d, d, ew4);
 }
 
-// Curvature terms of one pair along y: of g+ at window rows 1, 2, 3 and of g- at rows 2, 3, 4.
+// One pair (g, U) along y, in the window's rows: its flux at the interface between rows 2 and 3.
+// WENO5 carries the curvature terms, of g+ at rows 1, 2, 3 and of g- at rows 2, 3, 4, from row to row.
+template <int SCHEME>
 struct MarchPair {
+  __device__ __forceinline__ void init(const float*, const float*, float) {}
+  __device__ __forceinline__ void next(const float*, const float*, float) {}
+  __device__ __forceinline__ float flux(const float* g, const float* u, float ew4) const {
+    if (SCHEME == LF1_C2) return 0.5f * (g[2] + g[3] - (u[3] - u[2]));
+    return weno3<float>(g[1] + u[1], g[2] + u[2], g[3] + u[3], ew4) + weno3<float>(g[4] - u[4], g[3] - u[3], g[2] - u[2], ew4);
+  }
+};
+template <>
+struct MarchPair<WENO5_C4> {
   float p[3], m[3];
   __device__ __forceinline__ void init(const float* g, const float* u, float ew4) {
 #pragma unroll
@@ -80,37 +92,54 @@ struct MarchPair {
     m[1] = m[2];
     m[2] = march_curv(g[3] - u[3], g[4] - u[4], g[5] - u[5], ew4);
   }
-  // flux at the interface between window rows 2 and 3
-  __device__ __forceinline__ float flux(const float* g, const float* u) const {
+  __device__ __forceinline__ float flux(const float* g, const float* u, float) const {
     return w5_rec_f32(g[0] + u[0], g[1] + u[1], g[2] + u[2], g[3] + u[3], g[4] + u[4], p[0], p[1], p[2]) +
            w5_rec_f32(g[5] - u[5], g[4] - u[4], g[3] - u[3], g[2] - u[2], g[1] - u[1], m[2], m[1], m[0]);
   }
 };
 
 // Difference of the x fluxes at this lane's cell (its right interface minus its left one).
+template <int SCHEME>
 __device__ __forceinline__ float march_dx(float g, float u, float ew4) {
-  const float P = g + u, M = g - u;
-  const float pa = lane_up(P, 2), pb = lane_up(P, 1), pd = lane_dn(P, 1), pe = lane_dn(P, 2);
-  const float cp = march_curv(pb, P, pd, ew4);
-  const float l = w5_rec_f32(pa, pb, P, pd, pe, lane_up(cp, 1), cp, lane_dn(cp, 1));
-  const float ma = lane_up(M, 1), mc = lane_dn(M, 1), md = lane_dn(M, 2), me = lane_dn(M, 3);
-  const float cm = march_curv(ma, M, mc, ew4);
-  const float f = l + w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm);
+  float f;
+  if constexpr (SCHEME == LF1_C2) {
+    f = 0.5f * (g + lane_dn(g, 1) - (lane_dn(u, 1) - u));
+  } else {
+    const float P = g + u, M = g - u;
+    const float pb = lane_up(P, 1), pd = lane_dn(P, 1), mc = lane_dn(M, 1), md = lane_dn(M, 2);
+    if constexpr (SCHEME == WENO3_C4) {
+      f = weno3<float>(pb, P, pd, ew4) + weno3<float>(md, mc, M, ew4);
+    } else {
+      const float pa = lane_up(P, 2), pe = lane_dn(P, 2);
+      const float cp = march_curv(pb, P, pd, ew4);
+      const float l = w5_rec_f32(pa, pb, P, pd, pe, lane_up(cp, 1), cp, lane_dn(cp, 1));
+      const float ma = lane_up(M, 1), me = lane_dn(M, 3);
+      const float cm = march_curv(ma, M, mc, ew4);
+      f = l + w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm);
+    }
+  }
   return f - lane_up(f, 1);
 }
 
-// Fourth-order central differences, first and second, along x (lanes) and along y (window rows 0 .. 4),
-// without 1/(12 h) and 1/(12 h^2).
+// The scheme's central differences, first and second, along x (lanes) and along y (window rows 0 .. 4),
+// without their scales d1_scale and d2_scale.
+template <int SCHEME>
 __device__ __forceinline__ float march_c1(float am2, float am1, float ap1, float ap2) {
+  if (SCHEME == LF1_C2) return ap1 - am1;
   return fmaf(8.f, ap1 - am1, am2 - ap2);
 }
+template <int SCHEME>
 __device__ __forceinline__ float march_c2(float am2, float am1, float a, float ap1, float ap2) {
+  if (SCHEME == LF1_C2) return fmaf(-2.f, a, ap1 + am1);
   return fmaf(-30.f, a, fmaf(16.f, ap1 + am1, -(ap2 + am2)));
 }
+template <int SCHEME>
 __device__ __forceinline__ float march_c1x(float a) {
-  return march_c1(lane_up(a, 2), lane_up(a, 1), lane_dn(a, 1), lane_dn(a, 2));
+  if (SCHEME == LF1_C2) return march_c1<SCHEME>(0.f, lane_up(a, 1), lane_dn(a, 1), 0.f);
+  return march_c1<SCHEME>(lane_up(a, 2), lane_up(a, 1), lane_dn(a, 1), lane_dn(a, 2));
 }
-__device__ __forceinline__ float march_c1y(const float* w) { return march_c1(w[0], w[1], w[3], w[4]); }
+template <int SCHEME>
+__device__ __forceinline__ float march_c1y(const float* w) { return march_c1<SCHEME>(w[0], w[1], w[3], w[4]); }
 
 __device__ __forceinline__ void march_push(float* w, float v) {
 #pragma unroll
@@ -154,13 +183,13 @@ struct MarchTerms {
 // k_explicit (stencil_kernels.cuh) for stage j; E and B: whether its E^(j) and its
 // D_LF . B(v^(j)) + D_0 theta^(j) are needed; NT: terms of v^(j+1) read from memory
 // (v^n and the earlier stages' E and v; 5: up to that many).
-template <bool E, bool B, int NT>
+template <int SCHEME, bool E, bool B, int NT>
 __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_march(const __grid_constant__ BatchDev b, int j, unsigned need,
                                                                                   double weno_eps) {
   grid_dependency();
   const int lane = threadIdx.x & 31;
   const int ntasks = b.march_start[0][b.counts[3]];
-  const float ew4 = 16.f * float(weno_eps);
+  const float ew4 = (SCHEME == WENO5_C4 ? 16.f : 4.f) * float(weno_eps);   // of the doubled split
   const int i = j + 1;
   const bool curE = has(b.m_ex[i], j), curV = has(b.m_im[i], j);
   for (int task = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5); task < ntasks; task += gridDim.x * MARCH_WARPS) {
@@ -174,7 +203,8 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
     const bool out = lane >= 3 && lane < 3 + MARCH_OUT && xs < nx;
     const float* X = reinterpret_cast<const float*>(I.Xs[j]);
     const float* base = reinterpret_cast<const float*>(I.X);
-    const float cx = K.cdx, cy = K.cdy, fx = flux_scale<float, WENO5_C4>(K.inv_dx), fy = flux_scale<float, WENO5_C4>(K.inv_dy);
+    const float cx = SCHEME == LF1_C2 ? 0.5f * K.inv_dx : K.cdx, cy = SCHEME == LF1_C2 ? 0.5f * K.inv_dy : K.cdy;
+    const float fx = flux_scale<float, SCHEME>(K.inv_dx), fy = flux_scale<float, SCHEME>(K.inv_dy);
     const float qt = K.qtau, te2 = K.te2;
     MarchTerms<NT, (NT > 2)> tm;
     tm.add(base, base + 3 * (size_t)pl, K.r_n[i], I.k32lo.r_n[i]);
@@ -204,7 +234,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
       th[k] = q[k] = 0.f;
       load(t.y0 - 3 + k, u1[k], u2[k], th[k], v1[k], v2[k], q[k]);
     }
-    MarchPair a, bu, bv;   // along y: (q;v2), (v2;u1), (v1;u2)
+    MarchPair<SCHEME> a, bu, bv;   // along y: (q;v2), (v2;u1), (v1;u2)
     if (E) a.init(q, v2, ew4);
     if (B) {
       bu.init(v2, u1, ew4);
@@ -227,14 +257,14 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
           x2[k] = p[pl];
         }
       }
-      const float gq = E ? a.flux(q, v2) : 0.f, gu = B ? bu.flux(v2, u1) : 0.f, gv = B ? bv.flux(v1, u2) : 0.f;
+      const float gq = E ? a.flux(q, v2, ew4) : 0.f, gu = B ? bu.flux(v2, u1, ew4) : 0.f, gv = B ? bv.flux(v1, u2, ew4) : 0.f;
       if (r >= t.y0) {
         float e1 = 0.f, e2 = 0.f;
-        const float u1x = march_c1x(u1[2]), u2y = march_c1y(u2);
+        const float u1x = march_c1x<SCHEME>(u1[2]), u2y = march_c1y<SCHEME>(u2);
         if ((need & NEED_DU) && out) oDu[o] = fmaf(cx, u1x, cy * u2y);
         if (E) {
-          const float u2x = march_c1x(u2[2]), u1y = march_c1y(u1);
-          const float g1 = march_dx(q[2], v1[2], ew4) * fx, g2 = (gq - fq) * fy;
+          const float u2x = march_c1x<SCHEME>(u2[2]), u1y = march_c1y<SCHEME>(u1);
+          const float g1 = march_dx<SCHEME>(q[2], v1[2], ew4) * fx, g2 = (gq - fq) * fy;
           const float a1 = u1[2], a2 = u2[2];
           const float f1 = 0.5f * (a2 * a2 - a1 * a1), f2 = a1 * a2;
           e1 = qt * (cy * u2y - cx * u1x) + te2 * g1 - f1;
@@ -245,14 +275,14 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
           }
         }
         if (need & NEED_LTH) {
-          const float lx = march_c2(lane_up(th[2], 2), lane_up(th[2], 1), th[2], lane_dn(th[2], 1), lane_dn(th[2], 2));
-          const float ly = march_c2(th[0], th[1], th[2], th[3], th[4]);
-          if (out) oL[o] = fmaf(K.ldx, lx, K.ldy * ly);
+          const float lx = march_c2<SCHEME>(lane_up(th[2], 2), lane_up(th[2], 1), th[2], lane_dn(th[2], 1), lane_dn(th[2], 2));
+          const float ly = march_c2<SCHEME>(th[0], th[1], th[2], th[3], th[4]);
+          if (out) oL[o] = fmaf(d2_scale<float, SCHEME>(K.inv_dx), lx, d2_scale<float, SCHEME>(K.inv_dy) * ly);
         }
         if (B) {
-          const float d1 = march_dx(-v1[2], u1[2], ew4) * fx + (gu - fu) * fy;
-          const float d2 = march_dx(v2[2], u2[2], ew4) * fx + (gv - fv) * fy;
-          const float t1 = march_c1x(th[2]), t2 = march_c1y(th);
+          const float d1 = march_dx<SCHEME>(-v1[2], u1[2], ew4) * fx + (gu - fu) * fy;
+          const float d2 = march_dx<SCHEME>(v2[2], u2[2], ew4) * fx + (gv - fv) * fy;
+          const float t1 = march_c1x<SCHEME>(th[2]), t2 = march_c1y<SCHEME>(th);
           if (out) {
             oB[o] = fmaf(cx, t1, d1);
             oB[o + (size_t)pl] = fmaf(cy, t2, d2);
@@ -304,7 +334,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
 // ---------------------------------------------------------------------------
 // k_update (stencil_kernels.cuh) for stage i.  NW: stages in the dissipation partner, NT: earlier
 // stages in the sums of steps 3 and 4 (NT = 3: up to NW and NT of them).
-template <int NW, int NT>
+template <int SCHEME, int NW, int NT>
 __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_march(const __grid_constant__ BatchDev b, int i, double weno_eps,
                                                                                 int close_step, int form) {
   grid_dependency();
@@ -312,7 +342,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
   constexpr int MT = NT > 0 ? NT : 1;
   const int lane = threadIdx.x & 31;
   const int ntasks = b.march_start[1][b.counts[3]];
-  const float ew4 = 16.f * float(weno_eps);
+  const float ew4 = (SCHEME == WENO5_C4 ? 16.f : 4.f) * float(weno_eps);   // of the doubled split
   const unsigned mwp = b.m_wp[i], mim = b.m_im[i];
   for (int task = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5); task < ntasks; task += gridDim.x * MARCH_WARPS) {
     const MarchTask t = march_task(b, 1, task);
@@ -323,7 +353,8 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
     const int xs = t.x0 + lane - 3;
     const int x = xs < 0 ? xs + nx : xs % nx;
     const bool out = lane >= 3 && lane < 3 + MARCH_OUT && xs < nx;
-    const float cx = K.cdx, cy = K.cdy, fx = flux_scale<float, WENO5_C4>(K.inv_dx), fy = flux_scale<float, WENO5_C4>(K.inv_dy);
+    const float cx = SCHEME == LF1_C2 ? 0.5f * K.inv_dx : K.cdx, cy = SCHEME == LF1_C2 ? 0.5f * K.inv_dy : K.cdy;
+    const float fx = flux_scale<float, SCHEME>(K.inv_dx), fy = flux_scale<float, SCHEME>(K.inv_dy);
     const float dt = K.dt, aii = K.aim[i][i], rn = K.r_n[i], rnl = I.k32lo.r_n[i], rd = K.rq_d[i][i], rdl = I.k32lo.rq_d[i][i];
     const bool pairs = I.relax64 != 0;
     float* Xi = reinterpret_cast<float*>(I.Xs[i]);
@@ -370,7 +401,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
       p1[k] = partner(f);
       p2[k] = partner(g);
     }
-    MarchPair a, c;   // along y: (v2;p1), (v1;p2)
+    MarchPair<SCHEME> a, c;   // along y: (v2;p1), (v1;p2)
     a.init(v2, p1, ew4);
     c.init(v1, p2, ew4);
     float fa = 0.f, fc = 0.f;
@@ -399,12 +430,12 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
             xq[k] = base[(ptrdiff_t)(tq.off[k] + o)];
           }
       }
-      const float ga = a.flux(v2, p1), gc = c.flux(v1, p2);
+      const float ga = a.flux(v2, p1, ew4), gc = c.flux(v1, p2, ew4);
       if (r >= t.y0) {
-        const float d1 = march_dx(-v1[2], p1[2], ew4) * fx + (ga - fa) * fy;
-        const float d2 = march_dx(v2[2], p2[2], ew4) * fx + (gc - fc) * fy;
-        const float t1 = march_c1x(th[2]), t2 = march_c1y(th);
-        const float dvi = fmaf(cx, march_c1x(v1[2]), cy * march_c1y(v2));
+        const float d1 = march_dx<SCHEME>(-v1[2], p1[2], ew4) * fx + (ga - fa) * fy;
+        const float d2 = march_dx<SCHEME>(v2[2], p2[2], ew4) * fx + (gc - fc) * fy;
+        const float t1 = march_c1x<SCHEME>(th[2]), t2 = march_c1y<SCHEME>(th);
+        const float dvi = fmaf(cx, march_c1x<SCHEME>(v1[2]), cy * march_c1y<SCHEME>(v2));
         if (out) {
           // step 3
           float s1 = 0.f, s2 = 0.f;

@@ -96,15 +96,15 @@ inline bool split_fluxes(const ap_dvm_params& p) {
   return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;
 }
 
-// Whether a solve is taken by the marching kernels: FP32 WENO5, enough cells for their warps (each holds
+// Whether a solve is taken by the marching kernels: FP32, enough cells for their warps (each holds
 // a row of 26 columns) to fill the chip, and a width that does not leave over a quarter of their
-// columns beyond the grid.  Explicit + update, us per step, marching against tiles: 256^2 57 and 48,
-// 320^2 62 and 54, 384^2 61 and 65, 512^2 69 and 81, 1024^2 148 and 227, 2048^2 489 and 817,
-// 4096^2 1787 and 3165.  A property of the solve alone, so that a batch does not change its result.
+// columns beyond the grid.  Explicit + update, us per step, marching against tiles: WENO5 256^2 54 and
+// 45, 384^2 58 and 61, 512^2 66 and 78, 1024^2 147 and 216, 2048^2 477 and 774; WENO3 56 and 51, 59 and
+// 68, 66 and 85, 141 and 240, 464 and 888; LF1 47 and 41, 49 and 55, 52 and 65, 110 and 169, 383 and 605.  A property of the solve alone, so that a batch does not change its result.
 constexpr long long kMarchMinCells = 384LL * 384;
 inline bool marching(const ap_dvm_params& p) {
   const int covered = (p.nx + MARCH_OUT - 1) / MARCH_OUT * MARCH_OUT;
-  return p.precision != AP_DVM_FP64 && p.space_scheme == AP_DVM_WENO5_C4 && (long long)p.nx * p.ny >= kMarchMinCells &&
+  return p.precision != AP_DVM_FP64 && (long long)p.nx * p.ny >= kMarchMinCells &&
          4LL * covered <= 5LL * p.nx;
 }
 inline unsigned stencil_kind(const ap_dvm_params& p) {

@@ -1,6 +1,6 @@
-"""FP32 WENO5 solves of at least 384 x 384 cells are taken by the marching kernels: against the
+"""FP32 solves of at least 384 x 384 cells are taken by the marching kernels: against the
 oracle at column counts about multiples of a warp's 26, ragged row segments, every tableau
-form (stored terms: the second-order tableau's and the general ones), with and without the
+form (stored terms: the second-order tableau's and the general ones), every scheme, with and without the
 relaxation in pairs, and in a batch beside solves of the tile kernels."""
 import math
 
@@ -16,15 +16,16 @@ pytestmark = pytest.mark.gpu
 TABS = {"gsa2": tableaux.gsa2, "euler": tableaux.euler, "type_a3": tableaux.type_a3, "ars4": tableaux.ars4}
 
 
-def _setup(nx, ny, tab, eps, prec=api.FP32_DEV):
+def _setup(nx, ny, tab, eps, prec=api.FP32_DEV, scheme="WENO5_C4"):
     A_ex, A_im = TABS[tab]()
     X, Y = W.cell_centres(nx, ny)
     u1 = np.sin(X + 0.3) * np.cos(2 * Y) + 0.3 * np.cos(3 * Y + 0.1)
     u2 = -0.5 * np.cos(X + 0.3) * np.sin(2 * Y) + 0.2 * np.sin(2 * X)
     X0 = O.equilibrium_state(u1, u2, 0.25 * np.cos(X + Y))
     dt = W.stable_dt(u1, u2, 2 * math.pi / max(nx, ny), 0.05)
-    p = api.default_params(nx, ny, eps=eps, dt=dt, tau=0.05, mach=1e-2, tableau=(A_ex, A_im), precision=prec)
-    return X0, p, O.Params(nx, ny, eps, 0.05, dt, np.array(A_ex), np.array(A_im), scheme="WENO5_C4")
+    p = api.default_params(nx, ny, eps=eps, dt=dt, tau=0.05, mach=1e-2, tableau=(A_ex, A_im), precision=prec,
+                           space_scheme=scheme)
+    return X0, p, O.Params(nx, ny, eps, 0.05, dt, np.array(A_ex), np.array(A_im), scheme=scheme)
 
 
 def _run(X0, p, steps, graph=0):
@@ -53,6 +54,13 @@ def _check(X0, p, o, eps, steps=2, graph=0):
 @pytest.mark.parametrize("nx,ny", [(384, 384), (390, 384), (391, 400), (416, 355), (509, 291), (1000, 150), (156, 1001), (2048, 73)])
 def test_sizes(nx, ny):
     X0, p, o = _setup(nx, ny, "gsa2", 0.5)
+    _check(X0, p, o, 0.5)
+
+
+@pytest.mark.parametrize("scheme", ["LF1_C2", "WENO3_C4"])
+@pytest.mark.parametrize("nx,ny,tab", [(390, 384, "gsa2"), (509, 291, "gsa2"), (391, 400, "ars4")])
+def test_schemes(nx, ny, tab, scheme):
+    X0, p, o = _setup(nx, ny, tab, 0.5, scheme=scheme)
     _check(X0, p, o, 0.5)
 
 
