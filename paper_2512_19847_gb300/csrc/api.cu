@@ -252,12 +252,21 @@ unsigned fft_kinds_of(const ap_dvm_handle* h) {
   return k;
 }
 
+// Whether the attached solves together fill the chip with marching warps (stencil_kind).
+bool march_all(const ap_dvm_handle* h) {
+  long long cells = 0;
+  for (const Slot& s : h->slots)
+    if (s.attached && march_wide(s.p)) cells += (long long)s.p.nx * s.p.ny;
+  return cells >= kMarchMinBatchCells;
+}
+
 // StencilKinds of the attached solves (of the template while none is attached).
 unsigned stencil_kinds_of(const ap_dvm_handle* h) {
   unsigned k = 0;
+  const bool all = march_all(h);
   for (const Slot& s : h->slots)
-    if (s.attached) k |= stencil_kind(s.p);
-  return k ? k : stencil_kind(h->tmpl);
+    if (s.attached) k |= stencil_kind(s.p, all);
+  return k ? k : stencil_kind(h->tmpl, false);
 }
 
 int auto_tile(const ap_dvm_handle* h) {
@@ -347,7 +356,7 @@ ap_dvm_status prepare_kernels(ap_dvm_handle* h) {
 
 // Rows per task of the marching kernels: the fewest rounds of tasks over the resident warps, a
 // task's start-up (the window's rows and curvature terms) counted as 5 rows.
-int march_rows(const std::vector<Slot*>& order, int grid) {
+int march_rows(const std::vector<Slot*>& order, bool all, int grid) {
   static constexpr int kRows[] = {8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 72, 80, 96, 112, 128};
   const long long warps = 4LL * std::max(1, grid);
   int best = 0;
@@ -355,7 +364,7 @@ int march_rows(const std::vector<Slot*>& order, int grid) {
   for (int rows : kRows) {
     long long tasks = 0;
     for (const Slot* s : order)
-      if (marching(s->p)) tasks += march_tasks(s->p.nx, s->p.ny, rows);
+      if (stencil_kind(s->p, all) == STENCIL_MARCH) tasks += march_tasks(s->p.nx, s->p.ny, rows);
     const long long cost = (tasks + warps - 1) / warps * (rows + 5);
     if (!best || cost < best_cost) { best = rows; best_cost = cost; }
   }
@@ -374,6 +383,7 @@ ap_dvm_status flush(ap_dvm_handle* h) {
   const int TX = h->ks.tx, TY = h->ks.ty;
   const unsigned kinds = fft_kinds_of(h);
   const unsigned skinds = stencil_kinds_of(h);
+  const bool all = march_all(h);
   if (kinds != h->fft_kinds || skinds != h->stencil_kinds) {   // the launch sequence changed
     h->fft_kinds = kinds;
     h->stencil_kinds = skinds;
@@ -403,11 +413,11 @@ ap_dvm_status flush(ap_dvm_handle* h) {
   std::vector<Slot*> order;
   for (int other = 0; other < 2; ++other)
     for (Slot& s : h->slots)
-      if (s.attached && !s.paused && (stencil_kind(s.p) != STENCIL_WHOLE) == (other != 0)) order.push_back(&s);
+      if (s.attached && !s.paused && (stencil_kind(s.p, all) != STENCIL_WHOLE) == (other != 0)) order.push_back(&s);
   h->up_counts[5] = 0;
   for (int m = 0; m < 2; ++m) {
     h->up_march[m].assign(1, 0);
-    h->up_counts[6 + m] = march_rows(order, m ? h->grid_update_march : h->grid_explicit_march);
+    h->up_counts[6 + m] = march_rows(order, all, m ? h->grid_update_march : h->grid_explicit_march);
   }
   for (Slot* sp : order) {
     Slot& s = *sp;
@@ -437,9 +447,9 @@ ap_dvm_status flush(ap_dvm_handle* h) {
       h->up_inst[par].push_back(v);
     }
     h->up_tiles.push_back(h->up_tiles.back() + d.tiles_x * d.tiles_y);
-    if (stencil_kind(s.p) == STENCIL_WHOLE) h->up_counts[5] = h->up_tiles.back();
+    if (stencil_kind(s.p, all) == STENCIL_WHOLE) h->up_counts[5] = h->up_tiles.back();
     for (int m = 0; m < 2; ++m)
-      h->up_march[m].push_back(h->up_march[m].back() + (marching(s.p) ? march_tasks(s.p.nx, s.p.ny, h->up_counts[6 + m]) : 0));
+      h->up_march[m].push_back(h->up_march[m].back() + (stencil_kind(s.p, all) == STENCIL_MARCH ? march_tasks(s.p.nx, s.p.ny, h->up_counts[6 + m]) : 0));
     h->up_rows.push_back(h->up_rows.back() + (pairs + d.row_pairs - 1) / d.row_pairs);
     h->up_rhs.push_back(h->up_rhs.back() + rhs_items(s.p.nx, s.p.ny, h->f32));
     h->up_cols.push_back(h->up_cols.back() + (s.p.nx / 2 + 1 + d.col_group - 1) / d.col_group);

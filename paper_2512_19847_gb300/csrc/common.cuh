@@ -194,31 +194,21 @@ __device__ __forceinline__ bool has(unsigned mask, int j) { return (mask >> j) &
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T weno3(T a, T b, T c, T ew) {
-  const T p0 = (T(3) * b - a) * T(0.5);
+  const T p0 = fma(T(3), b, -a) * T(0.5);
   const T p1 = (b + c) * T(0.5);
-  T s0 = ew + (b - a) * (b - a); s0 *= s0;
-  T s1 = ew + (c - b) * (c - b); s1 *= s1;
+  T s0 = fma(b - a, b - a, ew); s0 *= s0;
+  T s1 = fma(c - b, c - b, ew); s1 *= s1;
   const T w0 = T(1.0 / 3.0) * s1;
   const T w1 = T(2.0 / 3.0) * s0;
-  return (w0 * p0 + w1 * p1) / (w0 + w1);
+  return fma(w0, p0, w1 * p1) / (w0 + w1);
 }
 
-// Central first difference (Sec. 3.2 D_0; fourth order under the WENO schemes)
-// along a line with stride st, times 1/h.
-template <typename T, int SCHEME>
-__device__ __forceinline__ T cdiff(const T* f, int st, T inv_h) {
-  if (SCHEME == LF1_C2) return (f[st] - f[-st]) * (T(0.5) * inv_h);
-  return (-f[2 * st] + T(8) * f[st] - T(8) * f[-st] + f[-2 * st]) * (inv_h * T(1.0 / 12.0));
-}
+// a + b, never contracted with a product that formed either.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
-// Central second difference along a line, times 1/h^2 (compact 3-point or 5-point).
-template <typename T, int SCHEME>
-__device__ __forceinline__ T cdiff2(const T* f, int st, T inv_h2) {
-  if (SCHEME == LF1_C2) return (f[st] - T(2) * f[0] + f[-st]) * inv_h2;
-  return (-f[2 * st] + T(16) * f[st] - T(30) * f[0] + T(16) * f[-st] - f[-2 * st]) * (inv_h2 * T(1.0 / 12.0));
-}
-
-// The same two differences from the values at offsets -2 .. 2 along a line, without
+// Central first and second differences (Sec. 3.2 D_0 and the compact second difference; fourth order
+// under the WENO schemes) from the values at offsets -2 .. 2 along a line, without
 // their scale (fm2 and fp2 unused by the second-order scheme) and, the second, without its centre
 // value: the first difference is d1_scale(inv_h) * d1_sum(...), the second
 // d2_scale(inv_h) * (d2_sum(...) + d2_centre() * f0).

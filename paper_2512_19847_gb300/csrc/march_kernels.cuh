@@ -69,8 +69,8 @@ struct MarchPair {
   __device__ __forceinline__ void init(const float*, const float*, float) {}
   __device__ __forceinline__ void next(const float*, const float*, float) {}
   __device__ __forceinline__ float flux(const float* g, const float* u, float ew4) const {
-    if (SCHEME == LF1_C2) return 0.5f * (g[2] + g[3] - (u[3] - u[2]));
-    return weno3<float>(g[1] + u[1], g[2] + u[2], g[3] + u[3], ew4) + weno3<float>(g[4] - u[4], g[3] - u[3], g[2] - u[2], ew4);
+    if (SCHEME == LF1_C2) return cell_lf1(g[2], g[3], u[2], u[3]);
+    return add_rn(weno3<float>(g[1] + u[1], g[2] + u[2], g[3] + u[3], ew4), weno3<float>(g[4] - u[4], g[3] - u[3], g[2] - u[2], ew4));
   }
 };
 template <>
@@ -93,8 +93,8 @@ struct MarchPair<WENO5_C4> {
     m[2] = march_curv(g[3] - u[3], g[4] - u[4], g[5] - u[5], ew4);
   }
   __device__ __forceinline__ float flux(const float* g, const float* u, float) const {
-    return w5_rec_f32(g[0] + u[0], g[1] + u[1], g[2] + u[2], g[3] + u[3], g[4] + u[4], p[0], p[1], p[2]) +
-           w5_rec_f32(g[5] - u[5], g[4] - u[4], g[3] - u[3], g[2] - u[2], g[1] - u[1], m[2], m[1], m[0]);
+    return add_rn(w5_rec_f32(g[0] + u[0], g[1] + u[1], g[2] + u[2], g[3] + u[3], g[4] + u[4], p[0], p[1], p[2]),
+                  w5_rec_f32(g[5] - u[5], g[4] - u[4], g[3] - u[3], g[2] - u[2], g[1] - u[1], m[2], m[1], m[0]));
   }
 };
 
@@ -103,43 +103,32 @@ template <int SCHEME>
 __device__ __forceinline__ float march_dx(float g, float u, float ew4) {
   float f;
   if constexpr (SCHEME == LF1_C2) {
-    f = 0.5f * (g + lane_dn(g, 1) - (lane_dn(u, 1) - u));
+    f = cell_lf1(g, lane_dn(g, 1), u, lane_dn(u, 1));
   } else {
     const float P = g + u, M = g - u;
     const float pb = lane_up(P, 1), pd = lane_dn(P, 1), mc = lane_dn(M, 1), md = lane_dn(M, 2);
     if constexpr (SCHEME == WENO3_C4) {
-      f = weno3<float>(pb, P, pd, ew4) + weno3<float>(md, mc, M, ew4);
+      f = add_rn(weno3<float>(pb, P, pd, ew4), weno3<float>(md, mc, M, ew4));
     } else {
       const float pa = lane_up(P, 2), pe = lane_dn(P, 2);
       const float cp = march_curv(pb, P, pd, ew4);
       const float l = w5_rec_f32(pa, pb, P, pd, pe, lane_up(cp, 1), cp, lane_dn(cp, 1));
       const float ma = lane_up(M, 1), me = lane_dn(M, 3);
       const float cm = march_curv(ma, M, mc, ew4);
-      f = l + w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm);
+      f = add_rn(l, w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm));
     }
   }
   return f - lane_up(f, 1);
 }
 
-// The scheme's central differences, first and second, along x (lanes) and along y (window rows 0 .. 4),
-// without their scales d1_scale and d2_scale.
-template <int SCHEME>
-__device__ __forceinline__ float march_c1(float am2, float am1, float ap1, float ap2) {
-  if (SCHEME == LF1_C2) return ap1 - am1;
-  return fmaf(8.f, ap1 - am1, am2 - ap2);
-}
-template <int SCHEME>
-__device__ __forceinline__ float march_c2(float am2, float am1, float a, float ap1, float ap2) {
-  if (SCHEME == LF1_C2) return fmaf(-2.f, a, ap1 + am1);
-  return fmaf(-30.f, a, fmaf(16.f, ap1 + am1, -(ap2 + am2)));
-}
+// The scheme's central differences along x (lanes) and along y (window rows 0 .. 4).
 template <int SCHEME>
 __device__ __forceinline__ float march_c1x(float a) {
-  if (SCHEME == LF1_C2) return march_c1<SCHEME>(0.f, lane_up(a, 1), lane_dn(a, 1), 0.f);
-  return march_c1<SCHEME>(lane_up(a, 2), lane_up(a, 1), lane_dn(a, 1), lane_dn(a, 2));
+  if (SCHEME == LF1_C2) return cell_c1<float, SCHEME>(0.f, lane_up(a, 1), lane_dn(a, 1), 0.f);
+  return cell_c1<float, SCHEME>(lane_up(a, 2), lane_up(a, 1), lane_dn(a, 1), lane_dn(a, 2));
 }
 template <int SCHEME>
-__device__ __forceinline__ float march_c1y(const float* w) { return march_c1<SCHEME>(w[0], w[1], w[3], w[4]); }
+__device__ __forceinline__ float march_c1y(const float* w) { return cell_c1<float, SCHEME>(w[0], w[1], w[3], w[4]); }
 
 __device__ __forceinline__ void march_push(float* w, float v) {
 #pragma unroll
@@ -203,7 +192,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
     const bool out = lane >= 3 && lane < 3 + MARCH_OUT && xs < nx;
     const float* X = reinterpret_cast<const float*>(I.Xs[j]);
     const float* base = reinterpret_cast<const float*>(I.X);
-    const float cx = SCHEME == LF1_C2 ? 0.5f * K.inv_dx : K.cdx, cy = SCHEME == LF1_C2 ? 0.5f * K.inv_dy : K.cdy;
+    const float cx = c1_scale<SCHEME>(K.inv_dx, K.cdx), cy = c1_scale<SCHEME>(K.inv_dy, K.cdy);
     const float fx = flux_scale<float, SCHEME>(K.inv_dx), fy = flux_scale<float, SCHEME>(K.inv_dy);
     const float qt = K.qtau, te2 = K.te2;
     MarchTerms<NT, (NT > 2)> tm;
@@ -261,27 +250,24 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_E) k_explicit_ma
       if (r >= t.y0) {
         float e1 = 0.f, e2 = 0.f;
         const float u1x = march_c1x<SCHEME>(u1[2]), u2y = march_c1y<SCHEME>(u2);
-        if ((need & NEED_DU) && out) oDu[o] = fmaf(cx, u1x, cy * u2y);
+        if ((need & NEED_DU) && out) oDu[o] = cell_sum(cx, u1x, cy, u2y);
         if (E) {
           const float u2x = march_c1x<SCHEME>(u2[2]), u1y = march_c1y<SCHEME>(u1);
           const float g1 = march_dx<SCHEME>(q[2], v1[2], ew4) * fx, g2 = (gq - fq) * fy;
-          const float a1 = u1[2], a2 = u2[2];
-          const float f1 = 0.5f * (a2 * a2 - a1 * a1), f2 = a1 * a2;
-          e1 = qt * (cy * u2y - cx * u1x) + te2 * g1 - f1;
-          e2 = qt * (cx * u2x + cy * u1y) + te2 * g2 - f2;
+          cell_e<float>(qt, te2, cx, cy, u1x, u2y, u2x, u1y, g1, g2, u1[2], u2[2], e1, e2);
           if (out) {
             oE[o] = e1;
             oE[o + (size_t)pl] = e2;
           }
         }
         if (need & NEED_LTH) {
-          const float lx = march_c2<SCHEME>(lane_up(th[2], 2), lane_up(th[2], 1), th[2], lane_dn(th[2], 1), lane_dn(th[2], 2));
-          const float ly = march_c2<SCHEME>(th[0], th[1], th[2], th[3], th[4]);
-          if (out) oL[o] = fmaf(d2_scale<float, SCHEME>(K.inv_dx), lx, d2_scale<float, SCHEME>(K.inv_dy) * ly);
+          const float lx = cell_c2<float, SCHEME>(lane_up(th[2], 2), lane_up(th[2], 1), th[2], lane_dn(th[2], 1), lane_dn(th[2], 2));
+          const float ly = cell_c2<float, SCHEME>(th[0], th[1], th[2], th[3], th[4]);
+          if (out) oL[o] = cell_sum(d2_scale<float, SCHEME>(K.inv_dx), lx, d2_scale<float, SCHEME>(K.inv_dy), ly);
         }
         if (B) {
-          const float d1 = march_dx<SCHEME>(-v1[2], u1[2], ew4) * fx + (gu - fu) * fy;
-          const float d2 = march_dx<SCHEME>(v2[2], u2[2], ew4) * fx + (gv - fv) * fy;
+          const float d1 = cell_sum(march_dx<SCHEME>(-v1[2], u1[2], ew4), fx, gu - fu, fy);
+          const float d2 = cell_sum(march_dx<SCHEME>(v2[2], u2[2], ew4), fx, gv - fv, fy);
           const float t1 = march_c1x<SCHEME>(th[2]), t2 = march_c1y<SCHEME>(th);
           if (out) {
             oB[o] = fmaf(cx, t1, d1);
@@ -353,7 +339,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
     const int xs = t.x0 + lane - 3;
     const int x = xs < 0 ? xs + nx : xs % nx;
     const bool out = lane >= 3 && lane < 3 + MARCH_OUT && xs < nx;
-    const float cx = SCHEME == LF1_C2 ? 0.5f * K.inv_dx : K.cdx, cy = SCHEME == LF1_C2 ? 0.5f * K.inv_dy : K.cdy;
+    const float cx = c1_scale<SCHEME>(K.inv_dx, K.cdx), cy = c1_scale<SCHEME>(K.inv_dy, K.cdy);
     const float fx = flux_scale<float, SCHEME>(K.inv_dx), fy = flux_scale<float, SCHEME>(K.inv_dy);
     const float dt = K.dt, aii = K.aim[i][i], rn = K.r_n[i], rnl = I.k32lo.r_n[i], rd = K.rq_d[i][i], rdl = I.k32lo.rq_d[i][i];
     const bool pairs = I.relax64 != 0;
@@ -391,7 +377,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
       float s = 0.f;
 #pragma unroll
       for (int k = 0; k < NW; ++k)
-        if (pw.on(k)) s = s + pw.c[k] * f[k];
+        if (pw.on(k)) s = fmaf(pw.c[k], f[k], s);
       return s;
     };
 #pragma unroll
@@ -432,22 +418,22 @@ __global__ void __launch_bounds__(MARCH_THREADS, APD_MARCH_MINB_U) k_update_marc
       }
       const float ga = a.flux(v2, p1, ew4), gc = c.flux(v1, p2, ew4);
       if (r >= t.y0) {
-        const float d1 = march_dx<SCHEME>(-v1[2], p1[2], ew4) * fx + (ga - fa) * fy;
-        const float d2 = march_dx<SCHEME>(v2[2], p2[2], ew4) * fx + (gc - fc) * fy;
+        const float d1 = cell_sum(march_dx<SCHEME>(-v1[2], p1[2], ew4), fx, ga - fa, fy);
+        const float d2 = cell_sum(march_dx<SCHEME>(v2[2], p2[2], ew4), fx, gc - fc, fy);
         const float t1 = march_c1x<SCHEME>(th[2]), t2 = march_c1y<SCHEME>(th);
-        const float dvi = fmaf(cx, march_c1x<SCHEME>(v1[2]), cy * march_c1y<SCHEME>(v2));
+        const float dvi = cell_sum(cx, march_c1x<SCHEME>(v1[2]), cy, march_c1y<SCHEME>(v2));
         if (out) {
           // step 3
           float s1 = 0.f, s2 = 0.f;
 #pragma unroll
           for (int k = 0; k < NT; ++k)
             if (ts.on(k)) {
-              s1 = s1 + ts.c[k] * b1[k];
-              s2 = s2 + ts.c[k] * b2[k];
+              s1 = fmaf(ts.c[k], b1[k], s1);
+              s2 = fmaf(ts.c[k], b2[k], s2);
             }
-          s1 = s1 + aii * fmaf(cx, t1, d1);
-          s2 = s2 + aii * fmaf(cy, t2, d2);
-          const float w1 = n1 - dt * s1, w2 = n2 - dt * s2;
+          s1 = fmaf(aii, fmaf(cx, t1, d1), s1);
+          s2 = fmaf(aii, fmaf(cy, t2, d2), s2);
+          const float w1 = fmaf(-dt, s1, n1), w2 = fmaf(-dt, s2, n2);
           // step 4
           auto step4 = [&](auto sum) {
             sum.start(rn, rnl, n3);

@@ -350,7 +350,7 @@ __device__ __forceinline__ void axis_fluxes(const T* const* g, const T* const* U
       const T sg = ((NEG >> pr) & 1u) ? T(-1) : T(1);
       const T* gp = pick<NP>(g, pr);
       const T* up = pick<NP>(U, pr);
-      out[pr * NL * NI + out_off(line, m)] = T(0.5) * (sg * gp[o0] + sg * gp[o1] - (up[o1] - up[o0]));
+      out[pr * NL * NI + out_off(line, m)] = T(0.5) * ((sg * gp[o0] + sg * gp[o1]) - (up[o1] - up[o0]));
     }
     return;
   }
@@ -376,7 +376,7 @@ __device__ __forceinline__ void axis_fluxes(const T* const* g, const T* const* U
       const T* Pp = split + (4 * pr + 0) * LS + c;
       const T* Mm = split + (4 * pr + 1) * LS + c;
       out[pr * NL * NI + out_off(line, m)] =
-          weno3<T>(Pp[-PS], Pp[0], Pp[PS], T(4) * ew) + weno3<T>(Mm[2 * PS], Mm[PS], Mm[0], T(4) * ew);
+          add_rn(weno3<T>(Pp[-PS], Pp[0], Pp[PS], T(4) * ew), weno3<T>(Mm[2 * PS], Mm[PS], Mm[0], T(4) * ew));
     }
     return;
   }
@@ -433,7 +433,7 @@ __device__ __forceinline__ float w5_rec_f32(float a, float b, float c, float d, 
   const float p1x3 = fmaf(2.5f, c, fmaf(-0.5f, b, d));          // 3 p_1
   const float ta = l0 + l1, tb = 1.5f * (l1 - l2);              // 3 (p_0 - p_1), 9 (p_2 - p_1)
   const float num = fmaf(p1x3, den, fmaf(r0, ta, r2 * tb));     // 30 sum_k d_k r_k p_k
-  return num * rcp_approx(den);
+  return __fmul_rn(num, rcp_approx(den));   // (not contracted with what it is added to: every kernel the same)
 }
 
 // Values of the LF partner U at a staged point: one plane, or the weighted sum of
@@ -451,7 +451,7 @@ struct PlaneSum {
     float r = 0.f;
 #pragma unroll
     for (int m = 0; m < APD_MAXS - 1; ++m)
-      if (m < n) r = r + w[m] * f[m][o];
+      if (m < n) r = fma(w[m], f[m][o], r);
     return r;
   }
 };
@@ -494,7 +494,7 @@ __device__ __forceinline__ void w5_runs_item(const float* g, const UF& U, bool n
     // left-biased reconstruction of g+ (points m..m+4 of the run), mirrored right-biased of g- (points m+5..m+1)
     const float fl = w5_rec_f32(Pp[i], Pp[i + 1], Pp[i + 2], Pp[i + 3], Pp[i + 4], Cp[i + 1], Cp[i + 2], Cp[i + 3]);
     const float fr = w5_rec_f32(Pm[i + 5], Pm[i + 4], Pm[i + 3], Pm[i + 2], Pm[i + 1], Cm[i + 4], Cm[i + 3], Cm[i + 2]);
-    if (NI % KR == 0 || m < NI) out[AX == 0 ? line * NI + m : m * TX + line] = fl + fr;
+    if (NI % KR == 0 || m < NI) out[AX == 0 ? line * NI + m : m * TX + line] = __fadd_rn(fl, fr);
   }
 }
 
@@ -652,7 +652,7 @@ template <bool PAIRS, typename T>
 struct RelaxSum {
   T s;
   __device__ __forceinline__ void start(T c, float, T x) { s = c * x; }
-  __device__ __forceinline__ void add(T c, float, T x) { s = s + c * x; }
+  __device__ __forceinline__ void add(T c, float, T x) { s = fma(c, x, s); }
   __device__ __forceinline__ T value() const { return s; }
 };
 template <>
@@ -726,6 +726,48 @@ __device__ __forceinline__ T flux_scale(T inv_h) {
 }
 
 // ---------------------------------------------------------------------------
+// The per-cell forms of the tile and the marching kernels, with every contraction written out, so that a
+// solve's result does not depend on which of them takes it.
+//
+// The scheme's central differences without their scales (c1_scale, d2_scale), from the values at offsets
+// -2 .. 2 along a line.
+template <typename T, int SCHEME>
+__device__ __forceinline__ T cell_c1(T am2, T am1, T ap1, T ap2) {
+  if (SCHEME == LF1_C2) return ap1 - am1;
+  return fma(T(8), ap1 - am1, am2 - ap2);
+}
+template <typename T, int SCHEME>
+__device__ __forceinline__ T cell_c2(T am2, T am1, T a, T ap1, T ap2) {
+  if (SCHEME == LF1_C2) return fma(T(-2), a, ap1 + am1);
+  return fma(T(-30), a, fma(T(16), ap1 + am1, -(ap2 + am2)));
+}
+template <typename T, int SCHEME>
+__device__ __forceinline__ T tile_c1(const T* f, int st) {
+  if constexpr (SCHEME == LF1_C2) return cell_c1<T, SCHEME>(T(0), f[-st], f[st], T(0));
+  else return cell_c1<T, SCHEME>(f[-2 * st], f[-st], f[st], f[2 * st]);
+}
+template <typename T, int SCHEME>
+__device__ __forceinline__ T tile_c2(const T* f, int st) {
+  if constexpr (SCHEME == LF1_C2) return cell_c2<T, SCHEME>(T(0), f[-st], f[0], f[st], T(0));
+  else return cell_c2<T, SCHEME>(f[-2 * st], f[-st], f[0], f[st], f[2 * st]);
+}
+template <int SCHEME, typename T>
+__device__ __forceinline__ T c1_scale(T inv_h, T inv_12h) { return SCHEME == LF1_C2 ? T(0.5) * inv_h : inv_12h; }
+// x a + y b
+template <typename T>
+__device__ __forceinline__ T cell_sum(T x, T a, T y, T b) { return fma(x, a, y * b); }
+// E at a cell: (tau/4) (sy b - sx a, sx c + sy d) + tau eps^2 (g1, g2) - F(u)
+template <typename T>
+__device__ __forceinline__ void cell_e(T qt, T te2, T sx, T sy, T u1x, T u2y, T u2x, T u1y, T g1, T g2, T a1, T a2, T& e1, T& e2) {
+  const T f1 = T(0.5) * fma(a2, a2, -(a1 * a1)), f2 = a1 * a2;
+  e1 = fma(qt, fma(sy, u2y, -(sx * u1x)), fma(te2, g1, -f1));
+  e2 = fma(qt, fma(sx, u2x, sy * u1y), fma(te2, g2, -f2));
+}
+// Interfaces of a line: the LF1 flux (Sec. 3.2, alpha = 1), and the sum of the two reconstructions.
+template <typename T>
+__device__ __forceinline__ T cell_lf1(T g0, T g1, T u0, T u1) { return T(0.5) * ((g0 + g1) - (u1 - u0)); }
+
+// ---------------------------------------------------------------------------
 template <typename T, int SCHEME, int TX, int TY>
 __global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks<T>(Geo<T, SCHEME, TX, TY>::NT)) k_explicit(const __grid_constant__ BatchDev b, int j, unsigned need, double weno_eps) {
   grid_dependency();
@@ -779,38 +821,35 @@ __global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks
     const int c = G::C00 + ty * BW + tx;
     const size_t o = (size_t)(t.y0 + ty) * nx + (t.x0 + tx);
     T e1 = T(0), e2 = T(0);
-    if (needE) {
-      const T b1 = cdiff<T, SCHEME>(su2 + c, BW, idy) - cdiff<T, SCHEME>(su1 + c, 1, idx);
-      const T b2 = cdiff<T, SCHEME>(su2 + c, 1, idx) + cdiff<T, SCHEME>(su1 + c, BW, idy);
-      const T g1 = (fx[ty * (TX + 1) + tx + 1] - fx[ty * (TX + 1) + tx]) * fidx;
-      const T g2 = (fy[(ty + 1) * TX + tx] - fy[ty * TX + tx]) * fidy;
-      const T a1 = su1[c], a2 = su2[c];
-      const T f1 = T(0.5) * (a2 * a2 - a1 * a1), f2 = a1 * a2;
-      const T qt = K.qtau, te2 = K.te2;
-      e1 = qt * b1 + te2 * g1 - f1;
-      e2 = qt * b2 + te2 * g2 - f2;
-      T* e = reinterpret_cast<T*>(I.E[j]);
-      e[o] = e1;
-      e[o + pl] = e2;
-    }
-    if (need & NEED_DU) {
-      reinterpret_cast<T*>(I.Du[j])[o] = cdiff<T, SCHEME>(su1 + c, 1, idx) + cdiff<T, SCHEME>(su2 + c, BW, idy);
+    const T cx = c1_scale<SCHEME>(idx, K.cdx), cy = c1_scale<SCHEME>(idy, K.cdy);
+    if (needE || (need & NEED_DU)) {
+      const T u1x = tile_c1<T, SCHEME>(su1 + c, 1), u2y = tile_c1<T, SCHEME>(su2 + c, BW);
+      if (need & NEED_DU) reinterpret_cast<T*>(I.Du[j])[o] = cell_sum(cx, u1x, cy, u2y);
+      if (needE) {
+        const T g1 = (fx[ty * (TX + 1) + tx + 1] - fx[ty * (TX + 1) + tx]) * fidx;
+        const T g2 = (fy[(ty + 1) * TX + tx] - fy[ty * TX + tx]) * fidy;
+        cell_e<T>(K.qtau, K.te2, cx, cy, u1x, u2y, tile_c1<T, SCHEME>(su2 + c, 1), tile_c1<T, SCHEME>(su1 + c, BW), g1, g2, su1[c],
+                  su2[c], e1, e2);
+        T* e = reinterpret_cast<T*>(I.E[j]);
+        e[o] = e1;
+        e[o + pl] = e2;
+      }
     }
     if (need & NEED_LTH) {
-      reinterpret_cast<T*>(I.Lth[j])[o] = cdiff2<T, SCHEME>(sth + c, 1, idx * idx) + cdiff2<T, SCHEME>(sth + c, BW, idy * idy);
+      reinterpret_cast<T*>(I.Lth[j])[o] = cell_sum(d2_scale<T, SCHEME>(idx), tile_c2<T, SCHEME>(sth + c, 1), d2_scale<T, SCHEME>(idy),
+                                                   tile_c2<T, SCHEME>(sth + c, BW));
     }
     if (needB) {
       // step 3 of every later stage uses D_LF . B(v^(j)) and D_0 theta^(j) only as their
       // sum (times a_ij): one 2-plane field, summed here as it was summed there
       const T* fxb = fx + NX;
       const T* fyb = fy + NY;
-      const T d1 = (fxb[ty * (TX + 1) + tx + 1] - fxb[ty * (TX + 1) + tx]) * fidx +
-                   (fyb[(ty + 1) * TX + tx] - fyb[ty * TX + tx]) * fidy;
-      const T d2 = (fxb[NX + ty * (TX + 1) + tx + 1] - fxb[NX + ty * (TX + 1) + tx]) * fidx +
-                   (fyb[NY + (ty + 1) * TX + tx] - fyb[NY + ty * TX + tx]) * fidy;
+      const T d1 = cell_sum(fxb[ty * (TX + 1) + tx + 1] - fxb[ty * (TX + 1) + tx], fidx, fyb[(ty + 1) * TX + tx] - fyb[ty * TX + tx], fidy);
+      const T d2 = cell_sum(fxb[NX + ty * (TX + 1) + tx + 1] - fxb[NX + ty * (TX + 1) + tx], fidx,
+                            fyb[NY + (ty + 1) * TX + tx] - fyb[NY + ty * TX + tx], fidy);
       T* db = reinterpret_cast<T*>(I.DLFB[j]);
-      db[o] = d1 + cdiff<T, SCHEME>(sth + c, 1, idx);
-      db[o + pl] = d2 + cdiff<T, SCHEME>(sth + c, BW, idy);
+      db[o] = fma(cx, tile_c1<T, SCHEME>(sth + c, 1), d1);
+      db[o + pl] = fma(cy, tile_c1<T, SCHEME>(sth + c, BW), d2);
     }
     if (need & NEED_V) {
       // step 1 of stage i = j + 1 at this cell
@@ -1037,8 +1076,8 @@ __global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks
         int k = 3;
         for (int jj = 1; jj < i; ++jj) {
           if (has(mwp, jj)) {
-            p1 = p1 + K.wp[i][jj] * s[k * PL + e];
-            p2 = p2 + K.wp[i][jj] * s[(k + 1) * PL + e];
+            p1 = fma(K.wp[i][jj], s[k * PL + e], p1);
+            p2 = fma(K.wp[i][jj], s[(k + 1) * PL + e], p2);
             k += 2;
           }
         }
@@ -1058,26 +1097,26 @@ __global__ void __launch_bounds__(Geo<T, SCHEME, TX, TY>::NT, stencil_min_blocks
     const T fidx = flux_scale<T, SCHEME>(idx), fidy = flux_scale<T, SCHEME>(idy);
     const int c = G::C00 + ty * BW + tx;
     const size_t o = (size_t)(t.y0 + ty) * nx + (t.x0 + tx);
-    const T d1 = (fx[ty * (TX + 1) + tx + 1] - fx[ty * (TX + 1) + tx]) * fidx + (fy[(ty + 1) * TX + tx] - fy[ty * TX + tx]) * fidy;
-    const T d2 = (fx[NX + ty * (TX + 1) + tx + 1] - fx[NX + ty * (TX + 1) + tx]) * fidx +
-                 (fy[NY + (ty + 1) * TX + tx] - fy[NY + ty * TX + tx]) * fidy;
-    const T g1 = cdiff<T, SCHEME>(sth + c, 1, idx), g2 = cdiff<T, SCHEME>(sth + c, BW, idy);
-    const T dvi = cdiff<T, SCHEME>(sv1 + c, 1, idx) + cdiff<T, SCHEME>(sv2 + c, BW, idy);
+    const T cx = c1_scale<SCHEME>(idx, K.cdx), cy = c1_scale<SCHEME>(idy, K.cdy);
+    const T d1 = cell_sum(fx[ty * (TX + 1) + tx + 1] - fx[ty * (TX + 1) + tx], fidx, fy[(ty + 1) * TX + tx] - fy[ty * TX + tx], fidy);
+    const T d2 = cell_sum(fx[NX + ty * (TX + 1) + tx + 1] - fx[NX + ty * (TX + 1) + tx], fidx,
+                          fy[NY + (ty + 1) * TX + tx] - fy[NY + ty * TX + tx], fidy);
+    const T dvi = cell_sum(cx, tile_c1<T, SCHEME>(sv1 + c, 1), cy, tile_c1<T, SCHEME>(sv2 + c, BW));
     // step 3
     T s1 = T(0), s2 = T(0);
     for (int jj = 1; jj < i; ++jj) {
       if (has(mim, jj)) {
         const T* bg = reinterpret_cast<const T*>(I.DLFB[jj]);   // D_LF . B(v^(jj)) + D_0 theta^(jj)
-        s1 = s1 + K.aim[i][jj] * bg[o];
-        s2 = s2 + K.aim[i][jj] * bg[o + pl];
+        s1 = fma(K.aim[i][jj], bg[o], s1);
+        s2 = fma(K.aim[i][jj], bg[o + pl], s2);
       }
     }
-    s1 = s1 + K.aim[i][i] * (d1 + g1);
-    s2 = s2 + K.aim[i][i] * (d2 + g2);
+    s1 = fma(K.aim[i][i], fma(cx, tile_c1<T, SCHEME>(sth + c, 1), d1), s1);
+    s2 = fma(K.aim[i][i], fma(cy, tile_c1<T, SCHEME>(sth + c, BW), d2), s2);
     const T* Xn = reinterpret_cast<const T*>(I.X);
     T* out = reinterpret_cast<T*>(I.Xs[i]);
     const T dt = K.dt;
-    const T u1 = Xn[o] - dt * s1, u2 = Xn[o + pl] - dt * s2;
+    const T u1 = fma(-dt, s1, Xn[o]), u2 = fma(-dt, s2, Xn[o + pl]);
     if (!close_step) {
       out[o] = u1;
       out[o + pl] = u2;

@@ -96,19 +96,21 @@ inline bool split_fluxes(const ap_dvm_params& p) {
   return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;
 }
 
-// Whether a solve is taken by the marching kernels: FP32, enough cells for their warps (each holds
-// a row of 26 columns) to fill the chip, and a width that does not leave over a quarter of their
-// columns beyond the grid.  Explicit + update, us per step, marching against tiles: WENO5 256^2 54 and
-// 45, 384^2 58 and 61, 512^2 66 and 78, 1024^2 147 and 216, 2048^2 477 and 774; WENO3 56 and 51, 59 and
-// 68, 66 and 85, 141 and 240, 464 and 888; LF1 47 and 41, 49 and 55, 52 and 65, 110 and 169, 383 and 605.  A property of the solve alone, so that a batch does not change its result.
-constexpr long long kMarchMinCells = 384LL * 384;
-inline bool marching(const ap_dvm_params& p) {
+// Whether a solve is taken by the marching kernels: FP32, a width that does not leave over a quarter of
+// their warps' columns (26 each) beyond the grid, and enough cells, of its own or of its batch, for
+// these warps to fill the chip.  Explicit + update, us per step, marching against tiles: WENO5 256^2 54
+// and 45, 384^2 58 and 61, 512^2 66 and 78, 1024^2 147 and 216, 2048^2 477 and 774; WENO3 56 and 51, 59
+// and 68, 66 and 85, 141 and 240, 464 and 888; LF1 47 and 41, 49 and 55, 52 and 65, 110 and 169, 383 and
+// 605.  24 uneven solves of 64 to 512 cells a side, 5 steps: PLACEHOLDER7.  Both kinds give the same bits
+// (cell_c1 and what follows it in stencil_kernels.cuh), so that a batch does not change a solve's result.
+constexpr long long kMarchMinCells = 384LL * 384, kMarchMinBatchCells = 2 * kMarchMinCells;
+inline bool march_wide(const ap_dvm_params& p) {
   const int covered = (p.nx + MARCH_OUT - 1) / MARCH_OUT * MARCH_OUT;
-  return p.precision != AP_DVM_FP64 && (long long)p.nx * p.ny >= kMarchMinCells &&
-         4LL * covered <= 5LL * p.nx;
+  return p.precision != AP_DVM_FP64 && 4LL * covered <= 5LL * p.nx;
 }
-inline unsigned stencil_kind(const ap_dvm_params& p) {
-  return split_fluxes(p) ? STENCIL_SPLIT : (marching(p) ? STENCIL_MARCH : STENCIL_WHOLE);
+inline unsigned stencil_kind(const ap_dvm_params& p, bool march_all) {
+  if (split_fluxes(p)) return STENCIL_SPLIT;
+  return march_wide(p) && (march_all || (long long)p.nx * p.ny >= kMarchMinCells) ? STENCIL_MARCH : STENCIL_WHOLE;
 }
 inline int march_tasks(int nx, int ny, int rows) { return ((nx + MARCH_OUT - 1) / MARCH_OUT) * ((ny + rows - 1) / rows); }
 

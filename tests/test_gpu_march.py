@@ -92,6 +92,26 @@ def test_batch_beside_tiles_equals_alone(prec):
     b.sync_status()
 
 
+@pytest.mark.parametrize("scheme", ["LF1_C2", "WENO3_C4", "WENO5_C4"])
+@pytest.mark.parametrize("eps,tab", [(1e-2, "gsa2"), (1e-5, "gsa2"), (1e-2, "ars4")])
+def test_small_solves_of_a_large_batch_equal_alone(scheme, eps, tab):
+    """Enough cells together, so that every solve of the batch is taken by the marching kernels (but the
+    one too narrow for them): bit for bit what the tile kernels give each alone."""
+    sizes = [(256, 256), (128, 128), (64, 64), (100, 200), (127, 255), (300, 300), (40, 400), (210, 300)]
+    tmpl = _setup(1024, 1024, tab, eps, scheme=scheme)[1]
+    b = api.Batch(tmpl, len(sizes))
+    want = []
+    for k, (nx, ny) in enumerate(sizes):
+        X0, p, _ = _setup(nx, ny, tab, eps, scheme=scheme)
+        b.attach(k, p)
+        b.set_state(torch.from_numpy(X0).cuda(), slot=k)
+        want.append(_run(X0, p, 2).get_populations(dtype=torch.float32))
+    b.step(2)
+    b.sync_status()
+    for k in range(len(sizes)):
+        assert torch.equal(b.get_populations(k, dtype=torch.float32), want[k]), sizes[k]
+
+
 def test_non_finite_values_reach_the_status():
     X0, p, _ = _setup(400, 400, "gsa2", 1e-2)
     X0[0, 11, 399] = np.inf
