@@ -80,9 +80,13 @@ enum { AP_DVM_FP64 = 0, AP_DVM_FP32_DEV = 1, AP_DVM_FP32_DEV_TH = 2 }; /* precis
  *              with i = 1), with a_ii > 0 for i >= 2, and the pair globally
  *              stiffly accurate, so that the last stage is the new state.
  *  space_scheme  AP_DVM_LF1_C2, AP_DVM_WENO3_C4 or AP_DVM_WENO5_C4.
- *  precision   AP_DVM_FP64 (all in FP64) or AP_DVM_FP32_DEV (FP32 deviation
- *              populations and FP32 transport; FP64 moment sums, division by
- *              rho0*mach, and closed-form relaxation when eps <= 1e-4).
+ *  precision   AP_DVM_FP64 (all in FP64; WENO solves of at least 256 cells per
+ *              side evaluate the part of their fluxes that is not linear in the
+ *              data, nonlinear weight times difference, in pairs of floats of 48
+ *              bits, from differences taken in FP64) or AP_DVM_FP32_DEV (FP32
+ *              deviation populations and FP32 transport; moment sums, division by
+ *              rho0*mach, and closed-form relaxation when eps <= 1e-4 in pairs of
+ *              floats, rounded once).
  *              AP_DVM_FP32_DEV_TH is AP_DVM_FP32_DEV with theta carried from
  *              step to step in its own FP32 plane beside the populations
  *              instead of being summed back from them: theta rides at O(eps)
@@ -204,7 +208,9 @@ ap_dvm_status ap_dvm_step_slots(ap_dvm_handle* h, int nsteps, const int* steps_p
 /* Use a captured CUDA graph of k steps for ap_dvm_step (k = 0: direct launches). */
 ap_dvm_status ap_dvm_set_graph_steps(ap_dvm_handle* h, int k);
 /* Tile shape of the stencil kernels: 0 = 32x8, 1 = 32x4, 2 = 16x8, 3 = 8x8,
- * 4 = 64x4, 5 = 32x16, -1 = automatic.  Every attached grid must be at least the tile. */
+ * 4 = 64x4, 5 = 32x16, -1 = automatic.  Every attached grid must be at least the tile.
+ * (FP32 solves that the marching kernels take, large ones and those of a large batch, use no
+ * tile; their results are the same bits.) */
 ap_dvm_status ap_dvm_set_tile(ap_dvm_handle* h, int tile);
 int ap_dvm_get_tile(const ap_dvm_handle* h);
 /* Kernel launches enqueued by one ap_dvm_step(h, 1). */
@@ -291,9 +297,8 @@ void ap_dvm_destroy(ap_dvm_handle* h);
 ap_dvm_status ap_dvm_fma_peak(int precision, int iters, int reps, void* cuda_stream, double* tflops,
                               double* ms_per_launch);
 
-/* Self-check of the integer-pipe FP32 <-> FP64 conversions the FP32 forms use in place
- * of the conversion instructions (the moment sums of the close and the FP64
- * relaxations): for each of the n FP64 values at d_in (device), the narrowing to FP32
+/* Self-check of the library's integer-pipe FP32 <-> FP64 conversions (widen_f32,
+ * narrow_f64_rn, exact stand-ins for the conversion instructions): for each of the n FP64 values at d_in (device), the narrowing to FP32
  * (nearest, ties to even) and the widening of that FP32 value back to FP64 are compared
  * with the instructions' results bit for bit (a NaN only as a NaN).  d_counts (device,
  * 2 unsigned, caller-owned) receives the numbers of mismatching narrowings and

@@ -93,8 +93,8 @@ struct MarchPair<WENO5_C4> {
     m[2] = march_curv(g[3] - u[3], g[4] - u[4], g[5] - u[5], ew4);
   }
   __device__ __forceinline__ float flux(const float* g, const float* u, float) const {
-    return add_rn(w5_rec_f32(g[0] + u[0], g[1] + u[1], g[2] + u[2], g[3] + u[3], g[4] + u[4], p[0], p[1], p[2]),
-                  w5_rec_f32(g[5] - u[5], g[4] - u[4], g[3] - u[3], g[2] - u[2], g[1] - u[1], m[2], m[1], m[0]));
+    return w5_flux_f32(w5_rec_f32(g[0] + u[0], g[1] + u[1], g[2] + u[2], g[3] + u[3], g[4] + u[4], p[0], p[1], p[2]),
+                       w5_rec_f32(g[5] - u[5], g[4] - u[4], g[3] - u[3], g[2] - u[2], g[1] - u[1], m[2], m[1], m[0]));
   }
 };
 
@@ -112,10 +112,10 @@ __device__ __forceinline__ float march_dx(float g, float u, float ew4) {
     } else {
       const float pa = lane_up(P, 2), pe = lane_dn(P, 2);
       const float cp = march_curv(pb, P, pd, ew4);
-      const float l = w5_rec_f32(pa, pb, P, pd, pe, lane_up(cp, 1), cp, lane_dn(cp, 1));
+      const float2 l = w5_rec_f32(pa, pb, P, pd, pe, lane_up(cp, 1), cp, lane_dn(cp, 1));
       const float ma = lane_up(M, 1), me = lane_dn(M, 3);
       const float cm = march_curv(ma, M, mc, ew4);
-      f = add_rn(l, w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm));
+      f = w5_flux_f32(l, w5_rec_f32(me, md, mc, M, ma, lane_dn(cm, 2), lane_dn(cm, 1), cm));
     }
   }
   return f - lane_up(f, 1);

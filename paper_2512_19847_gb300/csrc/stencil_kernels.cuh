@@ -423,7 +423,7 @@ __device__ __forceinline__ void axis_fluxes(const T* const* g, const T* const* U
 // Scalar FP32 WENO5 reconstruction from register values: the arithmetic of w5_nd
 // (about the centred candidate, three times the reconstruction) with reciprocal
 // weights r_k = 1 / s_k, as products of the s_k could leave the float range.
-__device__ __forceinline__ float w5_rec_f32(float a, float b, float c, float d, float e, float C0, float C1, float C2) {
+__device__ __forceinline__ float2 w5_rec_f32(float a, float b, float c, float d, float e, float C0, float C1, float C2) {
   const float l0 = fmaf(3.f, c, fmaf(-4.f, b, a));
   const float l1 = b - d;
   const float l2 = fmaf(3.f, c, fmaf(-4.f, d, e));
@@ -433,8 +433,10 @@ __device__ __forceinline__ float w5_rec_f32(float a, float b, float c, float d, 
   const float p1x3 = fmaf(2.5f, c, fmaf(-0.5f, b, d));          // 3 p_1
   const float ta = l0 + l1, tb = 1.5f * (l1 - l2);              // 3 (p_0 - p_1), 9 (p_2 - p_1)
   const float num = fmaf(p1x3, den, fmaf(r0, ta, r2 * tb));     // 30 sum_k d_k r_k p_k
-  return __fmul_rn(num, rcp_approx(den));   // (not contracted with what it is added to: every kernel the same)
+  return make_float2(num, rcp_approx(den));
 }
+// Interface flux from the left and right reconstructions (numerator, reciprocal of the denominator).
+__device__ __forceinline__ float w5_flux_f32(float2 l, float2 r) { return fmaf(l.x, l.y, __fmul_rn(r.x, r.y)); }
 
 // Values of the LF partner U at a staged point: one plane, or the weighted sum of
 // the staged u planes of earlier stages (the explicit-weight dissipation partner),
@@ -492,9 +494,9 @@ __device__ __forceinline__ void w5_runs_item(const float* g, const UF& U, bool n
   for (int i = 0; i < KR; ++i) {
     const int m = m0 + i;
     // left-biased reconstruction of g+ (points m..m+4 of the run), mirrored right-biased of g- (points m+5..m+1)
-    const float fl = w5_rec_f32(Pp[i], Pp[i + 1], Pp[i + 2], Pp[i + 3], Pp[i + 4], Cp[i + 1], Cp[i + 2], Cp[i + 3]);
-    const float fr = w5_rec_f32(Pm[i + 5], Pm[i + 4], Pm[i + 3], Pm[i + 2], Pm[i + 1], Cm[i + 4], Cm[i + 3], Cm[i + 2]);
-    if (NI % KR == 0 || m < NI) out[AX == 0 ? line * NI + m : m * TX + line] = __fadd_rn(fl, fr);
+    const float2 fl = w5_rec_f32(Pp[i], Pp[i + 1], Pp[i + 2], Pp[i + 3], Pp[i + 4], Cp[i + 1], Cp[i + 2], Cp[i + 3]);
+    const float2 fr = w5_rec_f32(Pm[i + 5], Pm[i + 4], Pm[i + 3], Pm[i + 2], Pm[i + 1], Cm[i + 4], Cm[i + 3], Cm[i + 2]);
+    if (NI % KR == 0 || m < NI) out[AX == 0 ? line * NI + m : m * TX + line] = w5_flux_f32(fl, fr);
   }
 }
 
@@ -731,15 +733,19 @@ __device__ __forceinline__ T flux_scale(T inv_h) {
 //
 // The scheme's central differences without their scales (c1_scale, d2_scale), from the values at offsets
 // -2 .. 2 along a line.
+// FP64 sums them from the upper value down: D_0 . u, a difference of nearly opposite sums that the
+// right-hand side divides by dt, then rounds as in a plain evaluation.
 template <typename T, int SCHEME>
 __device__ __forceinline__ T cell_c1(T am2, T am1, T ap1, T ap2) {
   if (SCHEME == LF1_C2) return ap1 - am1;
-  return fma(T(8), ap1 - am1, am2 - ap2);
+  if constexpr (sizeof(T) == 8) return fma(T(-8), am1, fma(T(8), ap1, -ap2)) + am2;
+  else return fma(T(8), ap1 - am1, am2 - ap2);
 }
 template <typename T, int SCHEME>
 __device__ __forceinline__ T cell_c2(T am2, T am1, T a, T ap1, T ap2) {
-  if (SCHEME == LF1_C2) return fma(T(-2), a, ap1 + am1);
-  return fma(T(-30), a, fma(T(16), ap1 + am1, -(ap2 + am2)));
+  if (SCHEME == LF1_C2) return fma(T(-2), a, ap1) + am1;
+  if constexpr (sizeof(T) == 8) return fma(T(16), am1, fma(T(-30), a, fma(T(16), ap1, -ap2))) - am2;
+  else return fma(T(-30), a, fma(T(16), ap1 + am1, -(ap2 + am2)));
 }
 template <typename T, int SCHEME>
 __device__ __forceinline__ T tile_c1(const T* f, int st) {
@@ -936,10 +942,9 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
     const int nt = s_nt;
     const int nx = I.nx, ny = I.ny;
     const size_t pl = (size_t)nx * ny;
-    // D_0^2:B(v) = -sx2 S_xx + 2 sx1 sy1 S_xy + sy2 S_yy with the unscaled sums S (d1_sum, d2_sum), the
-    // centre value of the two second differences taken once, times their weights' sum (0 on a square mesh)
+    // D_0^2:B(v) = -sx2 S_xx + 2 sx1 sy1 S_xy + sy2 S_yy with the unscaled sums S (d1_sum, d2_sum)
     const T msx2 = -d2_scale<T, SCHEME>(K.inv_dx), sy2 = d2_scale<T, SCHEME>(K.inv_dy);
-    const T sxy2 = T(2) * d1_scale<T, SCHEME>(K.inv_dx) * d1_scale<T, SCHEME>(K.inv_dy), sc = d2_centre<T, SCHEME>() * (msx2 + sy2);
+    const T sxy2 = T(2) * d1_scale<T, SCHEME>(K.inv_dx) * d1_scale<T, SCHEME>(K.inv_dy);
     const T kap = K.kappa[i];
     const T cdb = has(b.m_im[i], i) ? K.c_db[i][i] : T(0);
     const T* v1 = reinterpret_cast<const T*>(I.Xs[i]) + 3 * pl;
@@ -997,10 +1002,10 @@ __global__ void __launch_bounds__(RHS_THREADS, sizeof(T) == 4 ? APD_RHS_MINB32 :
         const T vp1 = __shfl_down_sync(FULL, v, 1), vp2 = __shfl_down_sync(FULL, v, 2);
         const T dm1 = __shfl_up_sync(FULL, dy, 1), dm2 = __shfl_up_sync(FULL, dy, 2);
         const T dp1 = __shfl_down_sync(FULL, dy, 1), dp2 = __shfl_down_sync(FULL, dy, 2);
-        const T sxx = d2_sum<T, SCHEME>(vm2, vm1, vp1, vp2);
+        const T sxx = d2_sum<T, SCHEME>(vm2, vm1, v, vp1, vp2);
         const T sxy = d1_sum<T, SCHEME>(dm2, dm1, dp1, dp2);
-        const T syy = d2_sum<T, SCHEME>(a[h], a[h + 1], a[h + 3], a[h + 4]);
-        const T Bh = fma(sc, v, fma(msx2, sxx, fma(sxy2, sxy, sy2 * syy)));
+        const T syy = d2_sum<T, SCHEME>(a[h], a[h + 1], a[h + 2], a[h + 3], a[h + 4]);
+        const T Bh = fma(sxy2, sxy, fma(msx2, sxx, sy2 * syy));
         if (outc && h < nrows) {
           const size_t o = (size_t)(y0 + h) * nx + x;
           if (keep_db) DBi[o] = Bh;
