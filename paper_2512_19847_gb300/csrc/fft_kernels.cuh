@@ -250,17 +250,24 @@ __device__ __forceinline__ void fft_rev(typename Cplx<T>::type* x, int ln, int n
 // in x[] (natural order, zero beyond n) with the Bluestein filter whose DFT is
 // filt (bit-reversed order, scaled by 1/M; conjugated when inv): forward
 // radix-2 DFT (natural in, bit-reversed out), product with the filter,
-// inverse DFT (bit-reversed in, natural out).
+// inverse DFT (bit-reversed in, natural out).  Shared memory padded as in the power-of-two kernels:
+// without it the passes of small distance read many lanes from one bank pair (FP32 509x251, four
+// steps: 485 us unpadded, 448 us padded).
 template <typename T>
 __device__ __forceinline__ void bluestein_conv(typename Cplx<T>::type* x, int lm, int ntr,
                                                const typename Cplx<T>::type* __restrict__ filt,
                                                const typename Cplx<T>::type* __restrict__ tw, int lnmax, bool inv,
                                                int tid, int nthr) {
-  fft_rev<T>(x, lm, ntr, tw, lnmax, false, tid, nthr);
+  using C = typename Cplx<T>::type;
+  constexpr int PS = pad_shift<T>();
+  fft_rev<T, PS>(x, lm, ntr, tw, lnmax, false, tid, nthr);
   const int m = 1 << lm;
-  for (int e = tid; e < ntr * m; e += nthr) x[e] = cmul_tw(filt[e & (m - 1)], x[e], inv);
+  for (int e = tid; e < ntr * m; e += nthr) {
+    C& v = x[pidx<PS>(e)];
+    v = cmul_tw(filt[e & (m - 1)], v, inv);
+  }
   __syncthreads();
-  fft_dit<T>(x, lm, ntr, tw, lnmax, true, tid, nthr);
+  fft_dit<T, PS>(x, lm, ntr, tw, lnmax, true, tid, nthr);
 }
 
 // mean(theta^n) of instance I from its nt partial sums (one per item of the first
@@ -585,6 +592,7 @@ __device__ __forceinline__ int stockham(typename Cplx<T>::type* x, int m, int n,
 
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs(const __grid_constant__ BatchDev b) {
+  constexpr int PS = pad_shift<T>();   // Bluestein's regions; the mixed-radix buffers are not padded
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -636,7 +644,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs
         if (row + 1 < (size_t)ny) z.y = R[(row + 1) * n + k];
         z = cmul_tw(ch[k], z, false);
       }
-      x[e] = z;
+      x[pidx<PS>(e)] = z;
     }
     __syncthreads();
     bluestein_conv<T>(x, ln, ntr, reinterpret_cast<const C*>(I.filt[0]), twiddles<T>(b), b.lnmax, false, tid, nthr);
@@ -644,7 +652,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_fwd_bs
     const int nh = (n >> 1) + 1;
     for (int e = tid; e < ntr * nh; e += nthr) {
       const int p = e / nh, k = e - p * nh, km = k == 0 ? 0 : n - k;
-      const C zk = cmul_tw(ch[k], x[p * m + k], false), zm = cmul_tw(ch[km], x[p * m + km], false);
+      const C zk = cmul_tw(ch[k], x[pidx<PS>(p * m + k)], false), zm = cmul_tw(ch[km], x[pidx<PS>(p * m + km)], false);
       const size_t row = (size_t)(2 * (pair0 + p));
       C A, B;
       A.x = T(0.5) * (zk.x + zm.x); A.y = T(0.5) * (zk.y - zm.y);
@@ -669,6 +677,7 @@ __device__ __forceinline__ void apply_factor(float2& v, double f) {
 // so the division by the symbol applies to the convolution directly.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(const __grid_constant__ BatchDev b, int i) {
+  constexpr int PS = pad_shift<T>();   // Bluestein's regions; the mixed-radix buffers are not padded
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -722,7 +731,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
       C z;
       z.x = T(0); z.y = T(0);
       if (y < n) z = cmul_tw(ch[y], S[(size_t)y * ss + col0 + g], false);
-      x[e] = z;
+      x[pidx<PS>(e)] = z;
     }
     __syncthreads();
     bluestein_conv<T>(x, ln, ntr, filt, twiddles<T>(b), b.lnmax, false, tid, nthr);
@@ -730,7 +739,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
     const double scale = I.hscale;
     for (int e = tid; e < ntr * m; e += nthr) {
       const int g = e >> ln, ky = e & (m - 1), kx = col0 + g;
-      C v = x[e];
+      C v = x[pidx<PS>(e)];
       if (ky >= n) {
         v.x = T(0); v.y = T(0);
       } else if (kx == 0 && ky == 0) {
@@ -739,13 +748,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
         const double f = scale * rcp_newton(I.lamx[kx] + I.lamy[ky] - kap);
         apply_factor(v, f);
       }
-      x[e] = v;
+      x[pidx<PS>(e)] = v;
     }
     __syncthreads();
     bluestein_conv<T>(x, ln, ntr, filt, twiddles<T>(b), b.lnmax, true, tid, nthr);
     for (int e = tid; e < ntr * m; e += nthr) {
       const int g = e >> ln, y = e & (m - 1);
-      if (y < n) S[(size_t)y * ss + col0 + g] = cmul_tw(ch[y], x[e], true);
+      if (y < n) S[(size_t)y * ss + col0 + g] = cmul_tw(ch[y], x[pidx<PS>(e)], true);
     }
     __syncthreads();
   }
@@ -753,6 +762,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_cols_bs(con
 
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs(const __grid_constant__ BatchDev b, int i) {
+  constexpr int PS = pad_shift<T>();   // Bluestein's regions; the mixed-radix buffers are not padded
   grid_dependency();
   using C = typename Cplx<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -809,7 +819,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs
         z.x = A.x - B.y; z.y = A.y + B.x;
         z = cmul_tw(ch[k], z, true);
       }
-      x[e] = z;
+      x[pidx<PS>(e)] = z;
     }
     __syncthreads();
     bluestein_conv<T>(x, ln, ntr, reinterpret_cast<const C*>(I.filt[0]), twiddles<T>(b), b.lnmax, true, tid, nthr);
@@ -818,7 +828,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_fft_rows_inv_bs
       const int p = e >> ln, mm = e & (m - 1);
       if (mm >= n) continue;
       const size_t row = (size_t)(2 * (pair0 + p));
-      const C z = cmul_tw(ch[mm], x[e], true);
+      const C z = cmul_tw(ch[mm], x[pidx<PS>(e)], true);
       th[row * n + mm] = z.x;
       if (row + 1 < (size_t)ny) th[(row + 1) * n + mm] = z.y;
     }
