@@ -123,6 +123,36 @@ __host__ __device__ constexpr int padded_len(int n, int ps) { return ps >= 31 ? 
 // 104 with twiddles and constant roots multiplied separately.  2048^2, FP64, ms per step: columns
 // 0.944 -> 0.652, rows 0.417 -> 0.312 (forward) and 0.406 -> 0.290 (inverse); FP32, which is not: 0.098
 // -> 0.095, 0.050 -> 0.052 and 0.049 -> 0.047.
+//
+// The eight elements of one step in registers: dit8 three stages from stage s (half h), dit8_first the same
+// at s = 1.
+template <typename C>
+__device__ __forceinline__ void dit8(C (&v)[8], const C* __restrict__ tw, int lnmax, int s, int pos, int h, bool inv) {
+  const C w1 = tw_of(tw[pos << (lnmax - s)], inv), w2 = tw_of(tw[pos << (lnmax - s - 1)], inv);
+  const C w3 = tw_of(tw[pos << (lnmax - s - 2)], inv), w4 = tw_of(tw[(pos + h) << (lnmax - s - 2)], inv);
+  bfly(v[0], v[1], w1); bfly(v[2], v[3], w1); bfly(v[4], v[5], w1); bfly(v[6], v[7], w1);
+  const C w2j = tw_j(w2, inv);
+  bfly(v[0], v[2], w2); bfly(v[1], v[3], w2j); bfly(v[4], v[6], w2); bfly(v[5], v[7], w2j);
+  bfly(v[0], v[4], w3); bfly(v[1], v[5], w4); bfly(v[2], v[6], tw_j(w3, inv)); bfly(v[3], v[7], tw_j(w4, inv));
+}
+template <typename C>
+__device__ __forceinline__ void dit8_first(C (&v)[8], bool inv) {
+  bfly1(v[0], v[1]); bfly1(v[2], v[3]); bfly1(v[4], v[5]); bfly1(v[6], v[7]);
+  bfly1(v[0], v[2]); bflyj(v[1], v[3], inv); bfly1(v[4], v[6]); bflyj(v[5], v[7], inv);
+  const C w8 = tw_8<C>(inv);
+  bfly1(v[0], v[4]); bfly(v[1], v[5], w8); bflyj(v[2], v[6], inv); bfly(v[3], v[7], tw_j(w8, inv));
+}
+template <int PS, typename C>
+__device__ __forceinline__ void load8(C (&v)[8], const C* x, int q, int h) {
+#pragma unroll
+  for (int m = 0; m < 8; ++m) v[m] = x[pidx<PS>(q + m * h)];
+}
+template <int PS, typename C>
+__device__ __forceinline__ void store8(const C (&v)[8], C* x, int q, int h) {
+#pragma unroll
+  for (int m = 0; m < 8; ++m) x[pidx<PS>(q + m * h)] = v[m];
+}
+
 template <typename T, int PS = 31>
 __device__ __forceinline__ void fft_dit(typename Cplx<T>::type* x, int ln, int ntr,
                                         const typename Cplx<T>::type* __restrict__ tw, int lnmax,
@@ -136,23 +166,11 @@ __device__ __forceinline__ void fft_dit(typename Cplx<T>::type* x, int ln, int n
       const int t = k >> (ln - 3), bi = k & (ne - 1);
       const int pos = bi & (h - 1), grp = bi >> (s - 1);
       const int q = t * n + grp * 8 * h + pos;
-      C v0 = x[pidx<PS>(q)], v1 = x[pidx<PS>(q + h)], v2 = x[pidx<PS>(q + 2 * h)], v3 = x[pidx<PS>(q + 3 * h)];
-      C v4 = x[pidx<PS>(q + 4 * h)], v5 = x[pidx<PS>(q + 5 * h)], v6 = x[pidx<PS>(q + 6 * h)], v7 = x[pidx<PS>(q + 7 * h)];
-      if (s == 1) {
-        bfly1(v0, v1); bfly1(v2, v3); bfly1(v4, v5); bfly1(v6, v7);
-        bfly1(v0, v2); bflyj(v1, v3, inv); bfly1(v4, v6); bflyj(v5, v7, inv);
-        const C w8 = tw_8<C>(inv);
-        bfly1(v0, v4); bfly(v1, v5, w8); bflyj(v2, v6, inv); bfly(v3, v7, tw_j(w8, inv));
-      } else {
-        const C w1 = tw_of(tw[pos << (lnmax - s)], inv), w2 = tw_of(tw[pos << (lnmax - s - 1)], inv);
-        const C w3 = tw_of(tw[pos << (lnmax - s - 2)], inv), w4 = tw_of(tw[(pos + h) << (lnmax - s - 2)], inv);
-        bfly(v0, v1, w1); bfly(v2, v3, w1); bfly(v4, v5, w1); bfly(v6, v7, w1);
-        const C w2j = tw_j(w2, inv);
-        bfly(v0, v2, w2); bfly(v1, v3, w2j); bfly(v4, v6, w2); bfly(v5, v7, w2j);
-        bfly(v0, v4, w3); bfly(v1, v5, w4); bfly(v2, v6, tw_j(w3, inv)); bfly(v3, v7, tw_j(w4, inv));
-      }
-      x[pidx<PS>(q)] = v0; x[pidx<PS>(q + h)] = v1; x[pidx<PS>(q + 2 * h)] = v2; x[pidx<PS>(q + 3 * h)] = v3;
-      x[pidx<PS>(q + 4 * h)] = v4; x[pidx<PS>(q + 5 * h)] = v5; x[pidx<PS>(q + 6 * h)] = v6; x[pidx<PS>(q + 7 * h)] = v7;
+      C v[8];
+      load8<PS>(v, x, q, h);
+      if (s == 1) dit8_first(v, inv);
+      else dit8(v, tw, lnmax, s, pos, h, inv);
+      store8<PS>(v, x, q, h);
     }
     __syncthreads();
   }
@@ -189,36 +207,55 @@ __device__ __forceinline__ void fft_dit(typename Cplx<T>::type* x, int ln, int n
 // one table in that order, tr[j] = exp(-pi i 0.b0 b1 b2 ...), serves all levels: block j of three
 // successive levels takes tr[j], tr[2j] (times 1 and W_4) and tr[4j], tr[4j + 2] = W_8 tr[4j].
 // tr follows the nmax / 2 values of tw.
-template <typename T, int PS = 31>
-__device__ __forceinline__ void fft_rev(typename Cplx<T>::type* x, int ln, int ntr,
-                                        const typename Cplx<T>::type* __restrict__ tw, int lnmax,
-                                        bool inv, int tid, int nthr) {
+//
+// rev8 takes three levels of block j in registers, rev8_first those of the only block of the first levels.
+template <typename C>
+__device__ __forceinline__ void rev8(C (&v)[8], const C* __restrict__ tr, int j, bool inv) {
+  const C w1 = tw_of(tr[j], inv), w2 = tw_of(tr[2 * j], inv), w3 = tw_of(tr[4 * j], inv), w4 = tw_of(tr[4 * j + 2], inv);
+  bfly(v[0], v[4], w1); bfly(v[1], v[5], w1); bfly(v[2], v[6], w1); bfly(v[3], v[7], w1);
+  const C w2j = tw_j(w2, inv);
+  bfly(v[0], v[2], w2); bfly(v[1], v[3], w2); bfly(v[4], v[6], w2j); bfly(v[5], v[7], w2j);
+  bfly(v[0], v[1], w3); bfly(v[2], v[3], tw_j(w3, inv)); bfly(v[4], v[5], w4); bfly(v[6], v[7], tw_j(w4, inv));
+}
+template <typename C>
+__device__ __forceinline__ void rev8_first(C (&v)[8], bool inv) {
+  bfly1(v[0], v[4]); bfly1(v[1], v[5]); bfly1(v[2], v[6]); bfly1(v[3], v[7]);
+  bfly1(v[0], v[2]); bfly1(v[1], v[3]); bflyj(v[4], v[6], inv); bflyj(v[5], v[7], inv);
+  const C w8 = tw_8<C>(inv);
+  bfly1(v[0], v[1]); bflyj(v[2], v[3], inv); bfly(v[4], v[5], w8); bfly(v[6], v[7], tw_j(w8, inv));
+}
+
+// The first step takes element i of transform t from load(t, i), so that a kernel's input passes
+// from global memory to the butterflies without a pass of its own through shared memory; n >= 8.
+// Row passes at 2048^2, FP32, bound by these passes: 0.050 -> 0.038 (forward) and 0.046 -> 0.037 ms
+// (inverse) per step; FP64 forward 0.308 -> 0.291.
+template <typename T, int PS = 31, typename Load>
+__device__ __forceinline__ void fft_rev_from(typename Cplx<T>::type* x, int ln, int ntr,
+                                             const typename Cplx<T>::type* __restrict__ tw, int lnmax,
+                                             bool inv, int tid, int nthr, Load load) {
   using C = typename Cplx<T>::type;
   const C* __restrict__ tr = tw + (1 << (lnmax - 1));
-  const int n = 1 << ln;
-  int s = ln;   // levels of size 2^s and below are left
+  const int n = 1 << ln, ne = n >> 3, nb = ntr * ne;
+  for (int k = tid; k < nb; k += nthr) {
+    const int t = k >> (ln - 3), pos = k & (ne - 1);
+    C v[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[m] = load(t, pos + m * ne);
+    rev8_first(v, inv);
+    store8<PS>(v, x, t * n + pos, ne);
+  }
+  __syncthreads();
+  int s = ln - 3;   // levels of size 2^s and below are left
   for (; s >= 3; s -= 3) {
-    const int h = 1 << (s - 3), ne = n >> 3, nb = ntr * ne;
+    const int h = 1 << (s - 3);
     for (int k = tid; k < nb; k += nthr) {
       const int t = k >> (ln - 3), bi = k & (ne - 1);
       const int pos = bi & (h - 1), j = bi >> (s - 3);
       const int q = t * n + j * 8 * h + pos;
-      C v0 = x[pidx<PS>(q)], v1 = x[pidx<PS>(q + h)], v2 = x[pidx<PS>(q + 2 * h)], v3 = x[pidx<PS>(q + 3 * h)];
-      C v4 = x[pidx<PS>(q + 4 * h)], v5 = x[pidx<PS>(q + 5 * h)], v6 = x[pidx<PS>(q + 6 * h)], v7 = x[pidx<PS>(q + 7 * h)];
-      if (s == ln) {   // one block: constant twiddles
-        bfly1(v0, v4); bfly1(v1, v5); bfly1(v2, v6); bfly1(v3, v7);
-        bfly1(v0, v2); bfly1(v1, v3); bflyj(v4, v6, inv); bflyj(v5, v7, inv);
-        const C w8 = tw_8<C>(inv);
-        bfly1(v0, v1); bflyj(v2, v3, inv); bfly(v4, v5, w8); bfly(v6, v7, tw_j(w8, inv));
-      } else {
-        const C w1 = tw_of(tr[j], inv), w2 = tw_of(tr[2 * j], inv), w3 = tw_of(tr[4 * j], inv), w4 = tw_of(tr[4 * j + 2], inv);
-        bfly(v0, v4, w1); bfly(v1, v5, w1); bfly(v2, v6, w1); bfly(v3, v7, w1);
-        const C w2j = tw_j(w2, inv);
-        bfly(v0, v2, w2); bfly(v1, v3, w2); bfly(v4, v6, w2j); bfly(v5, v7, w2j);
-        bfly(v0, v1, w3); bfly(v2, v3, tw_j(w3, inv)); bfly(v4, v5, w4); bfly(v6, v7, tw_j(w4, inv));
-      }
-      x[pidx<PS>(q)] = v0; x[pidx<PS>(q + h)] = v1; x[pidx<PS>(q + 2 * h)] = v2; x[pidx<PS>(q + 3 * h)] = v3;
-      x[pidx<PS>(q + 4 * h)] = v4; x[pidx<PS>(q + 5 * h)] = v5; x[pidx<PS>(q + 6 * h)] = v6; x[pidx<PS>(q + 7 * h)] = v7;
+      C v[8];
+      load8<PS>(v, x, q, h);
+      rev8(v, tr, j, inv);
+      store8<PS>(v, x, q, h);
     }
     __syncthreads();
   }
@@ -243,6 +280,169 @@ __device__ __forceinline__ void fft_rev(typename Cplx<T>::type* x, int ln, int n
       x[pidx<PS>(i1)] = c;
     }
     __syncthreads();
+  }
+}
+
+template <typename T, int PS = 31>
+__device__ __forceinline__ void fft_rev(typename Cplx<T>::type* x, int ln, int ntr,
+                                        const typename Cplx<T>::type* __restrict__ tw, int lnmax,
+                                        bool inv, int tid, int nthr) {
+  const int n = 1 << ln;
+  fft_rev_from<T, PS>(x, ln, ntr, tw, lnmax, inv, tid, nthr, [=](int t, int i) { return x[pidx<PS>(t * n + i)]; });
+}
+
+// Forward transform, an operation on the spectrum and inverse transform of ntr <= 2^lg sequences of length
+// n = 2^ln >= 8, from load(t, i) to store(t, i, v); op(t, ky, v) changes value ky of the spectrum.  The levels
+// are taken so that those which do not fill a step of three come first forwards and last
+// backwards: the last forward and the first backward step then hold the same eight elements,
+// and with op between them they stay in registers.  The first step reads load() and the last one
+// writes store(); in these two adjacent threads take the same element of adjacent sequences.  Length 2048 passes
+// through shared memory 6 times instead of 9 (in, 4, op, 4, out before, the first and the last a half).
+// Column pass, ms per step: FP32 2048^2 (bound by these passes) 0.094 -> 0.070, FP64 2048^2 (bound by the
+// FP64 pipe) 0.650 -> 0.637.  In FP64 op is a pass of its own (spread) where a step does not fill the
+// block: a warp instruction costs the FP64 pipe the same with few lanes as with all, and eight
+// reciprocals one after the other in few warps cost more than the exchange (64^2 and 256^2, ten
+// steps: 378 and 422 us together, 335 and 406 apart).
+template <typename T, int PS, typename Load, typename Op, typename Store>
+__device__ __forceinline__ void fft_there_and_back(typename Cplx<T>::type* x, int ln, int lg, int ntr,
+                                                   const typename Cplx<T>::type* __restrict__ tw, int lnmax,
+                                                   int tid, int nthr, Load load, Op op, Store store) {
+  using C = typename Cplx<T>::type;
+  const C* __restrict__ tr = tw + (1 << (lnmax - 1));
+  const int n = 1 << ln, ne = n >> 3, nb = ntr * ne, G = 1 << lg;
+  if (ln == 3) {   // one step each way: nothing to exchange
+    for (int t = tid; t < ntr; t += nthr) {
+      C v[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) v[m] = load(t, m);
+      rev8_first(v, false);
+#pragma unroll
+      for (int m = 0; m < 8; ++m) op(t, brev(m, 3), v[m]);
+      dit8_first(v, true);
+#pragma unroll
+      for (int m = 0; m < 8; ++m) store(t, m, v[m]);
+    }
+    return;
+  }
+  const int left = ln % 3;
+  int s = ln - (left ? left : 3);   // levels of size 2^s and below are left
+  if (left == 0) {
+    for (int k = tid; k < (ne << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg;
+      if (t >= ntr) continue;
+      C v[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) v[m] = load(t, pos + m * ne);
+      rev8_first(v, false);
+      store8<PS>(v, x, t * n + pos, ne);
+    }
+  } else if (left == 2) {
+    const int h = n >> 2;
+#pragma unroll 2
+    for (int k = tid; k < (h << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg, q = t * n + pos;
+      if (t >= ntr) continue;
+      C x0 = load(t, pos), x1 = load(t, pos + h), x2 = load(t, pos + 2 * h), x3 = load(t, pos + 3 * h);
+      bfly1(x0, x2); bfly1(x1, x3);
+      bfly1(x0, x1); bflyj(x2, x3, false);
+      x[pidx<PS>(q)] = x0; x[pidx<PS>(q + h)] = x1; x[pidx<PS>(q + 2 * h)] = x2; x[pidx<PS>(q + 3 * h)] = x3;
+    }
+  } else {
+    const int h = n >> 1;
+#pragma unroll 4
+    for (int k = tid; k < (h << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg, q = t * n + pos;
+      if (t >= ntr) continue;
+      C a = load(t, pos), c = load(t, pos + h);
+      bfly1(a, c);
+      x[pidx<PS>(q)] = a; x[pidx<PS>(q + h)] = c;
+    }
+  }
+  __syncthreads();
+  for (; s > 3; s -= 3) {
+    const int h = 1 << (s - 3);
+    for (int k = tid; k < nb; k += nthr) {
+      const int t = k >> (ln - 3), bi = k & (ne - 1);
+      const int pos = bi & (h - 1), j = bi >> (s - 3);
+      const int q = t * n + j * 8 * h + pos;
+      C v[8];
+      load8<PS>(v, x, q, h);
+      rev8(v, tr, j, false);
+      store8<PS>(v, x, q, h);
+    }
+    __syncthreads();
+  }
+  // Element 8 j + m holds the value at the reversed bits.
+  const bool spread = sizeof(T) == 8 && nb < nthr;
+  for (int k = tid; k < nb; k += nthr) {
+    const int t = k >> (ln - 3), j = k & (ne - 1), ky = brev(j, ln - 3);
+    C v[8];
+    load8<PS>(v, x, 8 * k, 1);
+    rev8(v, tr, j, false);
+    if (!spread) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) op(t, ky + (brev(m, 3) << (ln - 3)), v[m]);
+      dit8_first(v, true);
+    }
+    store8<PS>(v, x, 8 * k, 1);
+  }
+  __syncthreads();
+  if (spread) {
+    for (int e = tid; e < ntr * n; e += nthr) op(e >> ln, brev(e & (n - 1), ln), x[pidx<PS>(e)]);
+    __syncthreads();
+    for (int k = tid; k < nb; k += nthr) {
+      C v[8];
+      load8<PS>(v, x, 8 * k, 1);
+      dit8_first(v, true);
+      store8<PS>(v, x, 8 * k, 1);
+    }
+    __syncthreads();
+  }
+  for (s = 4; s + 2 < ln; s += 3) {
+    const int h = 1 << (s - 1);
+    for (int k = tid; k < nb; k += nthr) {
+      const int t = k >> (ln - 3), bi = k & (ne - 1);
+      const int pos = bi & (h - 1), grp = bi >> (s - 1);
+      const int q = t * n + grp * 8 * h + pos;
+      C v[8];
+      load8<PS>(v, x, q, h);
+      dit8(v, tw, lnmax, s, pos, h, true);
+      store8<PS>(v, x, q, h);
+    }
+    __syncthreads();
+  }
+  if (left == 0) {
+    for (int k = tid; k < (ne << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg;
+      if (t >= ntr) continue;
+      C v[8];
+      load8<PS>(v, x, t * n + pos, ne);
+      dit8(v, tw, lnmax, s, pos, ne, true);
+#pragma unroll
+      for (int m = 0; m < 8; ++m) store(t, pos + m * ne, v[m]);
+    }
+  } else if (left == 2) {
+    const int h = n >> 2;
+#pragma unroll 2
+    for (int k = tid; k < (h << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg, q = t * n + pos;
+      if (t >= ntr) continue;
+      C x0 = x[pidx<PS>(q)], x1 = x[pidx<PS>(q + h)], x2 = x[pidx<PS>(q + 2 * h)], x3 = x[pidx<PS>(q + 3 * h)];
+      const C w1 = tw_of(tw[pos << (lnmax - s)], true), w2 = tw_of(tw[pos << (lnmax - s - 1)], true);
+      bfly(x0, x1, w1); bfly(x2, x3, w1);
+      bfly(x0, x2, w2); bfly(x1, x3, tw_j(w2, true));
+      store(t, pos, x0); store(t, pos + h, x1); store(t, pos + 2 * h, x2); store(t, pos + 3 * h, x3);
+    }
+  } else {
+    const int h = n >> 1;
+#pragma unroll 4
+    for (int k = tid; k < (h << lg); k += nthr) {
+      const int t = k & (G - 1), pos = k >> lg, q = t * n + pos;
+      if (t >= ntr) continue;
+      C a = x[pidx<PS>(q)], c = x[pidx<PS>(q + h)];
+      bfly(a, c, tw_of(tw[pos << (lnmax - s)], true));
+      store(t, pos, a); store(t, pos + h, c);
+    }
   }
 }
 
@@ -324,20 +524,18 @@ __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft
     const int pair0 = (it - b.row_start[k_inst]) * I.row_pairs;
     const int ntr = min(I.row_pairs, ((ny + 1) >> 1) - pair0);
     const T* R = reinterpret_cast<const T*>(I.R);
-#pragma unroll 4
-    for (int e = tid; e < ntr * n; e += nthr) {
-      const int p = e >> ln, k = e & (n - 1);
+    fft_rev_from<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, false, tid, nthr, [=](int p, int k) {
       const size_t row = (size_t)(2 * (pair0 + p));
-      C z; z.x = R[row * n + k]; z.y = row + 1 < (size_t)ny ? R[(row + 1) * n + k] : T(0);
-      x[pidx<PS>(p * n + brev(k, ln))] = z;
-    }
-    __syncthreads();
-    fft_dit<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, false, tid, nthr);
+      C z;
+      z.x = R[row * n + k];
+      z.y = row + 1 < (size_t)ny ? R[(row + 1) * n + k] : T(0);
+      return z;
+    });
     C* S = reinterpret_cast<C*>(I.S);
     const int nh = (n >> 1) + 1;
     for (int e = tid; e < ntr * nh; e += nthr) {
       const int p = e / nh, k = e - p * nh;
-      const C zk = x[pidx<PS>(p * n + k)], zm = x[pidx<PS>(p * n + ((n - k) & (n - 1)))];
+      const C zk = x[pidx<PS>(p * n + brev(k, ln))], zm = x[pidx<PS>(p * n + brev((n - k) & (n - 1), ln))];
       const size_t row = (size_t)(2 * (pair0 + p));
       C A, B;
       A.x = T(0.5) * (zk.x + zm.x); A.y = T(0.5) * (zk.y - zm.y);
@@ -353,10 +551,11 @@ __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft
 // spectral columns, loaded and stored row by row (adjacent threads take
 // adjacent columns of one row); the forward transform runs from natural to
 // bit-reversed order and the inverse back, so the symbol division takes the
-// spectrum in bit-reversed order and no permutation pass is needed.  The FP32
+// spectrum in bit-reversed order and no permutation pass is needed
+// (fft_there_and_back).  The FP32
 // form runs it with blocks of 512 threads, two per SM (cols_threads<T>; at 2048^2
-// its 257 items of four columns then run in one wave: 0.098 ms per step against
-// 0.120 with one block of 1024 and 0.143 with 256), the FP64 form with 256 (its
+// its 257 items of four columns then run in one wave: 0.098 ms per step, with a pass more for input,
+// symbol and output each, against 0.120 with one block of 1024 and 0.143 with 256), the FP64 form with 256 (its
 // butterflies keep the FP64 pipe busy either way); the load and store loops are
 // unrolled so that several global accesses per thread are in flight.
 #ifndef APD_COLS_THREADS32
@@ -386,37 +585,24 @@ __global__ void __launch_bounds__(cols_threads<T>(), sizeof(T) == 4 ? 1024 / APD
     const int ntr = min(G, nh - col0);
     if (col0 == 0) theta_mean(I, b.rhs_start[k_inst + 1] - b.rhs_start[k_inst], red, &s_mean, tid, nthr);
     C* S = reinterpret_cast<C*>(I.S);
-#pragma unroll 4
-    for (int e = tid; e < (n << lg); e += nthr) {
-      const int y = e >> lg, g = e & (G - 1);
-      if (g < ntr) x[pidx<PS>(g * n + y)] = S[(size_t)y * ss + col0 + g];
-    }
-    __syncthreads();
-    fft_rev<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, false, tid, nthr);
-    const double kap = I.kappa[i];
-    const double scale = I.hscale;
-    for (int e = tid; e < ntr * n; e += nthr) {
-      const int g = e >> ln, ky = brev(e & (n - 1), ln), kx = col0 + g;
-      C v = x[pidx<PS>(e)];
-      if (kx == 0 && ky == 0) {
-        v.x = T(s_mean); v.y = T(0);
-      } else if (sizeof(T) == 8) {
-        const double f = scale * rcp_newton(I.lamx[kx] + I.lamy[ky] - kap);
-        v.x = T(double(v.x) * f); v.y = T(double(v.y) * f);
-      } else {
-        // FP32 form: the symbol in FP32 from the tables rounded once on the host
-        const float f = I.hscale32 * __frcp_rn(I.lamx32[kx] + I.lamy32[ky] - I.k32.kappa[i]);
-        v.x *= T(f); v.y *= T(f);
-      }
-      x[pidx<PS>(e)] = v;
-    }
-    __syncthreads();
-    fft_dit<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr);
-#pragma unroll 4
-    for (int e = tid; e < (n << lg); e += nthr) {
-      const int y = e >> lg, g = e & (G - 1);
-      if (g < ntr) S[(size_t)y * ss + col0 + g] = x[pidx<PS>(g * n + y)];
-    }
+    const double kap = I.kappa[i], scale = I.hscale;
+    fft_there_and_back<T, PS>(
+        x, ln, lg, ntr, twiddles<T>(b), b.lnmax, tid, nthr,
+        [=](int g, int y) { return S[(size_t)y * ss + col0 + g]; },
+        [&](int g, int ky, C& v) {
+          const int kx = col0 + g;
+          if (kx == 0 && ky == 0) {
+            v.x = T(s_mean); v.y = T(0);
+          } else if (sizeof(T) == 8) {
+            const double f = scale * rcp_newton(I.lamx[kx] + I.lamy[ky] - kap);
+            v.x = T(double(v.x) * f); v.y = T(double(v.y) * f);
+          } else {
+            // FP32 form: the symbol in FP32 from the tables rounded once on the host
+            const float f = I.hscale32 * __frcp_rn(I.lamx32[kx] + I.lamy32[ky] - I.k32.kappa[i]);
+            v.x *= T(f); v.y *= T(f);
+          }
+        },
+        [=](int g, int y, C v) { S[(size_t)y * ss + col0 + g] = v; });
     __syncthreads();
   }
 }
@@ -437,26 +623,27 @@ __global__ void __launch_bounds__(rows_threads<T>(), rows_min_blocks<T>()) k_fft
     const int pair0 = (it - b.row_start[k_inst]) * I.row_pairs;
     const int ntr = min(I.row_pairs, ((ny + 1) >> 1) - pair0);
     const C* S = reinterpret_cast<const C*>(I.S);
-#pragma unroll 4
-    for (int e = tid; e < ntr * n; e += nthr) {
-      const int p = e >> ln, k = e & (n - 1);
+    auto load = [=](int p, int k) {
       const size_t row = (size_t)(2 * (pair0 + p));
-      const bool two = row + 1 < (size_t)ny;
-      C A, B;
+      const int kk = k <= (n >> 1) ? k : n - k;
+      C A = S[row * ss + kk], B;
       B.x = B.y = T(0);
-      if (k <= (n >> 1)) {
-        A = S[row * ss + k];
-        if (two) B = S[(row + 1) * ss + k];
-      } else {
-        A = S[row * ss + (n - k)];
-        if (two) B = S[(row + 1) * ss + (n - k)];
-        A.y = -A.y; B.y = -B.y;
-      }
-      C z; z.x = A.x - B.y; z.y = A.y + B.x;
-      x[pidx<PS>(e)] = z;
+      if (row + 1 < (size_t)ny) B = S[(row + 1) * ss + kk];
+      if (kk != k) { A.y = -A.y; B.y = -B.y; }
+      C z;
+      z.x = A.x - B.y; z.y = A.y + B.x;
+      return z;
+    };
+    if constexpr (sizeof(T) == 4) {
+      fft_rev_from<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr, load);
+    } else {
+      // FP64: the two sums of load() on all threads, not on the n/8 of a step (256^2, ten steps: 244 us
+      // against 278; 2048^2: no difference)
+#pragma unroll 4
+      for (int e = tid; e < ntr * n; e += nthr) x[pidx<PS>(e)] = load(e >> ln, e & (n - 1));
+      __syncthreads();
+      fft_rev<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr);
     }
-    __syncthreads();
-    fft_rev<T, PS>(x, ln, ntr, twiddles<T>(b), b.lnmax, true, tid, nthr);
     T* th = reinterpret_cast<T*>(I.Xs[i]) + 2 * (size_t)I.nx * I.ny;
     for (int e = tid; e < ntr * n; e += nthr) {
       const int p = e >> ln, m = e & (n - 1);
