@@ -191,6 +191,8 @@ __device__ __forceinline__ bool has(unsigned mask, int j) { return (mask >> j) &
 // a single division: multiplying both alpha_k by prod_m (eps_W + beta_m)^2
 // gives alpha'_k = d_k prod_{m != k} (eps_W + beta_m)^2, the same weights.
 // (WENO5 is evaluated from per-point terms in the stencil kernels.)
+// Every contraction is written out, here and wherever several kernels hold the same form, so that
+// a result does not depend on the tile shape or the kind of kernel that takes a solve.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T weno3(T a, T b, T c, T ew) {
@@ -200,7 +202,7 @@ __device__ __forceinline__ T weno3(T a, T b, T c, T ew) {
   T s1 = fma(c - b, c - b, ew); s1 *= s1;
   const T w0 = T(1.0 / 3.0) * s1;
   const T w1 = T(2.0 / 3.0) * s0;
-  return fma(w0, p0, w1 * p1) / (w0 + w1);
+  return fma(w0, p0, w1 * p1) / fma(T(1.0 / 3.0), s1, w1);
 }
 
 // a + b, never contracted with a product that formed either.

@@ -32,18 +32,20 @@ __device__ __forceinline__ void pop_to_mom(const double* dF, const InstDev& I, d
 
 // moments -> dF, in the arithmetic type R (FP64 in the FP64 form and for
 // state input; FP32 when the FP32 form repacks its FP32 stage values, whose
-// result is stored in FP32 anyway)
+// result is stored in FP32 anyway); contractions written out, as several kernels close a step with it
 template <typename R>
 __device__ __forceinline__ void mom_to_pop(const R* m, R eps, R rho0, R amp, R* dF) {
   const R M0 = R(2) * eps * m[2], M1 = m[0], M2 = m[1];
   const R M3 = -eps * m[3], M4 = eps * m[4], M5 = eps * eps * m[5];
   const R r6 = R(1.0 / 6.0), r3 = R(1.0 / 3.0), t3 = R(2.0 / 3.0);
-  const R S1 = M0 * r6 + t3 * M3;
-  const R S2 = M0 * r6 - M3 * r3 + R(SQ3 / 3.0) * M4;
-  const R S3 = M0 * r6 - M3 * r3 - R(SQ3 / 3.0) * M4;
-  const R D1 = M1 * r3 - t3 * M5;
-  const R D2 = M1 * r6 + R(SQ3 / 6.0) * M2 + t3 * M5;
-  const R D3 = -M1 * r6 + R(SQ3 / 6.0) * M2 - t3 * M5;
+  const R S0 = fma(-M3, r3, M0 * r6);
+  const R S1 = fma(t3, M3, M0 * r6);
+  const R S2 = fma(R(SQ3 / 3.0), M4, S0);
+  const R S3 = fma(R(-SQ3 / 3.0), M4, S0);
+  const R D0 = R(SQ3 / 6.0) * M2, T5 = t3 * M5;
+  const R D1 = fma(M1, r3, -T5);
+  const R D2 = add_rn(fma(M1, r6, D0), T5);
+  const R D3 = add_rn(fma(-M1, r6, D0), -T5);
   const R a = rho0 * amp;
   dF[0] = a * (S1 + D1); dF[3] = a * (S1 - D1);
   dF[1] = a * (S2 + D2); dF[4] = a * (S2 - D2);

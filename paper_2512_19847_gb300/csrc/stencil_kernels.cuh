@@ -273,12 +273,12 @@ template <typename T>
 __device__ __forceinline__ void w5_nd(const T* P, const T* C, int st, T& num, T& den) {
   static_assert(std::is_same<T, double>::value, "FP64 reconstruction");
   const T a = P[-2 * st], b = P[-st], c = P[0], d = P[st], e = P[2 * st];
-  const T l0 = a - T(4) * b + T(3) * c;
+  const T l0 = fma(T(3), c, fma(T(-4), b, a));
   const T l1 = b - d;
-  const T l2 = T(3) * c - T(4) * d + e;
-  const T e0 = C[-st] + l0 * l0;
-  const T e1 = C[0] + l1 * l1;
-  const T e2 = C[st] + l2 * l2;
+  const T l2 = fma(T(3), c, fma(T(-4), d, e));
+  const T e0 = fma(l0, l0, C[-st]);
+  const T e1 = fma(l1, l1, C[0]);
+  const T e2 = fma(l2, l2, C[st]);
   const T s0 = e0 * e0, s1 = e1 * e1, s2 = e2 * e2;
   const T A = s1 * s2, B = s0 * s2, Cc = s0 * s1;     // 1 / s_k times s_0 s_1 s_2
   den = fma(T(3), Cc, fma(T(6), B, A));               // 10 (d_0 A + d_1 B + d_2 C)
@@ -296,7 +296,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // Interface flux from the left (g+) and right (g-) reconstructions (FP64).
 __device__ __forceinline__ double combine(double nl, double dl, double nr, double dr) {
-  return (nl * dr + nr * dl) * rcp_newton(dl * dr);
+  return fma(nl, dr, nr * dl) * rcp_newton(dl * dr);
 }
 
 // Select a[i] for a small compile-time-sized array without local memory.
@@ -390,8 +390,8 @@ __device__ __forceinline__ void axis_fluxes(const T* const* g, const T* const* U
       if (pt == 0 || pt == LL - 1) continue;
       const int pr = q >> 1, pm = q & 1;
       const T* f = split + (4 * pr + pm) * LS + r;
-      const T cv = f[-PS] - T(2) * f[0] + f[PS];
-      split[(4 * pr + 2 + pm) * LS + r] = T(13.0 / 3.0) * cv * cv + ew4;
+      const T cv = fma(T(-2), f[0], f[-PS]) + f[PS];
+      split[(4 * pr + 2 + pm) * LS + r] = fma(T(13.0 / 3.0) * cv, cv, ew4);
     }
     __syncthreads();
     // 3. interface fluxes: left-biased reconstruction of g+ centred at m, right-biased of g- centred at m+1
@@ -564,16 +564,16 @@ __device__ __forceinline__ void w5_fluxes_xy(const T* const* gx, const T* const*
       if (pt == 0 || pt == W - 1) continue;
       const int pr = q >> 1, pm = q & 1;
       const T* f = spx + (4 * pr + pm) * LSX + r;
-      const T cv = f[-1] - T(2) * f[0] + f[1];
-      spx[(4 * pr + 2 + pm) * LSX + r] = T(13.0 / 3.0) * cv * cv + ew4;
+      const T cv = fma(T(-2), f[0], f[-1]) + f[1];
+      spx[(4 * pr + 2 + pm) * LSX + r] = fma(T(13.0 / 3.0) * cv, cv, ew4);
     } else {
       const int kk = k - 2 * NP * LSX;
       const int q = kk / LSY, r = kk - q * LSY, pt = r / TX;
       if (pt == 0 || pt == HH - 1) continue;
       const int pr = q >> 1, pm = q & 1;
       const T* f = spy + (4 * pr + pm) * LSY + r;
-      const T cv = f[-TX] - T(2) * f[0] + f[TX];
-      spy[(4 * pr + 2 + pm) * LSY + r] = T(13.0 / 3.0) * cv * cv + ew4;
+      const T cv = fma(T(-2), f[0], f[-TX]) + f[TX];
+      spy[(4 * pr + 2 + pm) * LSY + r] = fma(T(13.0 / 3.0) * cv, cv, ew4);
     }
   }
   __syncthreads();
