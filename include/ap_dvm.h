@@ -83,7 +83,11 @@ enum { AP_DVM_FP64 = 0, AP_DVM_FP32_DEV = 1, AP_DVM_FP32_DEV_TH = 2 }; /* precis
  *  precision   AP_DVM_FP64 (all in FP64; WENO solves of at least 256 cells per
  *              side evaluate the part of their fluxes that is not linear in the
  *              data, nonlinear weight times difference, in pairs of floats of 48
- *              bits, from differences taken in FP64) or AP_DVM_FP32_DEV (FP32
+ *              bits, from differences taken in FP64, where the data are resolved:
+ *              an interface whose third differences exceed 1/32 of the field's
+ *              largest value (WENO3: second differences, 3/128), or whose values
+ *              or eps_W such pairs do not hold, takes the whole FP64 form, so that
+ *              rough data cost time, not precision) or AP_DVM_FP32_DEV (FP32
  *              deviation populations and FP32 transport; moment sums, division by
  *              rho0*mach, and closed-form relaxation when eps <= 1e-4 in pairs of
  *              floats, rounded once).

@@ -56,6 +56,7 @@ InstDev view(const Slot& s, int parity) {
   void* buf[2] = {s.dev.X, s.dev.Xnext};
   d.X = buf[q];
   d.Xnext = buf[q ^ 1];
+  if (q) std::swap(d.mag, d.magnext);
   if (s.p.A_im[0] == 0.0) {
     d.Xs[1] = d.X;
     d.Dun = d.Du[1];
@@ -751,6 +752,8 @@ ap_dvm_status ap_dvm_attach(ap_dvm_handle* h, int slot, const ap_dvm_params* p, 
   }
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));   // the symbol and transform-table vectors are about to go out of scope
   for (void* xb : {d.X, d.Xnext}) CUDA_TRY(h, cudaMemsetAsync(xb, 0, (size_t)6 * p->nx * p->ny * (h->f32 ? 4 : 8), h->stream));
+  if (!split_fluxes(*p)) d.mag = d.magnext = nullptr;
+  if (d.mag) CUDA_TRY(h, cudaMemsetAsync(d.mag, 0, 8 * sizeof(unsigned), h->stream));
   if (d.dF) CUDA_TRY(h, cudaMemsetAsync(d.dF, 0, (size_t)6 * p->nx * p->ny * sizeof(float), h->stream));
   s.flip = 0;
   s.paused = false;
@@ -787,6 +790,7 @@ static ap_dvm_status set_state_impl(ap_dvm_handle* h, int slot, const double* a,
   if (st) return st;
   InstDev d = view(*s, h->parity);
   int form = h->tmpl.precision;   // 0: FP64, 1: FP32 deviation form, 2: the same with theta carried
+  if (d.mag) CUDA_TRY(h, cudaMemsetAsync(d.mag, 0, 3 * sizeof(unsigned), h->stream));
   void* args[] = {&d, &a, &b, &c, &f, &mode, &form};
   return launch(h, h->stream, h->km.k_set_state, grid_for_cells((size_t)s->p.nx * s->p.ny), dim3(256), 0, args);
 }

@@ -114,6 +114,10 @@ struct InstDev {
   const void* tmap;             // tensor maps (128 B each) of the stage buffers Xs[j]
   int tma;                      // 1: tile loads through the tensor maps; 0: plain loads
   int pad1;
+  // Solves with split fluxes (null otherwise): high words of the largest |u|, |v| and |q| of X and of Xnext,
+  // kept with these buffers by whatever writes them (split_limits).
+  unsigned* mag;
+  unsigned* magnext;
 };
 
 // Work decomposition of the active instances, passed by value to the kernels of a step (its pointers and
@@ -166,6 +170,9 @@ __host__ __device__ constexpr int rhs_items(int nx, int ny, bool f32) {
 __device__ __forceinline__ void grid_dependency() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+
+// High word of |x|: ordered as the values are (NaN above infinity).
+__device__ __forceinline__ unsigned abs_high(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
 // Columns one warp of the marching stencil kernels (march_kernels.cuh) puts out.
 constexpr int MARCH_OUT = 26;

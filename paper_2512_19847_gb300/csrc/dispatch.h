@@ -43,8 +43,8 @@ struct StencilSet {
   const void* k_update;
   const void* k_explicit_split;        // FP64 WENO: the same with split fluxes (null otherwise)
   const void* k_update_split;
-  size_t smem_explicit_split, update_fixed_split;
-  int nbuf_split;
+  size_t smem_explicit_split;
+  size_t (*smem_update_split)(int planes);   // with so many staged planes
   // FP32: by marching warps (null otherwise).  Explicit: [terms of v read from memory: 1, 2, up to
   // 5][bit 0: E, bit 1: D_LF . B(v)]; update: [(stages in the partner, earlier stages in the sums):
   // (1, 0), (2, 1), up to (3, 3)]

@@ -113,6 +113,24 @@ __device__ __forceinline__ bool close_step_cell(const InstDev& I, size_t o, size
   return bad;
 }
 
+// Largest |u|, |v| and |q| of a state (InstDev::mag), as high words of doubles: of one cell's moments, and
+// of a warp's (every lane of it) into three words by atomics.
+__device__ __forceinline__ void field_max(const double* m, unsigned& mu, unsigned& mv, unsigned& mq) {
+  mu = max(mu, max(abs_high(m[0]), abs_high(m[1])));
+  mv = max(mv, max(abs_high(m[3]), abs_high(m[4])));
+  mq = max(mq, abs_high(m[5]));
+}
+__device__ __forceinline__ void field_max_to(unsigned* to, unsigned mu, unsigned mv, unsigned mq, int tid) {
+  mu = __reduce_max_sync(0xffffffffu, mu);
+  mv = __reduce_max_sync(0xffffffffu, mv);
+  mq = __reduce_max_sync(0xffffffffu, mq);
+  if ((tid & 31) == 0) {
+    atomicMax(to, mu);
+    atomicMax(to + 1, mv);
+    atomicMax(to + 2, mq);
+  }
+}
+
 // ---- per-instance conversions (one instance, grid-stride over cells)
 
 // mode 0: moments (double) -> state;  mode 1: equilibrium from (u1, u2, p);
@@ -124,6 +142,7 @@ template <typename T>
 __global__ void k_set_state(InstDev I, const double* __restrict__ a, const double* __restrict__ b2,
                             const double* __restrict__ c3, const float* __restrict__ f32, int mode, int f32form) {
   const size_t pl = (size_t)I.nx * I.ny;
+  unsigned mu = 0u, mv = 0u, mq = 0u;   // of the moments set (I.mag)
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < pl; o += (size_t)gridDim.x * blockDim.x) {
     double m[6];
     if (mode == 4) {
@@ -165,7 +184,16 @@ __global__ void k_set_state(InstDev I, const double* __restrict__ a, const doubl
     } else {
       T* X = reinterpret_cast<T*>(I.X);
       for (int k = 0; k < 6; ++k) X[o + k * pl] = T(m[k]);
+      field_max(m, mu, mv, mq);
     }
+  }
+  if (sizeof(T) == 8 && I.mag) {
+    __shared__ unsigned blk[3];
+    if (threadIdx.x < 3) blk[threadIdx.x] = 0u;
+    __syncthreads();
+    field_max_to(blk, mu, mv, mq, threadIdx.x);
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMax(I.mag + threadIdx.x, blk[threadIdx.x]);
   }
 }
 

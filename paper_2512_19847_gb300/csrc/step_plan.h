@@ -77,20 +77,24 @@ inline int fft_eblk_cols(int nmax, bool f32) {
 }
 
 inline size_t update_smem_split(const StencilSet& ks, const ap_dvm_params& t) {
-  return ks.update_fixed_split + (size_t)ks.nbuf_split * update_planes_max(t) * ks.plane_bytes;
+  return ks.smem_update_split(update_planes_max(t));
 }
 
 // Whether the fluxes of a solve are split (split_flux.cuh): FP64 with a WENO scheme and at least
-// kSplitMinCells cells on each side.
+// kSplitMinCells cells on each side.  Where its data are rough, the split kernels themselves fall back on the
+// whole form; the line keeps grids that are rough all over off them.
 // Why the line lies there: the pairs of floats round second and third differences to about 2^-47 of
 // the increments, FP64 rounds the whole flux to 2^-52 of its own size.  For fields of wavenumbers up
 // to 16 (the workloads') the rms error of a flux difference against 113-bit arithmetic, split and
 // whole, in units of 1e-17: WENO5 at 2048 cells a side 0.4 and 5.3, 512: 1.6 and 5.3, 256: 3.2 and
-// 5.3, 128: 9.2 and 5.4; WENO3 at 512: 1.9 and 5.3, 256: 6.0 and 5.5, 128: 21 and 5.7.  Whole steps
-// against 64-bit-mantissa arithmetic (relative; u1, theta, v1): 512^2 Taylor-Green 0.80e-16, 5.7e-15,
-// 1.29e-16 split, 1.09e-16, 6.0e-15, 1.41e-16 whole; 256^2 WENO3 layer 0.87e-16, 4.3e-15, 1.6e-16 and
-// 1.48e-16, 5.6e-15, 2.3e-16; 256^2 random field 1.19e-16, 3.5e-15, 2.7e-16 and 1.16e-16, 2.9e-15,
-// 2.6e-16 (a plain FP64 evaluation: 1.57e-16, 3.7e-15, 2.4e-16).
+// 5.3, 128: 9.2 and 5.4; WENO3 at 512: 1.9 and 5.3, 256: 6.0 and 5.5, 128: 21 and 5.7 (WENO3's meet near 300
+// cells for these fields; the layers it is run on, smooth along x, stay below to 256: a fifth of the whole form's).
+// Whole steps against 64-bit-mantissa arithmetic (relative; u1, theta, v1): 512^2 Taylor-Green 0.90e-16, 8.5e-15,
+// 1.30e-16 split, 1.15e-16, 7.0e-15, 1.43e-16 whole; 256^2 WENO3 layer 0.93e-16, 4.6e-15, 1.7e-16 and
+// 1.55e-16, 3.3e-15, 2.5e-16; 256^2 random field, WENO5 1.19e-16, 3.6e-15, 2.7e-16 and 1.15e-16, 2.9e-15,
+// 2.8e-16, WENO3 1.69e-16, 3.3e-15, 2.9e-16 and 1.43e-16, 3.1e-15, 2.9e-16; 300^2 WENO3 1.46e-16, 2.7e-15, 1.7e-16
+// and 1.44e-16, 2.7e-15, 1.7e-16.  (Theta's is the sum of a few low modes' roundings: it varies by a third
+// with the draw, for both forms alike.)
 constexpr int kSplitMinCells = 256;
 inline bool split_fluxes(const ap_dvm_params& p) {
   return p.precision == AP_DVM_FP64 && p.space_scheme != AP_DVM_LF1_C2 && p.nx >= kSplitMinCells && p.ny >= kSplitMinCells;

@@ -100,6 +100,8 @@ inline size_t carve_instance(const ap_dvm_params& p, char* base, InstDev* d, boo
   }
   I.dF = f32 ? reinterpret_cast<float*>(take(6 * cells * sizeof(float))) : nullptr;
   I.tmap = take(sizeof(CUtensorMap) * (APD_MAXS + 1) * (two_states ? 2 : 1));
+  I.mag = two_states && !f32 ? reinterpret_cast<unsigned*>(take(8 * sizeof(unsigned))) : nullptr;
+  I.magnext = I.mag ? I.mag + 4 : nullptr;
   return align_up(off, 256);
 }
 
