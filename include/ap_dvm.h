@@ -217,6 +217,9 @@ ap_dvm_status ap_dvm_set_graph_steps(ap_dvm_handle* h, int k);
  * tile; their results are the same bits.) */
 ap_dvm_status ap_dvm_set_tile(ap_dvm_handle* h, int tile);
 int ap_dvm_get_tile(const ap_dvm_handle* h);
+/* 1 when a stencil kernel that works on tiles takes any attached solve, 0 when the
+ * tile shape plays no part (all are taken by the marching kernels). */
+int ap_dvm_uses_tiles(const ap_dvm_handle* h);
 /* Kernel launches enqueued by one ap_dvm_step(h, 1). */
 int ap_dvm_launches_per_step(const ap_dvm_handle* h);
 

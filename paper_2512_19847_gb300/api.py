@@ -100,6 +100,7 @@ def lib():
         "ap_dvm_set_graph_steps": (i32, [H, i32]),
         "ap_dvm_set_tile": (i32, [H, i32]),
         "ap_dvm_get_tile": (i32, [H]),
+        "ap_dvm_uses_tiles": (i32, [H]),
         "ap_dvm_launches_per_step": (i32, [H]),
         "ap_dvm_run_host": (i32, [H, i32, vp, vp, vp, i32]),
         "ap_dvm_sync_status": (i32, [H]),
@@ -261,6 +262,11 @@ class _Handle:
     @property
     def tile(self) -> int:
         return lib().ap_dvm_get_tile(self._h)
+
+    @property
+    def uses_tiles(self) -> bool:
+        """Whether a kernel that works on tiles takes any attached solve."""
+        return bool(lib().ap_dvm_uses_tiles(self._h))
 
     @property
     def launches_per_step(self) -> int:

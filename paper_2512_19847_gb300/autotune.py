@@ -1,6 +1,7 @@
 """Tile-shape autotuner for the stencil kernels of a Solver or Batch.
 
-Every tile shape the attached grids admit is timed on the handle's own solves
+Every tile shape the attached grids admit is timed on the handle's own solves, unless
+the marching kernels, which use no tile, take them all
 (a few IMEX steps, CUDA events on the handle's stream); the state is saved
 before and restored bit for bit afterwards, so tuning never changes results.
 The winner is cached in a JSON file keyed by GPU name, precision, scheme,
@@ -77,7 +78,10 @@ def load_cache(path: str = DEFAULT_CACHE) -> dict:
 
 def tune(h, steps: int = 2, path: str | None = DEFAULT_CACHE, use_cache: bool = True) -> dict:
     """Pick and set the fastest tile shape for the solves attached to h.
-    Returns {"tile": t, "ms_per_step": {t: ms}, "cached": bool}."""
+    Returns {"tile": t, "ms_per_step": {t: ms}, "cached": bool}; where no attached solve works
+    on tiles (ap_dvm_uses_tiles), the shape is left as it is and nothing is timed."""
+    if not getattr(h, "uses_tiles", True):
+        return {"tile": h.tile, "ms_per_step": {}, "cached": False}
     key = signature(h)
     cache = load_cache(path) if (path and use_cache) else {}
     if key in cache:

@@ -981,6 +981,8 @@ ap_dvm_status ap_dvm_set_tile(ap_dvm_handle* h, int tile) {
 
 int ap_dvm_get_tile(const ap_dvm_handle* h) { return h ? h->tile : -1; }
 
+int ap_dvm_uses_tiles(const ap_dvm_handle* h) { return h && (stencil_kinds_of(h) & ~STENCIL_MARCH) ? 1 : 0; }
+
 int ap_dvm_launches_per_step(const ap_dvm_handle* h) {
   if (!h) return 0;
   const ap_dvm_params& t = h->tmpl;
