@@ -304,11 +304,11 @@ void ap_dvm_destroy(ap_dvm_handle* h);
 ap_dvm_status ap_dvm_fma_peak(int precision, int iters, int reps, void* cuda_stream, double* tflops,
                               double* ms_per_launch);
 
-/* Self-check of the library's integer-pipe FP32 <-> FP64 conversions (widen_f32,
- * narrow_f64_rn, exact stand-ins for the conversion instructions): for each of the n FP64 values at d_in (device), the narrowing to FP32
- * (nearest, ties to even) and the widening of that FP32 value back to FP64 are compared
- * with the instructions' results bit for bit (a NaN only as a NaN).  d_counts (device,
- * 2 unsigned, caller-owned) receives the numbers of mismatching narrowings and
+/* Self-check of the integer-pipe conversions that the split fluxes use in place of the
+ * conversion instructions, on the n FP64 values at d_in (device): the pair of floats of each
+ * (to 2^-48 of it where 2^-74 <= |x| < 2^128, else against the instructions), and the
+ * widening of the value rounded to FP32 (bit for bit, a NaN only as a NaN).  d_counts
+ * (device, 2 unsigned, caller-owned) receives the numbers of mismatching pairs and
  * widenings; it is zeroed first.  Asynchronous on cuda_stream.  Returns AP_DVM_ERR_ARG
  * for null pointers or n < 0, AP_DVM_ERR_CUDA if a launch fails. */
 ap_dvm_status ap_dvm_check_conversions(const double* d_in, int n, unsigned* d_counts, void* cuda_stream);

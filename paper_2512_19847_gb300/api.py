@@ -149,7 +149,7 @@ def fma_peak(precision: int = FP64, iters: int = 256, reps: int = 50, stream=Non
 
 def check_conversions(x: torch.Tensor, stream=None) -> tuple[int, int]:
     """ap_dvm_check_conversions on the FP64 values of the device tensor x: the numbers of
-    integer-pipe narrowings and widenings that differ from the conversion instructions."""
+    integer-pipe conversions to a pair of floats, and of widenings, that are off."""
     x = x.contiguous()
     assert x.dtype == torch.float64 and x.is_cuda
     counts = torch.zeros(2, dtype=torch.int32, device=x.device)

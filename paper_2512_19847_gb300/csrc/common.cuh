@@ -257,71 +257,6 @@ __device__ __forceinline__ double rcp_newton(double d) {
   return r;
 }
 
-// FP32 <-> FP64 conversions on the integer pipe.  On this GPU the conversion
-// instructions issue on the FP64 pipe (2 per clock per SM); these rebuild the
-// IEEE 754 binary64 (binary32) bit pattern with integer operations and selects
-// only, for every class of input, with the instruction's result: exact
-// widening, narrowing rounded to nearest with ties to even (overflow to
-// infinity, subnormal results rounded likewise); a NaN stays a NaN
-// (ap_dvm_check_conversions compares them with the instructions bit for bit).
-// ap_dvm_check_conversions is their self-check; the FP32 forms' own sums and relaxations
-// work in pairs of floats (pairs.cuh) and convert nothing.
-// Every class of input: zero, subnormal, infinity, NaN as well.
-static __device__ __noinline__ double widen_f32_any(float x) {
-  const unsigned u = __float_as_uint(x), s = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-  // normal: exponent bias 127 -> 1023 (+896 in the exponent field), fraction 23 -> 52 bits
-  unsigned hi = s | (((u & 0x7fffffffu) >> 3) + (896u << 20)), lo = u << 29;
-  // subnormal: m 2^-149 = 1.f 2^(p - 149), p the position of the leading bit of m
-  const unsigned p = 31u - (unsigned)__clz(m | 1u), f = (m << (23u - p)) & 0x7fffffu;
-  if (e == 0u) {
-    hi = m ? (s | ((p + 874u) << 20) | (f >> 3)) : s;
-    lo = m ? (f << 29) : 0u;
-  }
-  if (e == 0xffu) hi = s | 0x7ff00000u | (m >> 3);   // infinity or NaN (lo as above)
-  return __hiloint2double((int)hi, (int)lo);
-}
-
-__device__ __forceinline__ double widen_f32(float x) {
-  const unsigned u = __float_as_uint(x);
-  if (((u >> 23) & 0xffu) - 1u < 254u)   // a normal value: rebias the exponent, extend the fraction
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-  return widen_f32_any(x);
-}
-
-// Every class of result: subnormal binary32 results and zero, overflow, infinity, NaN.
-static __device__ __noinline__ float narrow_f64_rn_any(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned s = hi & 0x80000000u, ea = (hi >> 20) & 0x7ffu;
-  // normal binary32 results (biased binary64 exponent 897 .. 1150): drop 29 fraction bits
-  unsigned r = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
-  r += ((lo & 0x1fffffffu) + 0x0fffffffu + (r & 1u)) >> 29;   // nearest, ties to even (may carry to infinity)
-  // smaller: subnormal binary32 or zero, (2^52 + fraction) / 2^k rounded the same way, k = 926 - ea >= 30
-  const unsigned long long M = (1ull << 52) | ((unsigned long long)(hi & 0xfffffu) << 32) | lo;
-  const unsigned k = 926u - min(ea, 896u);
-  unsigned q = 0u;
-  if (k < 64u) {
-    const unsigned long long rem = M & ((1ull << k) - 1ull), half = 1ull << (k - 1u);
-    q = (unsigned)(M >> k);
-    q += (rem > half || (rem == half && (q & 1u))) ? 1u : 0u;
-  }
-  unsigned out = ea >= 897u ? r : q;
-  if (ea > 1150u) out = 0x7f800000u;                                  // overflow
-  if (ea == 0x7ffu)
-    out = ((hi & 0xfffffu) | lo) ? (0x7fc00000u | ((hi & 0xfffffu) << 3) | (lo >> 29)) : 0x7f800000u;
-  return __uint_as_float(out | s);
-}
-
-__device__ __forceinline__ float narrow_f64_rn(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned ea = (hi >> 20) & 0x7ffu;
-  if (ea - 897u <= 1150u - 897u) {   // a normal binary32 result: drop 29 fraction bits, nearest, ties to even
-    unsigned r = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
-    r += ((lo & 0x1fffffffu) + 0x0fffffffu + (r & 1u)) >> 29;   // (a carry into the exponent reaches infinity)
-    return __uint_as_float(r | (hi & 0x80000000u));
-  }
-  return narrow_f64_rn_any(d);
-}
-
 // Periodic image of index g on a line of n cells, for g >= -n (any g a tile or
 // stencil reaches: at most a tile width plus the halo past the last cell).
 __device__ __forceinline__ int wrap_index(int g, int n) {

@@ -27,15 +27,19 @@ cudaError_t launch_wait_timeout(unsigned* err, unsigned long long limit_ns, cuda
   return cudaGetLastError();
 }
 
-// The integer-pipe conversions against the instructions, bit for bit (NaN as NaN):
-// bad[0] counts mismatching narrowings of the inputs, bad[1] mismatching widenings
-// of the narrowed values.
+// The integer-pipe conversions against the instructions (NaN as NaN): bad[0] counts inputs whose pair
+// of floats is off by more than 2^-48 of them or, outside 2^-74 .. 2^128, differs from the instructions'
+// pair; bad[1] mismatching widenings, bit for bit, of the inputs rounded to FP32.
 __global__ void k_check_conversions(const double* __restrict__ in, int n, unsigned* __restrict__ bad) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const double d = in[k];
-    const float a = narrow_f64_rn(d), b = __double2float_rn(d);
-    const bool nb = b != b;
-    if (nb ? !(a != a) : __float_as_uint(a) != __float_as_uint(b)) atomicAdd(&bad[0], 1u);
+    const double d = in[k], a = fabs(d);
+    const float b = __double2float_rn(d);
+    const F2 p = f2_from_double(d);
+    bool ok;
+    if (a >= 0x1p-74 && a < 0x1p128) ok = fabs((d - (double)p.h) - (double)p.l) <= 0x1p-48 * a;
+    else if (d != d) ok = p.h != p.h;
+    else ok = p.h == b && (isinf(b) || __float_as_uint(p.l) == __float_as_uint(__double2float_rn(d - (double)b)));
+    if (!ok) atomicAdd(&bad[0], 1u);
     const double w = widen_f32(b), v = (double)b;
     const bool nv = v != v;
     if (nv ? !(w != w) : __double_as_longlong(w) != __double_as_longlong(v)) atomicAdd(&bad[1], 1u);

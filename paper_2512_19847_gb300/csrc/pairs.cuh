@@ -73,15 +73,17 @@ __device__ __forceinline__ F2 f2_from_double(double d) {
   return f2(h, __double2float_rn(d - (double)h));
 }
 
-// h + l in FP64 (one FP64 operation; the widenings on the integer pipe).
-__device__ __forceinline__ double f2_widen1(float x) {
+// FP32 to FP64 on the integer pipe, exact: a normal value's exponent rebiased, its fraction extended
+// (subnormal values, infinities and NaN by the instruction).
+__device__ __forceinline__ double widen_f32(float x) {
   const unsigned u = __float_as_uint(x);
   if (((u >> 23) & 0xffu) - 1u < 254u)
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-  if ((u << 1) == 0u) return 0.0;
+  if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
   return (double)x;
 }
-__device__ __forceinline__ double f2_to_double(F2 a) { return f2_widen1(a.h) + f2_widen1(a.l); }
+// h + l in FP64 (one FP64 operation).
+__device__ __forceinline__ double f2_to_double(F2 a) { return widen_f32(a.h) + widen_f32(a.l); }
 
 // a float times a pair of constants, and two floats' sum and difference, exact up to the pair's rounding.
 __device__ __forceinline__ F2 f2_mulf(F2 c, float x) {
