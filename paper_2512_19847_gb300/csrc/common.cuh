@@ -63,7 +63,7 @@ struct InstDev {
   int tiles_x, tiles_y;         // tile grid for the batch's tile shape
   int row_pairs;                // row pairs per row-FFT work item
   int col_group;                // spectral columns per column-FFT work item
-  int relax64;                  // FP32 form: closed-form relaxation in FP64
+  int relax64;                  // FP32 form at eps <= 1e-4: closed-form relaxations in pairs of floats
   int sstride;                  // complex elements per spectral row (>= nx/2 + 1)
   double dx, dy, dt, eps, tau, te2, rho0, amp;
   float eps32, rho032, amp32;   // eps, rho0, amp rounded once (the FP32 form's repacking)
@@ -192,6 +192,10 @@ template <> __device__ __forceinline__ const Coef<double>& coef<double>(const In
 template <> __device__ __forceinline__ const Coef<float>& coef<float>(const InstDev& I) { return I.k32; }
 __device__ __forceinline__ bool has(unsigned mask, int j) { return (mask >> j) & 1u; }
 
+// a + b, never contracted with a product that formed either.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
 // ---------------------------------------------------------------------------
 // Jiang-Shu WENO3 reconstruction at x_{i+1/2} from the left-biased stencil.
 // The nonlinear weights alpha_k = d_k/(eps_W + beta_k)^2 are normalised with
@@ -209,12 +213,8 @@ __device__ __forceinline__ T weno3(T a, T b, T c, T ew) {
   T s1 = fma(c - b, c - b, ew); s1 *= s1;
   const T w0 = T(1.0 / 3.0) * s1;
   const T w1 = T(2.0 / 3.0) * s0;
-  return fma(w0, p0, w1 * p1) / fma(T(1.0 / 3.0), s1, w1);
+  return fma(w0, p0, w1 * p1) / add_rn(w0, w1);
 }
-
-// a + b, never contracted with a product that formed either.
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
 // Central first and second differences (Sec. 3.2 D_0 and the compact second difference; fourth order
 // under the WENO schemes) from the values at offsets -2 .. 2 along a line, without

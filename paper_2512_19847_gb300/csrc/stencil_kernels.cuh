@@ -273,9 +273,10 @@ template <typename T>
 __device__ __forceinline__ void w5_nd(const T* P, const T* C, int st, T& num, T& den) {
   static_assert(std::is_same<T, double>::value, "FP64 reconstruction");
   const T a = P[-2 * st], b = P[-st], c = P[0], d = P[st], e = P[2 * st];
-  const T l0 = fma(T(3), c, fma(T(-4), b, a));
+  const T c3 = T(3) * c;
+  const T l0 = add_rn(fma(T(-4), b, a), c3);
   const T l1 = b - d;
-  const T l2 = fma(T(3), c, fma(T(-4), d, e));
+  const T l2 = add_rn(fma(T(-4), d, c3), e);
   const T e0 = fma(l0, l0, C[-st]);
   const T e1 = fma(l1, l1, C[0]);
   const T e2 = fma(l2, l2, C[st]);
