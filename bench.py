@@ -224,6 +224,19 @@ def measured_traffic(kind: str, f32: bool, n: int):
     return None if v is None else float(v)
 
 
+# FP64 instructions per cell and step of the split WENO5 stencils, second-order tableau (ncu,
+# sm__inst_executed_pipe_fp64.sum, both stages; profiles/split_and_march_kernels.md)
+SPLIT_FP64_INSTR = {"explicit": 160.0, "update": 129.8}
+
+
+def fp64_pipe_frac(kind: str, cell_steps_per_s: float, scheme: str, n: int, peak_tflops: float):
+    """Share of the FP64 pipe's issue rate (half the FMA peak's flops) that a split stencil takes, None
+    for other kernels."""
+    if scheme != "WENO5_C4" or n < 256 or kind not in SPLIT_FP64_INSTR:
+        return None
+    return round(SPLIT_FP64_INSTR[kind] * cell_steps_per_s / (0.5e12 * peak_tflops), 4)
+
+
 def roofline(prof: dict, steps: int, cells: int, f32: bool, scheme: str, n: int, peaks: dict, fp64_peak: dict | None = None):
     flops = step_flops_per_cell(scheme, n)
     byts = step_bytes_per_cell(f32)
@@ -245,7 +258,9 @@ def roofline(prof: dict, steps: int, cells: int, f32: bool, scheme: str, n: int,
                   "frac": round(achieved / peak, 4), "traffic": measured_traffic(kind, False, n), "kernel": kind,
                   "algorithmic_flops_per_launch": alg, "ms_per_launch": round(per_launch_ms, 4),
                   "note": "the method's flops over the FP64 pipe's peak; from 256 cells a side the WENO weights' part of "
-                          "the fluxes runs in pairs of floats on the FP32 pipe, so the fraction may exceed 1",
+                          "the fluxes runs in pairs of floats on the FP32 pipe, so the fraction may exceed 1: "
+                          "fp64_pipe_frac counts what the kernel issues to the FP64 pipe",
+                  "fp64_pipe_frac": fp64_pipe_frac(kind, cells / (launches_per_step * per_launch_ms * 1e-3), scheme, n, peak),
                   "peak_source": fp64_peak["source"]}
 
 

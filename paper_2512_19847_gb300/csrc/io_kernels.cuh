@@ -7,7 +7,8 @@
 //   sum c1 c2 f = eps v2, sum c1 (c2^2 - 1/4) f = eps^2 q,
 // (v1 = sum (c2^2 - 1/2) f: the sign with which the moment system of Sec. 2.1 holds).  Opposite velocities c_{k+3} = -c_k make even
 // and odd pair sums s_k = f_k + f_{k+3}, d_k = f_k - f_{k+3} the natural
-// variables; both directions of the map are evaluated in FP64.
+// variables.  The map is evaluated in FP64 at the boundary; the FP32 forms repack their stage values in FP32
+// and sum the moments of a step in pairs of floats.
 #pragma once
 #include "common.cuh"
 

@@ -123,8 +123,9 @@ extern "C" ap_dvm_status ap_dvm_step_noalloc(const ap_dvm_params* p, double* d_s
   carve_instance(*p, base + L.ws, &I);
   I.nx = p->nx; I.ny = p->ny; I.lnx = ilog2(p->nx); I.lny = ilog2(p->ny);
   I.tiles_x = p->nx / ks.tx; I.tiles_y = p->ny / ks.ty;
+  // row pairs: what a block's shared memory holds; columns: two (the handle path gives each resident block a share of both)
   I.row_pairs = std::max(1, std::min(eblk / p->nx, p->ny / 2));
-  I.col_group = std::min(2, std::max(1, eblk_cols / p->ny));   // the handle path's rule (FP64)
+  I.col_group = std::min(2, std::max(1, eblk_cols / p->ny));
   I.relax64 = 0;
   fill_constants(*p, I);
   CUtensorMap maps[APD_MAXS + 1];

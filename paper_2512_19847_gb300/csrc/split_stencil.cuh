@@ -6,19 +6,15 @@
 // Where an interface of the tile is rough (split_flux.cuh), the whole FP64 fluxes are taken too, pair by pair
 // in the space of the increments (w5_fluxes_xy, axis_fluxes), for the cells beside such an interface:
 // which form a cell takes depends on its stencil and the field's largest values alone, not on tile
-// or batch.  The test of every interface costs 0.3 to 0.9 % of a step on smooth data (2048^2 5261 -> 5277 us,
-// 512^2 host call 1626 -> 1640).
-// What bounds them is still the FP64 pipe (2 operations per clock and SM), now with about 110
-// (explicit, all terms) and 70 (update) FP64 operations per cell instead of 510 and 370, beside
-// about 450 FP32 instructions per interface.  WENO5 at 2048^2, ms per step (32x8 tiles): explicit
-// 6.17 -> 1.77, update 6.06 -> 1.68 (2.16 and 2.18 with the fourth-order difference of g and the
-// fourth difference of U in FP64 and the partner as FP64 planes); WENO3 at 256^2, 10 steps:
-// 0.98 -> 0.47 and 1.00 -> 0.44.  Measured choices, with those earlier terms (2048^2, explicit +
-// update, ms): WENO5 768 threads per SM (85 registers) 2.16 + 2.18, 512 (128 registers) 2.30 + 2.31;
-// one staged plane buffer 2.30 + 2.31 against 2.31 + 2.35 with two (at 512 threads; the other blocks
-// on the SM hide the copies); runs of 3 interfaces 2.30 + 2.31, of 4 2.37 + 2.55.  WENO3 keeps 512
-// threads: 2.03 + 1.99 against 1.98 + 1.86 at 2048^2 but 0.056 + 0.053 against 0.070 + 0.066 at
-// 256^2, the size it is run at.
+// or batch.  The test of every interface costs 0.3 to 0.9 % of a step on smooth data.
+// What bounds them is still the FP64 pipe (2 operations per clock and SM), with 100 (explicit, all
+// terms) and 74 (update) FP64 operations per cell instead of 510 and 370, beside about 450 FP32
+// instructions per interface.  WENO5 at 2048^2, ms per step (32x8 tiles): explicit
+// 6.17 -> 1.65, update 6.06 -> 1.55; WENO3 at 256^2, 10 steps: 0.98 -> 0.44 and 1.00 -> 0.41.  Measured choices
+// (explicit + update, ms per step): WENO5 at 2048^2 768 threads per SM (80 registers) 1.65 + 1.55, 512 (128
+// registers) 1.77 + 1.71; runs of 3 interfaces 1.65 + 1.55, of 2 1.78 + 1.69, of 4 1.73 + 1.86.  WENO3 512
+// threads 0.044 + 0.041 at 256^2 and 1.48 + 1.41 at 2048^2, 768 0.050 + 0.045 and 1.40 + 1.31: a choice for
+// the sizes the paper runs WENO3 at, 6 % against the largest.
 #pragma once
 #include "split_flux.cuh"
 #include "stencil_kernels.cuh"

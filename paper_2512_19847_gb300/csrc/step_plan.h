@@ -18,12 +18,12 @@ namespace apd {
 
 enum KernelKind { KK_EXPLICIT, KK_RHS, KK_ROWS_FWD, KK_COLS, KK_ROWS_INV, KK_UPDATE, KK_FINISH, KK_STAGE1 };
 
-// Kinds of Helmholtz transform work a batch holds (bits of StepKernels::fft_kinds).
 // Kinds of stencil work a batch holds (bits of StepKernels::stencil_kinds): instances taken by the tile
 // kernels with whole fluxes, those with split fluxes (FP64, split_flux.cuh), and those taken by the
 // marching kernels (FP32, march_kernels.cuh).
 enum StencilKinds { STENCIL_WHOLE = 1, STENCIL_SPLIT = 2, STENCIL_MARCH = 4 };
 
+// Kinds of Helmholtz transform work a batch holds (bits of StepKernels::fft_kinds).
 enum FftKinds { FFT_X_POW2 = 1, FFT_X_BS = 2, FFT_Y_POW2 = 4, FFT_Y_BS = 8 };
 
 // Transform launches of one implicit stage for the given kinds.
